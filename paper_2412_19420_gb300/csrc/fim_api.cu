@@ -29,6 +29,13 @@ constexpr unsigned long long kTaskCap = 1ull << 20;
 constexpr unsigned long long kCandPoolCap = 1ull << 24;
 constexpr size_t kStackBudget = 8ull << 30;   // first try; grows on FIM_E_STACK
 constexpr size_t kStackBudgetMax = 64ull << 30;
+constexpr int64_t kDirectWords = 1 << 16;        // frequent columns up to this many words: no projection
+constexpr int64_t kDirectWordsShort = 3 << 17;   // the same for few items in short rows
+constexpr unsigned long long kSmallPlanWords = 64ull << 20;  // worst-case projection of a device-planned mine
+constexpr unsigned long long kProjWords = 1ull << 30;  // largest projection (words)
+constexpr unsigned long long kTriples = 64ull << 20;   // largest table of triple supports
+constexpr uint32_t kProjWmax = 1u << 15;         // longest projected column (words)
+constexpr size_t kProjStackBudget = 4ull << 30;  // warp workers' global stacks
 
 }  // namespace
 
@@ -181,7 +188,8 @@ void fim_destroy(fim_ctx *ctx) {
                      &ctx->rule_conf, &ctx->rule_lift, &ctx->rule_sets, &ctx->probe_buf, &ctx->shard_cost, &ctx->merge_off, &ctx->mlp_w32, &ctx->mlp_wbf, &ctx->trace_x,
                      &ctx->trace_y, &ctx->mlp_scratch, &ctx->root_order, &ctx->root_bucket,
                      &ctx->root_hist, &ctx->rec_db, &ctx->dbdesc, &ctx->epoch, &ctx->sp_idx,
-                     &ctx->sp_val, &ctx->sp_z};
+                     &ctx->sp_val, &ctx->sp_z, &ctx->proj_items, &ctx->proj_tiles, &ctx->proj_totals,
+                     &ctx->proj_mat, &ctx->proj_list, &ctx->proj_cands, &ctx->proj_triple, &ctx->proj_roots};
     for (DevBuf *b : all) fim_release(ctx, *b);
     fim_release(ctx, ctx->batch_prefix);
     fim_release(ctx, ctx->batch_units);
@@ -300,6 +308,7 @@ struct MineState {
     int depth_cap = 0;
     int64_t frame_pool = 0;
     size_t stack_budget = kStackBudget;
+    bool cta_dfs = false;  // the warp workers' stack was too small: CTA workers
 };
 
 // One attempt at the whole mine with the current capacities.  Returns
@@ -336,6 +345,34 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     cudaEventRecord(ctx->ev[1], st);
     const bool do_pairs = mf >= 2 && (maxlen == 0 || maxlen >= 2);
     const bool do_dfs = do_pairs && mf >= 3 && (maxlen == 0 || maxlen >= 3);
+    // The plain search runs on warp workers (k_proj.cu); the network, diffset,
+    // trace and no-split options, and searches too deep for a warp worker's
+    // stack, on the CTA workers, which look at whole columns.
+    const bool warp_dfs = do_dfs && !ms.cta_dfs &&
+                          !(flags & (FIM_LEARNED | FIM_DIFFSET_RULE | FIM_TRACE | FIM_NO_SPLIT));
+    // Small matrices of short rows: few triples, which the bit columns
+    // themselves count sooner than three more launches would (5,746 x 99: 228
+    // against 247 us a mine); rows that hold a third of the frequent items make
+    // wide classes, better projected (12,060 x 46 at density 0.29: 343 against
+    // 507 us).  With more items than the one-launch plan takes, the plan's
+    // totals come back to the host, and the line lies lower.
+    const bool direct = warp_dfs && (proj_small_plan_fits(mf) ? (int64_t)mf * ctx->nwp <= kDirectWordsShort &&
+                                                                    3 * ctx->max_row_len <= mf
+                                                              : (int64_t)mf * ctx->nwp <= kDirectWords);
+    // Few frequent items: one launch plans the whole search (pair threshold,
+    // roots, projection), sized for the worst case, so that nothing has to
+    // come back to the host before the search.
+    const size_t npairs_all = (size_t)mf * (size_t)(mf > 0 ? mf - 1 : 0) / 2;
+    ProjTotals proj{};
+    proj.wmax = (uint32_t)(ceil_div64(ctx->n, 128) * 4);
+    proj.words = (unsigned long long)npairs_all * proj.wmax;
+    proj.rows = (unsigned long long)mf * (unsigned long long)ctx->n;
+    proj.cands = npairs_all;
+    proj.tiles = (unsigned long long)mf * ((proj.wmax + 31) / 32);
+    proj.triples = (unsigned long long)mf * mf * mf;
+    proj.units = (unsigned long long)mf * proj_triple_units(mf);
+    const bool small_plan = warp_dfs && ctx->n_shards == 1 && proj_small_plan_fits(mf) && proj.wmax <= kProjWmax &&
+                            proj.words <= kSmallPlanWords && proj.rows <= kSmallPlanWords;
     // automatic: keep low-support classes sparse when the frequent item
     // columns do not fit in half of L2 (streaming whole columns from HBM
     // is latency-bound; from L2 the dense pass is as fast)
@@ -348,7 +385,8 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     // while the pair pass runs (their kernel fits beside its CTAs).
     int64_t sp_cap = sparse_div > 0 ? ctx->nw / sparse_div : 0;
     if (sp_cap > ctx->nwp / 2) sp_cap = ctx->nwp / 2;
-    const bool sp_items = do_dfs && sp_cap > 0 && (double)mf * (double)sp_cap * 8.0 <= (double)(1ull << 30);
+    const bool sp_fits = do_dfs && sp_cap > 0 && (double)mf * (double)sp_cap * 8.0 <= (double)(1ull << 30);
+    const bool sp_items = sp_fits && !warp_dfs;
     if (sp_items) {
         FIM_TRY(reserve_sparse_items(ctx, mf, sp_cap));
         FIM_TRY(fim_aux_stream(ctx));
@@ -372,31 +410,67 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
             FIM_TRY(launch_sparse_items(ctx, mf, sp_cap, ctx->aux_stream));
             FIM_CUDA_TRY(cudaEventRecord(ctx->aux_ev[1], ctx->aux_stream));
         }
-        FIM_TRY(launch_pairs_finalize(ctx, thr, d_ctr));
+        if (small_plan) {
+            FIM_TRY(reserve_root_plan(ctx, npairs));
+            FIM_TRY(launch_proj_small_plan(ctx, thr, d_ctr, !direct));
+        } else {
+            FIM_TRY(launch_pairs_finalize(ctx, thr, d_ctr));
+        }
         // a shard of a split mine takes only the root classes it owns
         if (ctx->n_shards > 1) FIM_TRY(launch_shard_roots(ctx, d_ctr, ctx->shard, ctx->n_shards));
     }
     cudaEventRecord(ctx->ev[2], st);
+    bool on_warps = warp_dfs;
+    ctx->dfs_workers = ctx->num_sms * ctx->dfs_ctas_per_sm;
     if (do_dfs) {
-        const int workers = ctx->num_sms * ctx->dfs_ctas_per_sm;
+        if (warp_dfs && !direct && !small_plan) {
+            FIM_TRY(launch_proj_plan(ctx, &proj));
+            on_warps = proj.words <= kProjWords && proj.wmax <= kProjWmax && proj.cands < 0xFFFFFFFFull;
+        }
+        const int workers = ctx->dfs_workers * (on_warps ? proj_workers_per_cta() : 1);
+        ctx->dfs_workers = workers;
         // deepest class: a prefix can hold at most min(longest row, m') items
         int bound = ctx->max_row_len < mf ? ctx->max_row_len : mf;
         if (maxlen && (int)maxlen < bound) bound = (int)maxlen;
         if (bound > 240) bound = 240;  // the worker's shared-memory frame arrays hold 256 levels
         const int levels_needed = bound > 2 ? bound - 1 : 1;
-        const size_t per_level = (size_t)workers * (size_t)ctx->nwp * sizeof(uint32_t);
-        if (ms.depth_cap == 0) {
-            size_t cap = ms.stack_budget / (per_level ? per_level : 1);
-            ms.depth_cap = (int)(cap < (size_t)levels_needed ? cap : (size_t)levels_needed);
-            if (ms.depth_cap < 2) ms.depth_cap = 2;
+        ProjParams q{};
+        if (on_warps) {
+            const bool triples = !direct && ctx->n_shards == 1 && proj.triples <= kTriples;
+            if (!direct) FIM_TRY(launch_projection(ctx, proj, small_plan, triples, thr));
+            if (triples) {
+                q.triple = ctx->proj_triple.as<uint32_t>();
+                q.roots = ctx->proj_roots.as<unsigned long long>();
+            } else if (!small_plan) {  // candidate-less pairs dropped, the others ordered
+                FIM_TRY(reserve_root_plan(ctx, npairs_all));
+                FIM_TRY(launch_root_plan(ctx, d_ctr, npairs_all, nullptr, ctx->root_sort, nullptr, st));
+            }
+            q.items = ctx->proj_items.as<ProjItem>();
+            q.mat = ctx->proj_mat.as<uint32_t>();
+            q.cands = ctx->proj_cands.as<uint32_t>();
+            q.direct = direct ? 1 : 0;
+            q.direct_words = (int)round_up64(ctx->nw, 4);
+            const int64_t level = direct ? q.direct_words : (int64_t)proj.wmax;
+            // one level more than the classes: a queued task's own prefix
+            q.gstack = min64((int64_t)(levels_needed + 1) * level,
+                             (int64_t)(kProjStackBudget / sizeof(uint32_t)) / workers / 4 * 4);
+            if (q.gstack < 4) q.gstack = 4;
+            FIM_TRY(fim_reserve(ctx, ctx->stack_bits, sizeof(uint32_t) * (size_t)workers * (size_t)q.gstack));
+        } else {
+            const size_t per_level = (size_t)workers * (size_t)ctx->nwp * sizeof(uint32_t);
+            if (ms.depth_cap == 0) {
+                size_t cap = ms.stack_budget / (per_level ? per_level : 1);
+                ms.depth_cap = (int)(cap < (size_t)levels_needed ? cap : (size_t)levels_needed);
+                if (ms.depth_cap < 2) ms.depth_cap = 2;
+            }
+            FIM_TRY(fim_reserve(ctx, ctx->stack_bits, per_level * (size_t)ms.depth_cap));
         }
         if (ms.frame_pool == 0) ms.frame_pool = 4LL * mf + 1024;
-        FIM_TRY(fim_reserve(ctx, ctx->stack_bits, per_level * (size_t)ms.depth_cap));
         FIM_TRY(fim_reserve(ctx, ctx->frame_items, sizeof(uint32_t) * (size_t)workers * ms.frame_pool));
-        FIM_TRY(fim_reserve(ctx, ctx->frame_sups, sizeof(uint32_t) * (size_t)workers * ms.frame_pool));
+        if (!on_warps) FIM_TRY(fim_reserve(ctx, ctx->frame_sups, sizeof(uint32_t) * (size_t)workers * ms.frame_pool));
         FIM_TRY(prepare_task_queue(ctx, sizeof(Task) * kTaskCap));
         FIM_TRY(fim_reserve(ctx, ctx->cand_pool, sizeof(uint32_t) * kCandPoolCap));
-        FIM_TRY(launch_epoch_bump(ctx));
+        if (!small_plan) FIM_TRY(launch_epoch_bump(ctx));
         const size_t npairs = (size_t)mf * (mf - 1) / 2;
         DfsParams p{};
         p.dbs = ctx->dbdesc.as<DbDesc>();
@@ -433,8 +507,13 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         p.learned_kmin = ctx->learned_kmin;
         p.rec_chunk = ctx->rec_chunk;
         p.root_reverse = ctx->root_reverse;
-        if (sp_items) {
-            FIM_CUDA_TRY(cudaStreamWaitEvent(st, ctx->aux_ev[1], 0));
+        const bool sp_late = sp_fits && warp_dfs && !on_warps;
+        if (sp_late) {  // the warp workers' projection was too large after all
+            FIM_TRY(reserve_sparse_items(ctx, mf, sp_cap));
+            FIM_TRY(launch_sparse_items(ctx, mf, sp_cap, st));
+        }
+        if (sp_items || sp_late) {
+            if (sp_items) FIM_CUDA_TRY(cudaStreamWaitEvent(st, ctx->aux_ev[1], 0));
             p.item_idx = ctx->sp_idx.as<uint32_t>();
             p.item_val = ctx->sp_val.as<uint32_t>();
             p.item_z = ctx->sp_z.as<int>();
@@ -446,7 +525,9 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         p.learned = (flags & FIM_LEARNED) ? 1 : 0;
         p.diffset_rule = (flags & FIM_DIFFSET_RULE) ? 1 : 0;
         p.mlp_w = ctx->mlp_wbf.as<__nv_bfloat16>();
-        {   // candidate-less roots dropped, the others ordered
+        if (on_warps) {
+            p.root_order = q.triple ? nullptr : ctx->root_order.as<uint32_t>();
+        } else {  // candidate-less roots dropped, the others ordered
             const int mode = (p.learned && ctx->learned_order) ? 2 : ctx->root_sort;
             FIM_TRY(reserve_root_plan(ctx, npairs));
             FIM_TRY(launch_root_plan(ctx, d_ctr, npairs, nullptr, mode, nullptr, st));
@@ -463,12 +544,18 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
             p.trace_y = ctx->trace_y.as<float>();
             p.trace_cap = ctx->trace_cap;
         }
-        FIM_TRY(launch_dfs(ctx, p, workers, ctx->dfs_block));
+        if (on_warps) FIM_TRY(launch_dfs_proj(ctx, p, q, ctx->dfs_ctas_per_sm));
+        else FIM_TRY(launch_dfs(ctx, p, workers, ctx->dfs_block));
     }
     cudaEventRecord(ctx->ev[3], st);
     FIM_CUDA_TRY(cudaMemcpyAsync(&ctx->host_ctr, d_ctr, sizeof(MineCounters), cudaMemcpyDeviceToHost, st));
     FIM_CUDA_TRY(cudaStreamSynchronize(st));
     const MineCounters &c = ctx->host_ctr;
+    if (c.err == FIM_E_STACK && on_warps) {
+        ms.cta_dfs = true;
+        *retry = true;
+        return FIM_OK;
+    }
     if (c.err == FIM_E_STACK) {
         if (ms.stack_budget >= kStackBudgetMax) return FIM_E_STACK;
         ms.stack_budget *= 2;
@@ -555,7 +642,7 @@ int fim_mine(fim_ctx *ctx, uint64_t minsup, uint32_t flags) {
     s.launches_mine = ctx->launches - launches0;
     s.dfs_busy_ns = c.busy_ns;
     s.dfs_span_ns = c.t_last > c.t_first && c.t_first != 0 ? c.t_last - c.t_first : 0;
-    s.dfs_workers = (uint64_t)ctx->num_sms * (uint64_t)ctx->dfs_ctas_per_sm;
+    s.dfs_workers = (uint64_t)ctx->dfs_workers;
     s.dfs_root_ns = c.root_ns;
     if (ctx->bytes_held > s.peak_device_bytes) s.peak_device_bytes = ctx->bytes_held;
     if (ctx->debug_checks) FIM_TRY(run_check_output(ctx, thr));

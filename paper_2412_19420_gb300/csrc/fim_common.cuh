@@ -102,6 +102,12 @@ struct MineCounters {
     // references), left out of the canonical output
     unsigned long long rec_holes;
     unsigned long long item_holes;
+    // The warp workers' queue (k_proj.cu), one counter to a 128-byte line: the
+    // waiting workers' polls and the busy ones' atomics do not share lines.
+    alignas(128) unsigned long long w_head;     // queue slots taken
+    alignas(128) unsigned long long w_tail;     // queue slots filled
+    alignas(128) unsigned long long w_pool;     // next free word of the candidate pool
+    unsigned long long n_triples;               // frequent triples with a later candidate (roots)
 };
 
 // A pushed prefix class: items (internal ids) + support + candidate list.
@@ -216,6 +222,33 @@ struct DfsParams {
     RootWindow *win;                // warp workers: only this window's roots (null: all of them)
 };
 
+// The projection of one frequent item a (k_proj.cu): its transactions and
+// the columns of its candidates restricted to them.
+struct ProjItem {
+    unsigned long long moff;  // first word of its columns
+    unsigned long long loff;  // first entry of its row list
+    uint32_t coff;            // first entry of its candidate list
+    uint32_t k;               // candidates (columns); 0: no projection
+    uint32_t W;               // words per column
+    uint32_t s;               // S(a): rows
+    uint32_t cursor;          // rows listed so far
+    uint32_t pad;
+    unsigned long long toff;  // first triple support
+};
+struct ProjTotals {
+    unsigned long long words, rows, cands, tiles, triples, units;
+    uint32_t wmax, pad;
+};
+struct ProjParams {
+    const ProjItem *items;
+    const uint32_t *mat, *cands;
+    const uint32_t *triple;            // triple supports (0: infrequent); null: the roots are pairs ...
+    const unsigned long long *roots;   // ... else the frequent triples
+    int64_t gstack;    // global stack words per worker
+    int direct;        // 1: no projection, the bit columns themselves ...
+    int direct_words;  // ... of this many words (a multiple of 4)
+};
+
 // ---------------------------------------------------------------- the ctx
 struct fim_ctx {
     int device = 0;
@@ -240,6 +273,7 @@ struct fim_ctx {
     DevBuf tasks, cand_pool, stack_bits, frame_items, frame_sups;
     DevBuf epoch;               // uint32: mine counter; a task slot is live when ready == epoch
     DevBuf sp_idx, sp_val, sp_z; // sparse copies of low-support frequent item columns
+    DevBuf proj_items, proj_tiles, proj_totals, proj_mat, proj_list, proj_cands, proj_triple, proj_roots;  // projected columns (k_proj.cu)
     DevBuf rec_off, rec_len, rec_sup, rec_items, rec_db;
     DevBuf counters;            // MineCounters
     DevBuf dbdesc;              // DbDesc table of the mine
@@ -311,6 +345,7 @@ struct fim_ctx {
     // tuning (autotuner may overwrite)
     int dfs_block = 256;
     int dfs_ctas_per_sm = 4;
+    int dfs_workers = 0;        // DFS workers (CTAs or warps) of the mine in progress
     int split_depth = 8;
     int sparse_div = -1;        // -1: automatic (frequent columns vs L2)
     int learned_kmin = 8;
@@ -382,6 +417,15 @@ int launch_dfs(fim_ctx *ctx, const DfsParams &p, int grid, int block);
 // replayed graph bumps it too) and clear the slots only when the buffer is new.
 int prepare_task_queue(fim_ctx *ctx, size_t bytes);
 int launch_epoch_bump(fim_ctx *ctx);
+// k_proj.cu: projected columns and the prefix extension on them.  The plan
+// synchronises the stream (its totals size the buffers).
+int launch_proj_plan(fim_ctx *ctx, ProjTotals *host);
+int launch_projection(fim_ctx *ctx, const ProjTotals &t, bool cands_listed, bool triples, uint32_t thr);
+bool proj_small_plan_fits(int mf);
+int launch_proj_small_plan(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr, bool triples);
+unsigned long long proj_triple_units(int mf);  // most units of the triple pass
+int launch_dfs_proj(fim_ctx *ctx, const DfsParams &p, const ProjParams &q, int ctas_per_sm);
+int proj_workers_per_cta();
 // Sparse copies of the frequent item columns with S <= cap (single database).
 // sparse copies of the low-support item columns for the root classes: the
 // buffers first (host side), then the copy, on a stream of the caller's
