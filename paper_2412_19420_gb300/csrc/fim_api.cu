@@ -161,7 +161,7 @@ int fim_create(fim_ctx **out, int device, void *cuda_stream) {
     }
     for (auto &e : ctx->ev) cudaEventCreate(&e);
     int rc = fim_reserve(ctx, ctx->counters, sizeof(MineCounters));
-    if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->dev_flag, 4 * sizeof(int));
+    if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->dev_flag, sizeof(BuildFlags));
     if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->epoch, sizeof(uint32_t));
     if (rc == FIM_OK && cudaMemsetAsync(ctx->epoch.p, 0, sizeof(uint32_t), ctx->stream) != cudaSuccess) rc = FIM_E_CUDA;
     if (rc != FIM_OK) {
@@ -177,7 +177,7 @@ void fim_destroy(fim_ctx *ctx) {
     if (!ctx) return;
     DeviceGuard g(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    DevBuf *all[] = {&ctx->csr_ptr, &ctx->csr_idx, &ctx->bm, &ctx->item_sup, &ctx->perm, &ctx->rank,
+    DevBuf *all[] = {&ctx->csr_ptr, &ctx->csr_idx, &ctx->bm, &ctx->row_ptr, &ctx->row_idx, &ctx->item_sup, &ctx->perm, &ctx->rank,
                      &ctx->dev_flag, &ctx->pair_cnt, &ctx->pairbits, &ctx->roots, &ctx->tasks,
                      &ctx->cand_pool, &ctx->stack_bits, &ctx->frame_items, &ctx->frame_sups,
                      &ctx->rec_off, &ctx->rec_len, &ctx->rec_sup, &ctx->rec_items, &ctx->counters,
@@ -209,6 +209,8 @@ void fim_destroy(fim_ctx *ctx) {
     for (cudaEvent_t e : ctx->copy_ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : ctx->aux_ev)
+        if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : ctx->pair_ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : ctx->up_ev)
         if (e) cudaEventDestroy(e);
@@ -287,11 +289,14 @@ int fim_build_bitmaps(fim_ctx *ctx, const void *indptr, const void *indices, int
     cudaEventRecord(ctx->ev[1], st);
     FIM_TRY(launch_item_support(ctx));
     cudaEventRecord(ctx->ev[2], st);
-    int flag[2] = {0, 0};
-    FIM_CUDA_TRY(cudaMemcpyAsync(flag, ctx->dev_flag.p, sizeof(flag), cudaMemcpyDeviceToHost, st));
+    BuildFlags bf{};
+    FIM_CUDA_TRY(cudaMemcpyAsync(&bf, ctx->dev_flag.p, sizeof(bf), cudaMemcpyDeviceToHost, st));
     FIM_CUDA_TRY(cudaStreamSynchronize(st));
-    if (flag[0]) return FIM_E_INVAL;
-    ctx->max_row_len = flag[1];
+    if (bf.bad) return FIM_E_INVAL;
+    ctx->max_row_len = bf.max_len;
+    ctx->row_nnz = bf.nnz;
+    ctx->row_pairs = bf.row_pairs;
+    ctx->rows_kept = ctx->row_cap > 0 && (uint64_t)bf.nnz <= ctx->row_cap;
     cudaEventElapsedTime(&ctx->stats.ms_build, ctx->ev[0], ctx->ev[1]);
     cudaEventElapsedTime(&ctx->stats.ms_singletons, ctx->ev[1], ctx->ev[2]);
     if (ctx->debug_checks) FIM_TRY(run_check_pads(ctx));
@@ -403,7 +408,8 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         FIM_TRY(fim_reserve(ctx, ctx->pairbits, sizeof(uint32_t) * (size_t)mf * mpw));
         FIM_TRY(fim_reserve(ctx, ctx->roots, sizeof(uint32_t) * 3 * npairs));
         int rc = FIM_E_INVAL;
-        if (!(flags & FIM_PAIRS_POPC)) rc = launch_pairs_tc(ctx);
+        if (!(flags & FIM_PAIRS_POPC))
+            rc = pairs_rows_pays(ctx) ? launch_pairs_rows(ctx) : launch_pairs_tc(ctx, 0, true, st);
         if (rc == FIM_OK) ctx->stats.pair_path = 1;
         else FIM_TRY(launch_pairs_popc(ctx));
         if (sp_items) {  // launched after the pair pass, so that its CTAs take the SMs first

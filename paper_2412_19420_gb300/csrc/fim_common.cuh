@@ -102,6 +102,7 @@ struct MineCounters {
     // references), left out of the canonical output
     unsigned long long rec_holes;
     unsigned long long item_holes;
+    unsigned long long sup_sum;      // sum of the item supports
     // The warp workers' queue (k_proj.cu), one counter to a 128-byte line: the
     // waiting workers' polls and the busy ones' atomics do not share lines.
     alignas(128) unsigned long long w_head;     // queue slots taken
@@ -222,6 +223,21 @@ struct DfsParams {
     RootWindow *win;                // warp workers: only this window's roots (null: all of them)
 };
 
+// What fim_build_bitmaps' kernels report.
+struct BuildFlags {
+    int bad;                       // 1: malformed CSR
+    int max_len;                   // longest row
+    long long nnz;                 // indptr[n]
+    unsigned long long row_pairs;  // sum over the rows of len (len - 1) / 2
+};
+// The rows kept for the pair pass; cap 0: none.
+struct RowCopy {
+    uint32_t *ptr;        // [n + 1]
+    unsigned short *idx;  // [cap]
+    uint64_t cap;         // rows with more items in all are not kept
+};
+constexpr uint64_t kRowCopyItems = 24;
+
 // The projection of one frequent item a (k_proj.cu): its transactions and
 // the columns of its candidates restricted to them.
 struct ProjItem {
@@ -263,6 +279,12 @@ struct fim_ctx {
     int64_t nw = 0, nwp = 0;
     int max_row_len = 0;
     DevBuf csr_ptr, csr_idx;   // staging for host input
+    DevBuf row_ptr, row_idx;   // the rows, kept for the pair pass (RowCopy)
+    uint64_t row_cap = 0;
+    int64_t row_nnz = 0;            // items in the rows
+    uint64_t row_pairs = 0;         // pairs of items that share a row
+    bool rows_kept = false;         // row_ptr / row_idx hold this matrix's rows
+    cudaEvent_t pair_ev[2] = {};    // fork and join of the pair pass's two halves
     DevBuf bm, item_sup, perm, rank, dev_flag;
 
     // mine
@@ -407,7 +429,11 @@ int launch_max_row_freq(fim_ctx *ctx, const int64_t *d_indptr, const int32_t *d_
 
 // k_pairs.cu
 int launch_pairs_popc(fim_ctx *ctx);
-int launch_pairs_tc(fim_ctx *ctx);   // tcgen05; returns FIM_E_INVAL if unsupported
+// tcgen05, the pairs of items a0 .. m' - 1 (0: all); the counts are cleared
+// first unless clear is false
+int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st);
+bool pairs_rows_pays(const fim_ctx *ctx);
+int launch_pairs_rows(fim_ctx *ctx);  // rows, and the most frequent items' block by launch_pairs_tc
 int launch_pairs_finalize(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr);
 
 // k_dfs.cu

@@ -22,7 +22,7 @@ template <bool CMP>
 __global__ void __launch_bounds__(BUILD_THREADS)
 build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__ indices_v,
                      int64_t n, int32_t m, int64_t nnz, int64_t nwp, int ib, int64_t blk0,
-                     uint32_t *__restrict__ bm, int *__restrict__ flag, int *__restrict__ max_len) {
+                     uint32_t *__restrict__ bm, BuildFlags *__restrict__ flags, RowCopy rows) {
     using Off = typename std::conditional<CMP, uint32_t, int64_t>::type;
     using Id = typename std::conditional<CMP, unsigned short, int32_t>::type;
     const Off *const indptr = static_cast<const Off *>(indptr_v);
@@ -30,6 +30,8 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
     // [WB][ib + 1], word-major and padded: the 32 rows of a warp's group share
     // their word, so their items' bits spread over the banks
     extern __shared__ __align__(16) uint32_t tile[];
+    __shared__ int s_max;
+    __shared__ unsigned long long s_pairs;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ms = ib + 1;
     const int64_t w0 = (blk0 + (int64_t)blockIdx.x) * WB;
@@ -38,13 +40,21 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
     const int64_t t0 = w0 * 32;
     const int64_t t1 = min(n, t0 + WB * 32);
     int bad = 0, my_max = 0;
+    unsigned long long my_pairs = 0;
     if (nnz < 0) {  // device input: indptr[n] read here, and indptr[0] checked once
         nnz = (int64_t)indptr[n];
         if (nnz < 0) bad = 1;
         if (blockIdx.x == 0 && blockIdx.y == 0 && blk0 == 0 && threadIdx.x == 0 && indptr[0] != 0) bad = 1;
     }
+    const bool first = blockIdx.y == 0;  // this CTA's items are the first: it also sees to the rows
+    const bool copy = first && (uint64_t)nnz <= rows.cap;
+    if (first && blk0 == 0 && blockIdx.x == 0 && threadIdx.x == 0) flags->nnz = nnz;
 
     for (int k = threadIdx.x; k < WB * ms; k += blockDim.x) tile[k] = 0u;
+    if (threadIdx.x == 0) {
+        s_max = 0;
+        s_pairs = 0;
+    }
     __syncthreads();
     // warp w takes 32-row groups: lane i holds the group's start of row i, the
     // warp streams the group's elements 32 at a time (coalesced) and each
@@ -57,7 +67,13 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         if (lane == nr - 1) off_next = e_end;
         if (lane < nr) {
             if (off_next < off || off < 0 || off_next > nnz) bad = 1;
-            else my_max = max(my_max, (int)min64(off_next - off, 1 << 30));
+            else {
+                const int64_t len = off_next - off;
+                my_max = max(my_max, (int)min64(len, 1 << 30));
+                my_pairs += (unsigned long long)len * (unsigned long long)(len - 1) / 2;
+                if (copy) rows.ptr[rb + lane] = (uint32_t)off;
+                if (copy && rb + lane == n - 1) rows.ptr[n] = (uint32_t)off_next;
+            }
         }
         if (__any_sync(0xffffffffu, bad)) continue;  // malformed: flagged, not read
         const int64_t e_begin = __shfl_sync(0xffffffffu, off, 0);
@@ -75,13 +91,26 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
             }
             if (!v) continue;
             if (it < 0 || it >= m) { bad = 1; continue; }
+            if (copy) rows.idx[e] = (unsigned short)it;
             if (it < i0 || it >= i0 + icount) continue;
             atomicOr(&tile[wl * ms + (it - i0)], 1u << r);
         }
     }
-    if (bad) atomicExch(flag, 1);
-    if (blockIdx.y == 0 && my_max > 0) atomicMax(max_len, my_max);
+    if (bad) atomicExch(&flags->bad, 1);
+    if (first) {  // one pair of global atomics per CTA
+        my_max = (int)__reduce_max_sync(0xffffffffu, (unsigned)my_max);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) my_pairs += __shfl_xor_sync(0xffffffffu, my_pairs, o);
+        if (lane == 0) {
+            atomicMax(&s_max, my_max);
+            atomicAdd(&s_pairs, my_pairs);
+        }
+    }
     __syncthreads();
+    if (first && threadIdx.x == 0 && s_max > 0) {
+        atomicMax(&flags->max_len, s_max);
+        atomicAdd(&flags->row_pairs, s_pairs);
+    }
     // write-out: 16-byte stores, four consecutive threads per 64-byte row
     for (int k = threadIdx.x; k < icount * (WB / 4); k += blockDim.x) {
         const int r = k / (WB / 4), c = k % (WB / 4);
@@ -123,6 +152,13 @@ __global__ void rank_items_kernel(const uint32_t *__restrict__ sup, int32_t m, u
     const int lane = threadIdx.x & 31;
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (j >= m) return;
+    if (j == 0) {  // the supports' sum tells whether a row repeats an item
+        unsigned long long t = 0;
+        for (int i = lane; i < m; i += 32) t += sup[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) ctr->sup_sum = t;
+    }
     const uint32_t sj = sup[j];
     if (sj < thr) {
         if (lane == 0) rank[j] = -1;
@@ -174,9 +210,24 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
     const int niblk = (int)ceil_div64(ctx->m > 0 ? ctx->m : 1, ib);
     const size_t smem = (size_t)(ib + 1) * WB * sizeof(uint32_t);
     FIM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int *flag = ctx->dev_flag.as<int>();
+    BuildFlags *flags = ctx->dev_flag.as<BuildFlags>();
     cudaStream_t st = ctx->stream;
-    FIM_CUDA_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(int), st));
+    FIM_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(BuildFlags), st));
+    // the rows, kept as 32-bit offsets and 16-bit ids for the pair pass, where
+    // they hold at most kRowCopyItems items on average (longer rows make more
+    // pairs than the tensor cores' pass costs)
+    RowCopy rows{};
+    if (ctx->n > 0 && ctx->m > 0) {
+        const uint64_t cap = (uint64_t)ctx->n * kRowCopyItems;
+        if (cap < 0xFFFFFFFFull) {
+            FIM_TRY(fim_reserve(ctx, ctx->row_ptr, sizeof(uint32_t) * (size_t)(ctx->n + 1)));
+            FIM_TRY(fim_reserve(ctx, ctx->row_idx, sizeof(unsigned short) * (size_t)cap));
+            rows.ptr = ctx->row_ptr.as<uint32_t>();
+            rows.idx = ctx->row_idx.as<unsigned short>();
+            rows.cap = cap;
+        }
+    }
+    ctx->row_cap = rows.cap;
     if (nblk <= 0 || ctx->m <= 0) return FIM_OK;
     // device input (nnz < 0): the kernel reads indptr[n] itself
     // Host input: the indices go up in chunks of row blocks on side streams,
@@ -217,7 +268,7 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
         dim3 grid((unsigned)(b1 - b0), (unsigned)niblk);
         ctx->launches++;
         kern<<<grid, BUILD_THREADS, smem, st>>>(d_indptr, d_indices, ctx->n, ctx->m, nnz, ctx->nwp, ib, b0,
-                                                ctx->bm.as<uint32_t>(), flag, flag + 1);
+                                                ctx->bm.as<uint32_t>(), flags, rows);
         FIM_CUDA_TRY(cudaGetLastError());
     }
     return FIM_OK;

@@ -38,6 +38,8 @@
 // Tensor memory: the 256-column accumulator at column 0, then one 32-column
 // A slot per pipeline stage.  Shared-memory traffic per stage is the B tile
 // written once and read once (64 KB for 8.4 MFLOP).
+// The pass covers the pairs of items a0 .. m' - 1: all of them, or (beside the
+// row pass of k_pairs_rows.cu) the block of the most frequent ones.
 // Every mbarrier wait is bounded; on expiry the CTA records an error, lets
 // its MMAs finish, frees its tensor memory and returns.
 #include "fim_common.cuh"
@@ -122,7 +124,7 @@ __device__ __forceinline__ Seg next_seg(int64_t w, int64_t w1, int64_t S, int kd
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
-pairs_tc_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ perm, int64_t nwp, int mf,
+pairs_tc_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ perm, int64_t nwp, int mf, int ld,
                 int ntb, int64_t S, int64_t W, int kd, int *__restrict__ pair_cnt, int *__restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     TcSmem &s = *reinterpret_cast<TcSmem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -282,7 +284,7 @@ pairs_tc_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ per
                     const int rr = 2 * i + (lane >> 4);
                     const int a = ta * TM + q * 32 + rr;
                     const int val = xp[c][rr];
-                    if (a < b && b < mf && val) atomicAdd(&pair_cnt[(int64_t)a * mf + b], val);
+                    if (a < b && b < mf && val) atomicAdd(&pair_cnt[(int64_t)a * ld + b], val);
                 }
                 __syncwarp();
             }
@@ -344,8 +346,8 @@ pairs_tc_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ per
 
 }  // namespace
 
-int launch_pairs_tc(fim_ctx *ctx) {
-    const int mf = ctx->mfreq;
+int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st) {
+    const int ld = ctx->mfreq, mf = ld - a0;
     if (mf < 2) return FIM_OK;
     const int nta = (int)ceil_div64(mf, TM), ntb = (int)ceil_div64(mf, TN);
     int64_t tiles = 0;
@@ -357,13 +359,13 @@ int launch_pairs_tc(fim_ctx *ctx) {
     if (grid > W) grid = W;
     const size_t smem = sizeof(TcSmem) + 1024;
     FIM_CUDA_TRY(cudaFuncSetAttribute(pairs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    FIM_CUDA_TRY(cudaMemsetAsync(ctx->pair_cnt.p, 0, sizeof(int) * (size_t)mf * mf, ctx->stream));
+    if (clear) FIM_CUDA_TRY(cudaMemsetAsync(ctx->pair_cnt.p, 0, sizeof(int) * (size_t)ld * ld, st));
     int *err = &ctx->counters.as<MineCounters>()->err;  // zeroed at the start of every mine
     if (grid > 0) {
         ctx->launches++;
-        pairs_tc_kernel<<<(unsigned)grid, THREADS, smem, ctx->stream>>>(
-            ctx->bm.as<uint32_t>(), ctx->perm.as<int32_t>(), ctx->nwp, mf, ntb, S, W, kd,
-            ctx->pair_cnt.as<int>(), err);
+        pairs_tc_kernel<<<(unsigned)grid, THREADS, smem, st>>>(
+            ctx->bm.as<uint32_t>(), ctx->perm.as<int32_t>() + a0, ctx->nwp, mf, ld, ntb, S, W, kd,
+            ctx->pair_cnt.as<int>() + (size_t)a0 * ld + a0, err);
         FIM_CUDA_TRY(cudaGetLastError());
     }
     return FIM_OK;

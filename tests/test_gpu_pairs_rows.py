@@ -1,0 +1,83 @@
+"""The row pass of the pair supports (k_pairs_rows.cu) against the oracle and
+the CUDA-core pair pass: taken where rows are short and items many, exact at
+the edges of a warp's tile of 32 rows, for empty, long and very long rows (a
+row longer than a warp's buffer), beside the tensor cores' block of the 256
+most frequent items, and left alone where a row repeats an item."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2412_19420_gb300 import datagen
+
+pytestmark = pytest.mark.gpu
+fim = pytest.importorskip("paper_2412_19420_gb300.fim")
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = fim.fim_create(0)
+    yield c
+    fim.fim_destroy(c)
+
+
+def _pairs(ctx, c, minsup, flags=0):
+    fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+    fim.fim_mine(ctx, minsup, flags | fim.FIM_MAXLEN(2))
+    return fim.fim_fetch_results(ctx).sha256()
+
+
+def _rows(n, m, seed, mean, long_rows=(), empty=0.1):
+    """Distinct ascending items a row, Poisson lengths, some rows empty, some
+    (row, length) very long."""
+    rng = np.random.default_rng(seed)
+    lens = rng.poisson(mean, n)
+    lens[rng.random(n) < empty] = 0
+    for r, k in long_rows:
+        lens[r] = k
+    return datagen.from_lists([sorted(rng.choice(m, size=k, replace=False)) for k in lens], m)
+
+
+# m' at the edge of the tensor cores' block (256), of a B tile (512), and far
+# beyond it; n at the edges of a 32-row tile
+@pytest.mark.parametrize("n,m", [(40_000, 257), (40_001, 300), (39_999, 513), (60_000, 1500)])
+def test_row_pairs_vs_oracle(ctx, n, m):
+    c = datagen.zipf_baskets(n, m, 0.3, 5.0, [n, m])
+    for minsup in (1, 12):
+        want = oracle.apriori(c.indptr, c.indices, c.m, minsup, max_len=2)
+        assert _pairs(ctx, c, minsup) == want.sha256()
+
+
+def test_long_and_empty_rows(ctx):
+    # rows of 31..33, 1,000..1,100 and 1,500 items: several to a buffer, one
+    # that just fits, one that does not
+    long_rows = [(0, 31), (1, 32), (2, 33), (500, 1000), (501, 1024), (502, 1025), (503, 1100), (29_999, 1500)]
+    c = _rows(30_000, 1600, 5, 4, long_rows)
+    want = oracle.apriori(c.indptr, c.indices, c.m, 3, max_len=2)
+    assert _pairs(ctx, c, 3) == want.sha256()
+    assert _pairs(ctx, c, 3, fim.FIM_PAIRS_POPC) == want.sha256()
+
+
+def test_repeated_items_take_the_set_path(ctx):
+    # one row in a thousand names an item twice: counted once all the same
+    rng = np.random.default_rng(8)
+    rows = [list(rng.choice(600, size=5, replace=False)) for _ in range(40_000)]
+    for r in range(0, 40_000, 1000):
+        rows[r] += rows[r][:2]
+    c = datagen.from_lists(rows, 600)
+    want = oracle.apriori(c.indptr, c.indices, c.m, 4, max_len=2)
+    assert _pairs(ctx, c, 4) == want.sha256()
+
+
+def test_compact_device_rows_and_rebuilds(ctx):
+    # the kept rows are this matrix's: build A, build B, mine B; device input
+    import torch
+    a, b = datagen.zipf_baskets(50_000, 700, 0.3, 6.0, 1), datagen.zipf_baskets(30_011, 900, 0.3, 5.0, 2)
+    for c in (a, b, a):
+        ip = torch.from_numpy(c.indptr.astype(np.int32)).cuda()
+        ix = torch.from_numpy(c.indices.astype(np.uint16).view(np.int16)).cuda()
+        fim.fim_build_bitmaps(ctx, ip, ix, c.m)
+        del ip, ix  # the library keeps no pointer of the caller's
+        torch.cuda.empty_cache()
+        fim.fim_mine(ctx, 15)
+        want = oracle.apriori(c.indptr, c.indices, c.m, 15)
+        assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
