@@ -487,13 +487,13 @@ bool batch_pairs_tc_units(const std::vector<DbDesc> &dbs, int d0, int d1, std::v
 // d_n_units: the unit count written on the device by the plan kernel (null:
 // n_units itself); n_units is then the capacity, which sizes the grid
 int launch_batch_pairs_tc(fim_ctx *ctx, const DbDesc *d_dbs, const unsigned long long *d_units, int64_t n_units,
-                          const long long *d_n_units, cudaStream_t st);
+                          const long long *d_n_units, const long long *d_pre, cudaStream_t st);
 // Device plan of one group's pair units once m'_d is known: ord[0 .. n) the
 // group's databases, most transactions first; databases with at most 64
 // frequent items are packed two to a tile; *d_n_units gets the count.
 // scratch: batch_pair_plan_scratch(n) bytes.
 int launch_batch_pair_plan(fim_ctx *ctx, const DbDesc *d_dbs, const int *d_ord, int n, unsigned long long *d_units,
-                           long long *d_n_units, void *scratch, cudaStream_t st);
+                           long long *d_pre, long long *d_n_units, void *scratch, cudaStream_t st);
 size_t batch_pair_plan_scratch(int n);
 extern const int kBatchPairsShapeCount;
 

@@ -135,6 +135,83 @@ __device__ __forceinline__ BUnit decode_unit(const DbDesc *__restrict__ dbs, uns
     return u;
 }
 
+// A CTA's work.  With pre (pre[u] = work before unit u, pre[n_units] = all of
+// it; a unit of S stages counts S + UNIT_COST) CTA c of G takes share
+// [c W / G, (c + 1) W / G) of the units laid end to end: every SM gets the same
+// work, however few or uneven the databases are, and a unit cut by a share's
+// end is summed from its parts by atomics (its counts are cleared beforehand).
+// Dealing whole units left SMs idle: 48 databases are 30 units, 293 us, and
+// 25 shared.  UNIT_COST is what a unit costs beside its stages (descriptors,
+// pipeline fill, drain: about 6 us), in stages of about 0.54 us; counted
+// without it, the CTAs that got the small databases took twice the others'
+// time (4,096 databases: 2.6 ms).
+constexpr int64_t UNIT_COST = 12;
+constexpr int64_t MIN_SHARE = 24;  // shorter shares pay UNIT_COST more than they save
+// With DEAL units a CTA or more, whole units in rounds of alternating direction
+// even out by themselves and nothing is cut (4,096 databases: 1.42 ms, 1.47 in
+// shares).
+constexpr int64_t DEAL = 3;
+__device__ __forceinline__ bool shares(int64_t n_units) { return n_units < DEAL * (int64_t)gridDim.x; }
+struct Walk {
+    int64_t k, ui;        // round (whole units), unit; ui >= n: done
+    int64_t n, w, w1;     // units; this share's next work and end
+    int64_t s0, s1;       // stages of the unit
+    bool split;           // the unit's other stages are another CTA's
+};
+__device__ __forceinline__ int64_t walk_grid(int64_t W) {
+    const int64_t most = W / MIN_SHARE > 1 ? W / MIN_SHARE : 1;
+    return most < (int64_t)gridDim.x ? most : (int64_t)gridDim.x;
+}
+// the unit at x.ui, or the next one in which this share has stages
+__device__ __forceinline__ void walk_set(Walk &x, const long long *pre) {
+    while (x.ui < x.n && x.w < x.w1) {
+        const int64_t b = pre[x.ui], e = pre[x.ui + 1], S = e - b - UNIT_COST;
+        x.s0 = max64(x.w - b - UNIT_COST, 0);
+        x.s1 = max64(min64(x.w1, e) - b - UNIT_COST, 0);
+        x.split = x.s0 > 0 || x.s1 < S;
+        if (x.s0 < x.s1) return;
+        x.w = e;  // the share ends inside the unit's fixed cost
+        x.ui++;
+    }
+    x.ui = x.n;
+}
+__device__ __forceinline__ Walk walk_begin(int64_t n_units, const long long *pre) {
+    Walk x{};
+    x.n = n_units;
+    if (!pre) {
+        x.ui = blockIdx.x;
+        return x;
+    }
+    const int64_t W = n_units > 0 ? pre[n_units] : 0, G = walk_grid(W);
+    if ((int64_t)blockIdx.x >= G || W == 0) { x.ui = n_units; return x; }
+    x.w = (int64_t)blockIdx.x * W / G;
+    x.w1 = ((int64_t)blockIdx.x + 1) * W / G;
+    int64_t lo = 0, hi = n_units;  // pre[lo] <= w < pre[hi]
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (pre[mid] <= x.w) lo = mid; else hi = mid;
+    }
+    x.ui = lo;
+    walk_set(x, pre);
+    return x;
+}
+__device__ __forceinline__ void walk_next(Walk &x, const long long *pre) {
+    if (!pre) {
+        const int64_t G = gridDim.x, c = blockIdx.x;
+        x.k++;
+        x.ui = x.k * G + ((x.k & 1) ? G - 1 - c : c);
+        return;
+    }
+    x.w = pre[x.ui + 1];
+    x.ui++;
+    walk_set(x, pre);
+}
+// the unit's stages this CTA runs
+__device__ __forceinline__ void walk_span(const Walk &x, const long long *pre, int64_t S, int64_t &s0, int64_t &s1) {
+    s0 = pre ? x.s0 : 0;
+    s1 = pre ? x.s1 : S;
+}
+
 template <typename S>
 __device__ __forceinline__ bool bwait(S &s, uint64_t *b, uint32_t parity) {
     return mbar_wait_bounded(b, parity, &s.abort, BWAIT_NS);
@@ -145,7 +222,7 @@ template <int STG, int DEPTH, int MINB, int BG>
 __global__ void __launch_bounds__(BTHREADS, MINB)
 batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *__restrict__ units,
                       int64_t n_units_host, const long long *__restrict__ n_units_dev,
-                      const uint32_t *__restrict__ bm, const int32_t *__restrict__ perm_base,
+                      const long long *pre, const uint32_t *__restrict__ bm, const int32_t *__restrict__ perm_base,
                       int *__restrict__ pair_cnt, int kd, int *__restrict__ err) {
     static_assert(DEPTH % 4 == 0 && DEPTH >= 8, "raw bits go in quads, two or more in flight");
     static_assert(BG == 2 || BG == 4, "a quad publishes in two or one fences");
@@ -157,11 +234,11 @@ batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the units the plan kernel wrote (this launch's stream, before it), or the host's
     const int64_t n_units = n_units_dev ? (int64_t)*n_units_dev : n_units_host;
-    // CTA c's k-th unit: units come longest first, so the rounds alternate
-    // direction (c, 2G - 1 - c, 2G + c, ...) to even out the CTAs' totals;
-    // every role walks the same sequence
-    const int64_t G = gridDim.x, c_ = blockIdx.x;
-    auto unit_of = [G, c_](int64_t k) { return k * G + ((k & 1) ? G - 1 - c_ : c_); };
+    // Every role walks the same sequence of (unit, stages): one contiguous
+    // share of all units' stages, or whole units, longest first, in rounds of
+    // alternating direction.
+    if (pre && !shares(n_units)) pre = nullptr;
+    const Walk walk0 = walk_begin(n_units, pre);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < BSTAGES; i++) { mbar_init(&s.full[i], BNPROD / 32); mbar_init(&s.empty[i], 1); }
@@ -191,22 +268,26 @@ batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *
         uint32_t zeroed = 0;                  // bit q: my row of ring slot q holds zeros
         int it = 0;                           // stages produced by this CTA (ring position)
         bool ok = true;
-        for (int64_t k = 0, ui = unit_of(0); ui < n_units && ok; ui = unit_of(++k)) {
-            const BUnit u = decode_unit(dbs, units[ui]);
+        for (Walk wk = walk0; wk.ui < n_units && ok; walk_next(wk, pre)) {
+            const BUnit u = decode_unit(dbs, units[wk.ui]);
             if (u.empty) continue;
+            int64_t s0, s1;
+            walk_span(wk, pre, u.S, s0, s1);
             const bool store = !(is_a && u.diag);  // warp-uniform: a warp's rows are all A or all B
             // the row's database, item and stage count (a packed pair: rows
             // 0 .. 63 the first database's items, 64 .. 127 the second's)
             const DbDesc *const Dr = u.packed ? (r < PACK_MAX ? u.D : u.D2) : u.D;
             const int item = u.packed ? (r & (PACK_MAX - 1)) : (is_a ? u.ta : u.tb) * BT + r;
             const int mfr = u.packed ? (r < PACK_MAX ? u.mf : u.mf2) : u.mf;
-            const int64_t lenr = u.packed ? (r < PACK_MAX ? u.S1 : u.S2) : u.S;
+            const int64_t lenu = u.packed ? (r < PACK_MAX ? u.S1 : u.S2) : u.S;
             const uint32_t *col =
                 (store && Dr && item < mfr)
                     ? bm + Dr->bm_off + (int64_t)__ldg(perm_base + Dr->item_off + item) * Dr->nwp
                     : nullptr;
-            const int64_t len = u.S;
-            // stage k of the unit lives in stg[k % BD]; a quad of 4 stages is
+            const int64_t len = s1 - s0;             // this share's stages ...
+            const int64_t lenr = lenu - s0;          // ... of which my row has so many
+            if (col) col += s0 * 4;
+            // stage k of the share lives in stg[k % BD]; a quad of 4 stages is
             // refilled at a time, 4 lanes per row copying 64 contiguous bytes
             auto refill = [&](int64_t q0) {
 #pragma unroll
@@ -216,7 +297,7 @@ batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *
                     const uint32_t *c = reinterpret_cast<const uint32_t *>(
                         __shfl_sync(0xffffffffu, reinterpret_cast<uintptr_t>(col), rw));
                     const int64_t lr = __shfl_sync(0xffffffffu, lenr, rw);
-                    if (c && k < lr) cp_async16(smem_addr(&s.stg[k % BD][row0 + rw]), c + k * 4);
+                    if (c && k < lr && k < len) cp_async16(smem_addr(&s.stg[k % BD][row0 + rw]), c + k * 4);
                 }
                 cp_async_commit();
             };
@@ -291,9 +372,11 @@ batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *
         const int q = warp & 3;  // TMEM lane quarter this warp may read
         int j = 0;               // segments drained by this CTA
         bool ok = true;
-        for (int64_t k = 0, ui = unit_of(0); ui < n_units && ok; ui = unit_of(++k)) {
-            const BUnit u = decode_unit(dbs, units[ui]);
+        for (Walk wk = walk0; wk.ui < n_units && ok; walk_next(wk, pre)) {
+            const BUnit u = decode_unit(dbs, units[wk.ui]);
             if (u.empty) continue;
+            int64_t s0, s1;
+            walk_span(wk, pre, u.S, s0, s1);
             // my accumulator row: item a of database Da (a packed pair's rows
             // 64 .. 127 are the second database's, its columns 64 .. 127 too)
             const int lr = q * 32 + lane;
@@ -303,7 +386,8 @@ batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *
             const int mfa = second ? u.mf2 : u.mf;
             const int coff = u.packed ? (second ? -PACK_MAX : 0) : u.tb * BT;  // column c holds item c + coff
             int *const row = Da ? pair_cnt + Da->pair_off + (int64_t)a * mfa : nullptr;
-            for (int64_t st0 = 0; st0 < u.S; st0 += kd, j++) {
+            const bool add = pre && wk.split;
+            for (int64_t st0 = s0; st0 < s1; st0 += kd, j++) {
                 const int buf = j & 1;
                 // warp-uniform: tcgen05.ld below is a .sync.aligned warp instruction
                 ok = __all_sync(0xffffffffu, bwait(s, &s.acc_full[buf], (uint32_t)(j >> 1) & 1u));
@@ -328,7 +412,11 @@ batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *
                             const int b = x * 16 + c + coff;
                             if (a < b && b < mfa) {
                                 const int val = __float2int_rn(__uint_as_float(v[c])) >> 2;
-                                row[b] = st0 == 0 ? val : row[b] + val;
+                                if (add) {
+                                    if (val) atomicAdd(row + b, val);
+                                } else {
+                                    row[b] = st0 == 0 ? val : row[b] + val;
+                                }
                             }
                         }
                     }
@@ -341,12 +429,14 @@ batch_pairs_tc_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *
         // ---------------- MMA issuer ----------------
         bool ok = true;
         int it = 0, j = 0;
-        for (int64_t k = 0, ui = unit_of(0); ui < n_units && ok; ui = unit_of(++k)) {
-            const BUnit u = decode_unit(dbs, units[ui]);
+        for (Walk wk = walk0; wk.ui < n_units && ok; walk_next(wk, pre)) {
+            const BUnit u = decode_unit(dbs, units[wk.ui]);
             if (u.empty) continue;
+            int64_t s0, s1;
+            walk_span(wk, pre, u.S, s0, s1);
             const uint32_t idesc = idesc_f8(BT, u.N);
-            for (int64_t st0 = 0; st0 < u.S && ok; st0 += kd, j++) {
-                const int64_t len = min64(kd, u.S - st0);
+            for (int64_t st0 = s0; st0 < s1 && ok; st0 += kd, j++) {
+                const int64_t len = min64(kd, s1 - st0);
                 const int buf = j & 1;
                 // buffer buf's previous run has been drained
                 if (!(ok = bwait(s, &s.acc_empty[buf], ((uint32_t)(j >> 1) & 1u) ^ 1u))) break;
@@ -422,19 +512,21 @@ __device__ long long block_scan_excl(long long v, long long *s_warp, long long *
 // two have about as many transactions); a larger one gets its upper-triangle
 // tiles of 128 items; a database without pairs gets nothing.  Units are
 // written in work order; *n_units receives their count.  One CTA of 1024
-// threads; scratch holds 4 n ints and n long longs.
+// threads; pre gets the work before each unit (pre[*n_units]: all of it).
 __global__ void __launch_bounds__(1024)
 batch_pair_plan_kernel(const DbDesc *__restrict__ dbs, const int *__restrict__ ord, int n,
                        int *__restrict__ srank, long long *__restrict__ off, int *__restrict__ small_list,
-                       unsigned long long *__restrict__ units, long long *__restrict__ n_units) {
+                       unsigned long long *__restrict__ units, long long *__restrict__ pre,
+                       long long *__restrict__ off_st, long long *__restrict__ n_units) {
     __shared__ long long s_warp[32];
-    long long base_small = 0, base_units = 0;
+    long long base_small = 0, base_units = 0, base_st = 0;
     for (int c0 = 0; c0 < n; c0 += 1024) {
         const int i = c0 + (int)threadIdx.x;
         int small = 0;
-        long long tiles = 0;
+        long long tiles = 0, S = 0;
         if (i < n) {
             const DbDesc &D = dbs[ord[i]];
+            S = (D.nw + 3) / 4;
             const int mf = *(volatile const int32_t *)&D.mfreq;
             const bool live = mf >= 2 && D.maxlen != 1;
             small = live && mf <= PACK_MAX;
@@ -447,20 +539,26 @@ batch_pair_plan_kernel(const DbDesc *__restrict__ dbs, const int *__restrict__ o
         const long long sr = block_scan_excl(small, s_warp, &t_small) + base_small;
         const long long cnt = small ? ((sr & 1) == 0 ? 1 : 0) : tiles;  // a pair opens at even ranks
         const long long o = block_scan_excl(cnt, s_warp, &t_units) + base_units;
+        long long t_st;  // a packed pair takes its longer (first) database's stages
+        const long long os = block_scan_excl(cnt * (S + UNIT_COST), s_warp, &t_st) + base_st;
         if (i < n) {
             srank[i] = small ? (int)sr : -1;
             off[i] = o;
+            off_st[i] = os;
             if (small) small_list[sr] = ord[i];
         }
         base_small += t_small;
         base_units += t_units;
+        base_st += t_st;
     }
     __syncthreads();  // small_list is complete
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int d = ord[i], sr = srank[i];
         long long o = off[i];
+        const long long S = (dbs[d].nw + 3) / 4, os = off_st[i];
         if (sr >= 0) {
             if ((sr & 1) == 0) {
+                pre[o] = os;
                 const uint32_t d2 = sr + 1 < base_small ? (uint32_t)small_list[sr + 1] : PACK_NONE;
                 units[o] = PACK | ((unsigned long long)d << 32) | d2;
             }
@@ -468,13 +566,49 @@ batch_pair_plan_kernel(const DbDesc *__restrict__ dbs, const int *__restrict__ o
             const int mf = *(volatile const int32_t *)&dbs[d].mfreq;
             if (mf >= 2 && dbs[d].maxlen != 1) {
                 const int nt = (mf + BT - 1) / BT;
+                long long x = os;
                 for (int ta = 0; ta < nt; ta++)
-                    for (int tb = ta; tb < nt; tb++)
+                    for (int tb = ta; tb < nt; tb++) {
+                        pre[o] = x;
+                        x += S + UNIT_COST;
                         units[o++] = ((unsigned long long)d << 32) | ((unsigned long long)ta << 16) | (unsigned)tb;
+                    }
             }
         }
     }
-    if (threadIdx.x == 0) *n_units = base_units;
+    if (threadIdx.x == 0) {
+        *n_units = base_units;
+        pre[base_units] = base_st;
+    }
+}
+
+// The counts of the units that a share's end cuts, cleared before the parts
+// add to them: CTA c looks at the end of share c.
+__global__ void __launch_bounds__(256)
+batch_pair_clear_kernel(const DbDesc *__restrict__ dbs, const unsigned long long *__restrict__ units,
+                        const long long *__restrict__ n_units_dev, const long long *__restrict__ pre,
+                        int *__restrict__ pair_cnt) {
+    const int64_t n = *n_units_dev;
+    const int64_t W = n > 0 ? pre[n] : 0;
+    if (W == 0 || !shares(n)) return;
+    const int64_t G = walk_grid(W), w = ((int64_t)blockIdx.x + 1) * W / G;
+    if ((int64_t)blockIdx.x + 1 >= G) return;
+    int64_t lo = 0, hi = n;  // pre[lo] <= w < pre[hi]
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (pre[mid] <= w) lo = mid; else hi = mid;
+    }
+    if (w - pre[lo] <= UNIT_COST) return;  // the end falls between two units
+    const BUnit u = decode_unit(dbs, units[lo]);
+    if (u.empty) return;
+    for (int part = 0; part < (u.D2 ? 2 : 1); part++) {
+        const DbDesc *D = part ? u.D2 : u.D;
+        const int mf = part ? u.mf2 : u.mf;
+        const int a0 = u.ta * BT, a1 = min(mf, a0 + BT), b0 = u.tb * BT, nb = min(mf, b0 + BT) - b0;
+        int *cnt = pair_cnt + D->pair_off;
+        for (int e = threadIdx.x; e < (a1 - a0) * nb; e += blockDim.x)
+            cnt[(int64_t)(a0 + e / nb) * mf + b0 + e % nb] = 0;
+    }
 }
 
 }  // namespace
@@ -518,7 +652,7 @@ namespace {
 
 template <int STG, int DEPTH, int MINB, int BG>
 int launch_shape(fim_ctx *ctx, const DbDesc *d_dbs, const unsigned long long *d_units, int64_t n_units,
-                 const long long *d_n_units, cudaStream_t st) {
+                 const long long *d_n_units, const long long *d_pre, cudaStream_t st) {
     using Smem = BtcSmem<STG, DEPTH>;
     static_assert(sizeof(Smem) + 1024 <= 232448, "shared memory per CTA");
     // MINB CTAs share an SM: their tensor memory and shared memory must fit
@@ -527,7 +661,7 @@ int launch_shape(fim_ctx *ctx, const DbDesc *d_dbs, const unsigned long long *d_
     static_assert(MINB * (sizeof(Smem) + 2048) <= 233472, "CTAs per SM as planned");
     const int kd = ctx->pairs_kdrain > 0 ? ctx->pairs_kdrain : BKDRAIN_MAX;
     int64_t grid = ctx->pairs_split > 0 ? ctx->pairs_split : (int64_t)ctx->num_sms * MINB;
-    if (grid > n_units) grid = n_units;
+    if (!d_pre && grid > n_units) grid = n_units;
     // one CTA per SM when MINB is 1: more shared memory than half an SM
     // keeps a second CTA (and its tensor-memory allocation) off
     size_t smem = sizeof(Smem) + 1024;
@@ -535,8 +669,12 @@ int launch_shape(fim_ctx *ctx, const DbDesc *d_dbs, const unsigned long long *d_
     auto *kern = batch_pairs_tc_kernel<STG, DEPTH, MINB, BG>;
     FIM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int *err = &ctx->counters.as<MineCounters>()->err;  // zeroed at the start of every batch
+    if (d_pre) {
+        ctx->launches++;
+        batch_pair_clear_kernel<<<(unsigned)grid, 256, 0, st>>>(d_dbs, d_units, d_n_units, d_pre, ctx->pair_cnt.as<int>());
+    }
     ctx->launches++;
-    kern<<<(unsigned)grid, BTHREADS, smem, st>>>(d_dbs, d_units, n_units, d_n_units, ctx->bm.as<uint32_t>(),
+    kern<<<(unsigned)grid, BTHREADS, smem, st>>>(d_dbs, d_units, n_units, d_n_units, d_pre, ctx->bm.as<uint32_t>(),
                                                  ctx->perm.as<int32_t>(), ctx->pair_cnt.as<int>(), kd, err);
     FIM_CUDA_TRY(cudaGetLastError());
     return FIM_OK;
@@ -552,31 +690,32 @@ const int kBatchPairsShapes[][4] = {{8, 8, 1, 2}, {6, 8, 1, 2}, {8, 16, 1, 2}, {
 const int kBatchPairsShapeCount = (int)(sizeof(kBatchPairsShapes) / sizeof(kBatchPairsShapes[0]));
 
 int launch_batch_pairs_tc(fim_ctx *ctx, const DbDesc *d_dbs, const unsigned long long *d_units, int64_t n_units,
-                          const long long *d_n_units, cudaStream_t st) {
+                          const long long *d_n_units, const long long *d_pre, cudaStream_t st) {
     if (n_units <= 0) return FIM_OK;
     switch (ctx->batch_pairs_shape) {
-        case 1: return launch_shape<6, 8, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, st);
-        case 2: return launch_shape<8, 16, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, st);
-        case 3: return launch_shape<4, 8, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, st);
-        case 4: return launch_shape<7, 12, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, st);
-        case 5: return launch_shape<8, 8, 1, 4>(ctx, d_dbs, d_units, n_units, d_n_units, st);
-        case 6: return launch_shape<8, 16, 1, 4>(ctx, d_dbs, d_units, n_units, d_n_units, st);
-        default: return launch_shape<8, 8, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, st);
+        case 1: return launch_shape<6, 8, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, d_pre, st);
+        case 2: return launch_shape<8, 16, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, d_pre, st);
+        case 3: return launch_shape<4, 8, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, d_pre, st);
+        case 4: return launch_shape<7, 12, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, d_pre, st);
+        case 5: return launch_shape<8, 8, 1, 4>(ctx, d_dbs, d_units, n_units, d_n_units, d_pre, st);
+        case 6: return launch_shape<8, 16, 1, 4>(ctx, d_dbs, d_units, n_units, d_n_units, d_pre, st);
+        default: return launch_shape<8, 8, 1, 2>(ctx, d_dbs, d_units, n_units, d_n_units, d_pre, st);
     }
 }
 
 int launch_batch_pair_plan(fim_ctx *ctx, const DbDesc *d_dbs, const int *d_ord, int n, unsigned long long *d_units,
-                           long long *d_n_units, void *scratch, cudaStream_t st) {
+                           long long *d_pre, long long *d_n_units, void *scratch, cudaStream_t st) {
     if (n <= 0) return FIM_OK;
     int *const srank = static_cast<int *>(scratch);
     int *const small_list = srank + n;
     long long *const off = reinterpret_cast<long long *>(small_list + n);  // 8n bytes in: aligned
     ctx->launches++;
-    batch_pair_plan_kernel<<<1, 1024, 0, st>>>(d_dbs, d_ord, n, srank, off, small_list, d_units, d_n_units);
+    batch_pair_plan_kernel<<<1, 1024, 0, st>>>(d_dbs, d_ord, n, srank, off, small_list, d_units, d_pre, off + n,
+                                               d_n_units);
     FIM_CUDA_TRY(cudaGetLastError());
     return FIM_OK;
 }
 
 size_t batch_pair_plan_scratch(int n) {
-    return sizeof(int) * 2 * (size_t)n + sizeof(long long) * (size_t)n;
+    return sizeof(int) * 2 * (size_t)n + 2 * sizeof(long long) * (size_t)n;
 }

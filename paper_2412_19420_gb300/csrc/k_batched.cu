@@ -1134,8 +1134,11 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
     // by the network's predicted work (FIM_LEARNED with learned_order) or as
     // root_sort says
     const int plan_mode = ((flags & FIM_LEARNED) && ctx->learned_order) ? 2 : ctx->root_sort;
+    // (the plan's stage prefix, a group's units and one more, follows the units)
+    const size_t unit_cap = (pair_units.size() ? pair_units.size() : 1);
     if (pairs_tc)
-        FIM_TRY(fim_reserve(ctx, ctx->batch_units, sizeof(unsigned long long) * (pair_units.size() ? pair_units.size() : 1)));
+        FIM_TRY(fim_reserve(ctx, ctx->batch_units,
+                            sizeof(unsigned long long) * (pack ? 2 * unit_cap + (size_t)n_seg : unit_cap)));
     // plan buffer: 32 unit counts, the database order, the plan's scratch
     const size_t plan_ord_off = 32 * sizeof(long long);
     const size_t plan_scr_off = plan_ord_off + ((sizeof(int) * (size_t)n_db + 255) & ~(size_t)255);
@@ -1359,13 +1362,14 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
             auto pair_pass = [&](int sg, cudaStream_t s_) -> int {
                 unsigned long long *const u = ctx->batch_units.as<unsigned long long>() + seg_unit[sg];
                 const int64_t cap = seg_unit[sg + 1] - seg_unit[sg];
-                if (!pack) return launch_batch_pairs_tc(ctx, d_dbs, u, cap, nullptr, s_);
+                if (!pack) return launch_batch_pairs_tc(ctx, d_dbs, u, cap, nullptr, nullptr, s_);
+                long long *const pre = ctx->batch_units.as<long long>() + unit_cap + seg_unit[sg] + sg;
                 char *const plan = static_cast<char *>(ctx->batch_plan.p);
                 long long *const cnt = reinterpret_cast<long long *>(plan) + sg;
                 const int *const ord = reinterpret_cast<const int *>(plan + plan_ord_off) + seg_db[sg];
-                const int rc = launch_batch_pair_plan(ctx, d_dbs, ord, seg_db[sg + 1] - seg_db[sg], u, cnt,
+                const int rc = launch_batch_pair_plan(ctx, d_dbs, ord, seg_db[sg + 1] - seg_db[sg], u, pre, cnt,
                                                       plan + plan_scr_off, s_);
-                return rc != FIM_OK ? rc : launch_batch_pairs_tc(ctx, d_dbs, u, cap, cnt, s_);
+                return rc != FIM_OK ? rc : launch_batch_pairs_tc(ctx, d_dbs, u, cap, cnt, pre, s_);
             };
             if (n_seg > 1) {
                 // group s: build + rank on the ctx stream, then its pair pass
@@ -1460,7 +1464,7 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
             if (ie != cudaSuccess) { fim_set_cuda_error(ie, "instantiate", __FILE__, __LINE__); return FIM_E_CUDA; }
             ctx->batch_graph_exec = ex;
             ctx->batch_graph_blob.swap(key);
-            ctx->batch_graph_launches = 10;  // unit map, build, rank, pairs, finalize, 3 root plan, DFS, epoch
+            ctx->batch_graph_launches = 12;  // unit map, build, rank, plan, clear, pairs, finalize, 3 root plan, DFS, epoch
         }
         FIM_CUDA_TRY(cudaGraphLaunch((cudaGraphExec_t)ctx->batch_graph_exec, st));
         ctx->launches += ctx->batch_graph_launches;
