@@ -25,139 +25,242 @@ constexpr int CACHE = 256;  // per sample: z1[64] z2[64] dz1[64] dz2[64]
 
 __device__ __forceinline__ float rb(float x, int bf) { return bf ? __bfloat162float(__float2bfloat16_rn(x)) : x; }
 
-__device__ void load_weights(float *w, const float *params, int bf) {
-    for (int i = threadIdx.x; i < P; i += blockDim.x) w[i] = rb(params[i], bf);
-    __syncthreads();
+// The forward and backward passes take MS samples a CTA: lane = sample, warp
+// = eight of a layer's 64 units, so a weight is read once per warp (a
+// broadcast) and 4,096 samples fill 128 CTAs of eight warps.  (One thread per
+// sample, with its 64 activations in local memory, left 32 CTAs of four warps
+// on long dependent chains: 66 us forward and 85 us backward at 4,096 samples
+// against 10 and 8.)  Every sum runs in the order it always did -- a unit's
+// inputs ascending, a chunk's samples ascending, chunks ascending -- so the
+// results are the same to the bit.
+constexpr int MS = 32, MT = 256;
+constexpr int W2P = 68;  // pitch of the transposed W2: 16-byte rows, few store conflicts
+
+// Eight consecutive floats of the caller's cache: two 16-byte accesses where
+// its rows are 16-byte aligned (a cache that starts on such a boundary).
+__device__ __forceinline__ bool cache_vec(const float *cache) { return (reinterpret_cast<uintptr_t>(cache) & 15) == 0; }
+__device__ __forceinline__ void put8(float *p, const float *v, bool vec) {
+    if (vec) {
+        reinterpret_cast<float4 *>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<float4 *>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 8; q++) p[q] = v[q];
+    }
+}
+__device__ __forceinline__ void get8(const float *p, float *v, bool vec) {
+    if (vec) {
+        const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 8; q++) v[q] = p[q];
+    }
 }
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(MT)
 mlp_forward_kernel(const float *__restrict__ params, const float *__restrict__ x, int64_t B,
                    float *__restrict__ y, float *__restrict__ cache, int bf) {
-    __shared__ float w[P];
-    load_weights(w, params, bf);
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    float xi[8], h1[64];
+    __shared__ __align__(16) float w1[64 * 8], w2t[64 * W2P];
+    __shared__ float b1[64], b2[64], w3[2 * 64], b3[2], h[2][64][MS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i0 = warp * 8;
+    const int64_t b = (int64_t)blockIdx.x * MS + lane;
+    float xi[8];
 #pragma unroll
-    for (int k = 0; k < 8; k++) xi[k] = rb(x[b * 8 + k], bf);
-    for (int i = 0; i < 64; i++) {
-        float a = w[OFF_B1 + i];
-#pragma unroll
-        for (int k = 0; k < 8; k++) a = fmaf(w[i * 8 + k], xi[k], a);
-        if (cache) cache[b * CACHE + i] = a;
-        h1[i] = rb(fmaxf(a, 0.f), bf);
+    for (int k = 0; k < 8; k++) xi[k] = b < B ? rb(x[b * 8 + k], bf) : 0.f;
+    for (int i = threadIdx.x; i < 64 * 8; i += MT) w1[i] = rb(params[i], bf);
+    for (int i = threadIdx.x; i < 64 * 64; i += MT) w2t[(i % 64) * W2P + i / 64] = rb(params[OFF_W2 + i], bf);
+    if (threadIdx.x < 64) {
+        b1[threadIdx.x] = rb(params[OFF_B1 + threadIdx.x], bf);
+        b2[threadIdx.x] = rb(params[OFF_B2 + threadIdx.x], bf);
+    } else if (threadIdx.x < 192) {
+        w3[threadIdx.x - 64] = rb(params[OFF_W3 + threadIdx.x - 64], bf);
+    } else if (threadIdx.x < 194) {
+        b3[threadIdx.x - 192] = rb(params[OFF_B3 + threadIdx.x - 192], bf);
     }
-    float y0 = w[OFF_B3], y1 = w[OFF_B3 + 1];
-    for (int i = 0; i < 64; i++) {
-        float a = w[OFF_B2 + i];
+    __syncthreads();
+    auto put = [&](const float *z, int layer) {  // pre-activations to the cache, activations to shared memory
+        if (cache && b < B) put8(cache + b * CACHE + 64 * layer + i0, z, cache_vec(cache));
+#pragma unroll
+        for (int q = 0; q < 8; q++) h[layer][i0 + q][lane] = rb(fmaxf(z[q], 0.f), bf);
+    };
+    float a[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        a[q] = b1[i0 + q];
+#pragma unroll
+        for (int k = 0; k < 8; k++) a[q] = fmaf(w1[(i0 + q) * 8 + k], xi[k], a[q]);
+    }
+    put(a, 0);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; q++) a[q] = b2[i0 + q];
+#pragma unroll 8
+    for (int k = 0; k < 64; k++) {
+        const float hk = h[0][k][lane];
+        const float4 wa = *reinterpret_cast<const float4 *>(w2t + k * W2P + i0);
+        const float4 wb = *reinterpret_cast<const float4 *>(w2t + k * W2P + i0 + 4);
+        a[0] = fmaf(wa.x, hk, a[0]);
+        a[1] = fmaf(wa.y, hk, a[1]);
+        a[2] = fmaf(wa.z, hk, a[2]);
+        a[3] = fmaf(wa.w, hk, a[3]);
+        a[4] = fmaf(wb.x, hk, a[4]);
+        a[5] = fmaf(wb.y, hk, a[5]);
+        a[6] = fmaf(wb.z, hk, a[6]);
+        a[7] = fmaf(wb.w, hk, a[7]);
+    }
+    put(a, 1);
+    __syncthreads();
+    if (warp < 2 && b < B) {  // output `warp` of sample b
+        float o = b3[warp];
 #pragma unroll 16
-        for (int k = 0; k < 64; k++) a = fmaf(w[OFF_W2 + i * 64 + k], h1[k], a);
-        if (cache) cache[b * CACHE + 64 + i] = a;
-        const float h2 = rb(fmaxf(a, 0.f), bf);
-        y0 = fmaf(w[OFF_W3 + i], h2, y0);
-        y1 = fmaf(w[OFF_W3 + 64 + i], h2, y1);
+        for (int i = 0; i < 64; i++) o = fmaf(w3[warp * 64 + i], h[1][i][lane], o);
+        y[b * 2 + warp] = o;
     }
-    y[b * 2 + 0] = y0;
-    y[b * 2 + 1] = y1;
 }
 
-// Per sample: dz2 = (W3^T dy) * [z2 > 0], dz1 = (W2^T dz2) * [z1 > 0]; loss.
-__global__ void __launch_bounds__(128)
+// Per sample: dz2 = (W3^T dy) * [z2 > 0], dz1 = (W2^T dz2) * [z1 > 0]; loss
+// (one part per 32 samples).
+__global__ void __launch_bounds__(MT)
 mlp_backward_sample_kernel(const float *__restrict__ params, const float *__restrict__ y,
                            const float *__restrict__ t, float *__restrict__ cache, int64_t B,
                            float *__restrict__ loss_parts, int bf) {
-    __shared__ float w[P];
-    __shared__ float red[4];
-    load_weights(w, params, bf);
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.f;
+    __shared__ __align__(16) float w2[64 * 64];
+    __shared__ float w3[2 * 64], d2[64][MS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i0 = warp * 8;
+    const int64_t b = (int64_t)blockIdx.x * MS + lane;
+    float *const c = cache + (b < B ? b : B - 1) * CACHE + i0;
+    const bool vec = cache_vec(cache);
+    float z1[8], z2[8];
+    get8(c, z1, vec);
+    get8(c + 64, z2, vec);
+    float y0 = 0.f, y1 = 0.f, t0 = 0.f, t1 = 0.f;
     if (b < B) {
-        const float y0 = y[b * 2], y1 = y[b * 2 + 1], t0 = t[b * 2], t1 = t[b * 2 + 1];
-        const float e = y0 - t0;
-        l = 0.5f * e * e + fmaxf(y1, 0.f) + log1pf(expf(-fabsf(y1))) - t1 * y1;
-        const float dy0 = e / (float)B, dy1 = (1.f / (1.f + expf(-y1)) - t1) / (float)B;
-        float *c = cache + b * CACHE;
-        float dz2[64];
-        for (int i = 0; i < 64; i++) {
-            const float g = w[OFF_W3 + i] * dy0 + w[OFF_W3 + 64 + i] * dy1;
-            dz2[i] = c[64 + i] > 0.f ? g : 0.f;
-            c[192 + i] = dz2[i];
-        }
-        for (int k = 0; k < 64; k++) {
-            float g = 0.f;
-#pragma unroll 16
-            for (int i = 0; i < 64; i++) g = fmaf(w[OFF_W2 + i * 64 + k], dz2[i], g);
-            c[128 + k] = c[k] > 0.f ? g : 0.f;
-        }
+        y0 = y[b * 2];
+        y1 = y[b * 2 + 1];
+        t0 = t[b * 2];
+        t1 = t[b * 2 + 1];
     }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
+    for (int i = threadIdx.x; i < 64 * 64; i += MT) w2[i] = rb(params[OFF_W2 + i], bf);
+    if (threadIdx.x < 128) w3[threadIdx.x] = rb(params[OFF_W3 + threadIdx.x], bf);
     __syncthreads();
-    if (threadIdx.x == 0) loss_parts[blockIdx.x] = red[0] + red[1] + red[2] + red[3];
+    const float e = y0 - t0;
+    const float dy0 = e / (float)B, dy1 = (1.f / (1.f + expf(-y1)) - t1) / (float)B;
+    float g[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        const float v = w3[i0 + q] * dy0 + w3[64 + i0 + q] * dy1;
+        g[q] = z2[q] > 0.f ? v : 0.f;
+        d2[i0 + q][lane] = g[q];
+    }
+    if (b < B) put8(c + 192, g, vec);
+    __syncthreads();
+    float a[8] = {};
+#pragma unroll 8
+    for (int i = 0; i < 64; i++) {
+        const float d = d2[i][lane];
+        const float4 wa = *reinterpret_cast<const float4 *>(w2 + i * 64 + i0);
+        const float4 wb = *reinterpret_cast<const float4 *>(w2 + i * 64 + i0 + 4);
+        a[0] = fmaf(wa.x, d, a[0]);
+        a[1] = fmaf(wa.y, d, a[1]);
+        a[2] = fmaf(wa.z, d, a[2]);
+        a[3] = fmaf(wa.w, d, a[3]);
+        a[4] = fmaf(wb.x, d, a[4]);
+        a[5] = fmaf(wb.y, d, a[5]);
+        a[6] = fmaf(wb.z, d, a[6]);
+        a[7] = fmaf(wb.w, d, a[7]);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; q++) a[q] = z1[q] > 0.f ? a[q] : 0.f;
+    if (b < B) put8(c + 128, a, vec);
+    if (warp == 0) {
+        float l = 0.f;
+        if (b < B) l = 0.5f * e * e + fmaxf(y1, 0.f) + log1pf(expf(-fabsf(y1))) - t1 * y1;
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) loss_parts[blockIdx.x] = l;
+    }
 }
 
-// Partial weight gradients over a chunk of samples: thread j owns parameters
-// j, j + 256, ...; every parameter's gradient is a sum over the batch of a
-// product of a cached backward term and a forward activation.
-constexpr int GCHUNK = 256;
+// Partial weight gradients over a chunk of samples: every parameter's gradient
+// is a sum over the batch of a product of a cached backward term and a forward
+// activation, one thread per parameter (two for W2).  A CTA takes one chunk
+// and one group of parameters: eight rows of W2, or W1 and b1, or b2, W3 and
+// b3 -- ten groups, so that 16 chunks fill the SMs (all parameters of a chunk
+// in one CTA: 75 us at 4,096 samples against 15).
+constexpr int GCHUNK = 256, GGROUPS = 10;
 __global__ void __launch_bounds__(256)
 mlp_grad_partial_kernel(const float *__restrict__ x, const float *__restrict__ y, const float *__restrict__ t,
                         const float *__restrict__ cache, int64_t B, float *__restrict__ part, int bf) {
-    __shared__ float sx[32][8], sz1[32][64], sz2[32][64], sd1[32][64], sd2[32][64], sdy[32][2];
-    float acc[(P + 255) / 256];
-#pragma unroll
-    for (int q = 0; q < (P + 255) / 256; q++) acc[q] = 0.f;
+    // 64 samples at a time: a forward activation row and the backward terms
+    __shared__ float act[64][64], dz[64][64], sdy[64][2];
+    const int grp = blockIdx.y, tid = threadIdx.x;
     const int64_t b0 = (int64_t)blockIdx.x * GCHUNK;
     const int64_t b1 = min64(B, b0 + GCHUNK);
-    for (int64_t s0 = b0; s0 < b1; s0 += 32) {
-        const int ns = (int)min64(32, b1 - s0);
+    float *const out = part + (int64_t)blockIdx.x * P;
+    float acc[3] = {};
+    for (int64_t s0 = b0; s0 < b1; s0 += 64) {
+        const int ns = (int)min64(64, b1 - s0);
         __syncthreads();
-        for (int i = threadIdx.x; i < ns * 64; i += 256) {
-            const int r = i / 64, c = i % 64;
-            const float *cc = cache + (s0 + r) * CACHE;
-            sz1[r][c] = rb(fmaxf(cc[c], 0.f), bf);      // h1
-            sz2[r][c] = rb(fmaxf(cc[64 + c], 0.f), bf); // h2
-            sd1[r][c] = cc[128 + c];
-            sd2[r][c] = cc[192 + c];
-        }
-        for (int i = threadIdx.x; i < ns * 8; i += 256) sx[i / 8][i % 8] = rb(x[(s0 + i / 8) * 8 + i % 8], bf);
-        if (threadIdx.x < ns) {
-            const int64_t bb = s0 + threadIdx.x;
-            sdy[threadIdx.x][0] = (y[bb * 2] - t[bb * 2]) / (float)B;
-            sdy[threadIdx.x][1] = (1.f / (1.f + expf(-y[bb * 2 + 1])) - t[bb * 2 + 1]) / (float)B;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < (P + 255) / 256; q++) {
-            const int j = threadIdx.x + q * 256;
-            if (j >= P) break;
-            float a = acc[q];
-            if (j < OFF_B1) {                 // W1[i][k] += dz1[i] x[k]
-                const int i = j / 8, k = j % 8;
-                for (int r = 0; r < ns; r++) a = fmaf(sd1[r][i], sx[r][k], a);
-            } else if (j < OFF_W2) {          // b1[i] += dz1[i]
-                const int i = j - OFF_B1;
-                for (int r = 0; r < ns; r++) a += sd1[r][i];
-            } else if (j < OFF_B2) {          // W2[i][k] += dz2[i] h1[k]
-                const int i = (j - OFF_W2) / 64, k = (j - OFF_W2) % 64;
-                for (int r = 0; r < ns; r++) a = fmaf(sd2[r][i], sz1[r][k], a);
-            } else if (j < OFF_W3) {          // b2[i] += dz2[i]
-                const int i = j - OFF_B2;
-                for (int r = 0; r < ns; r++) a += sd2[r][i];
-            } else if (j < OFF_B3) {          // W3[o][k] += dy[o] h2[k]
-                const int o = (j - OFF_W3) / 64, k = (j - OFF_W3) % 64;
-                for (int r = 0; r < ns; r++) a = fmaf(sdy[r][o], sz2[r][k], a);
-            } else {                          // b3[o] += dy[o]
-                const int o = j - OFF_B3;
-                for (int r = 0; r < ns; r++) a += sdy[r][o];
+        if (grp < 8) {  // dz2 of rows 8 grp .., h1
+            for (int i = tid; i < ns * 64; i += 256) act[i / 64][i % 64] = rb(fmaxf(cache[(s0 + i / 64) * CACHE + i % 64], 0.f), bf);
+            for (int i = tid; i < ns * 8; i += 256) dz[i / 8][i % 8] = cache[(s0 + i / 8) * CACHE + 192 + grp * 8 + i % 8];
+        } else if (grp == 8) {  // dz1, x
+            for (int i = tid; i < ns * 64; i += 256) dz[i / 64][i % 64] = cache[(s0 + i / 64) * CACHE + 128 + i % 64];
+            for (int i = tid; i < ns * 8; i += 256) act[i / 8][i % 8] = rb(x[(s0 + i / 8) * 8 + i % 8], bf);
+        } else {  // dz2, h2 (and dy below)
+            for (int i = tid; i < ns * 64; i += 256) {
+                act[i / 64][i % 64] = rb(fmaxf(cache[(s0 + i / 64) * CACHE + 64 + i % 64], 0.f), bf);
+                dz[i / 64][i % 64] = cache[(s0 + i / 64) * CACHE + 192 + i % 64];
             }
-            acc[q] = a;
+        }
+        if (grp == 9 && tid < ns) {
+            const int64_t bb = s0 + tid;
+            sdy[tid][0] = (y[bb * 2] - t[bb * 2]) / (float)B;
+            sdy[tid][1] = (1.f / (1.f + expf(-y[bb * 2 + 1])) - t[bb * 2 + 1]) / (float)B;
+        }
+        __syncthreads();
+        if (grp < 8) {  // W2[i][k] += dz2[i] h1[k], i = 8 grp + tid / 32, k = tid % 32 and + 32
+            const int i = tid >> 5, k = tid & 31;
+#pragma unroll 8
+            for (int r = 0; r < ns; r++) {
+                const float d = dz[r][i];
+                acc[0] = fmaf(d, act[r][k], acc[0]);
+                acc[1] = fmaf(d, act[r][k + 32], acc[1]);
+            }
+        } else if (grp == 8) {  // W1[i][k] += dz1[i] x[k] (two a thread); b1[i] += dz1[i]
+            const int i = tid >> 3, k = tid & 7;
+#pragma unroll 8
+            for (int r = 0; r < ns; r++) {
+                const float xk = act[r][k];
+                acc[0] = fmaf(dz[r][i], xk, acc[0]);
+                acc[1] = fmaf(dz[r][i + 32], xk, acc[1]);
+            }
+            if (tid < 64)
+#pragma unroll 8
+                for (int r = 0; r < ns; r++) acc[2] += dz[r][tid];
+        } else if (tid < 64) {  // b2[i] += dz2[i]
+            for (int r = 0; r < ns; r++) acc[0] += dz[r][tid];
+        } else if (tid < 192) {  // W3[o][k] += dy[o] h2[k]
+            const int o = (tid - 64) >> 6, k = tid & 63;
+#pragma unroll 8
+            for (int r = 0; r < ns; r++) acc[0] = fmaf(sdy[r][o], act[r][k], acc[0]);
+        } else if (tid < 194) {  // b3[o] += dy[o]
+            for (int r = 0; r < ns; r++) acc[0] += sdy[r][tid - 192];
         }
     }
-#pragma unroll
-    for (int q = 0; q < (P + 255) / 256; q++) {
-        const int j = threadIdx.x + q * 256;
-        if (j < P) part[(int64_t)blockIdx.x * P + j] = acc[q];
+    if (grp < 8) {
+        const int i = grp * 8 + (tid >> 5), k = tid & 31;
+        out[OFF_W2 + i * 64 + k] = acc[0];
+        out[OFF_W2 + i * 64 + k + 32] = acc[1];
+    } else if (grp == 8) {
+        const int i = tid >> 3, k = tid & 7;
+        out[i * 8 + k] = acc[0];
+        out[(i + 32) * 8 + k] = acc[1];
+        if (tid < 64) out[OFF_B1 + tid] = acc[2];
+    } else if (tid < 64) {
+        out[OFF_B2 + tid] = acc[0];
+    } else if (tid < 194) {
+        out[OFF_W3 + tid - 64] = acc[0];  // W3 and, after its 128, b3
     }
 }
 
@@ -167,12 +270,18 @@ __global__ void mlp_grad_sum_kernel(const float *__restrict__ part, int nchunks,
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < P) {
         float a = 0.f;
+#pragma unroll 8
         for (int c = 0; c < nchunks; c++) a += part[(int64_t)c * P + j];
         grad[j] = a;
     }
-    if (j == P) {
+    if (j == P) {  // four parts (128 samples) at a time
         float a = 0.f;
-        for (int c = 0; c < nloss; c++) a += loss_parts[c];
+        for (int c = 0; c < nloss; c += 4) {
+            float p[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) p[q] = c + q < nloss ? loss_parts[c + q] : 0.f;
+            a += p[0] + p[1] + p[2] + p[3];
+        }
         *loss = a;
     }
 }
@@ -423,7 +532,7 @@ int fim_mlp_forward(fim_ctx *ctx, const float *params, const float *x, int64_t B
     if (!ctx || !params || !x || !y || B < 0) return FIM_E_INVAL;
     if (B == 0) return FIM_OK;
     ctx->launches++;
-    mlp_forward_kernel<<<(unsigned)ceil_div64(B, 128), 128, 0, ctx->stream>>>(params, x, B, y, cache, bf16 ? 1 : 0);
+    mlp_forward_kernel<<<(unsigned)ceil_div64(B, MS), MT, 0, ctx->stream>>>(params, x, B, y, cache, bf16 ? 1 : 0);
     FIM_CUDA_TRY(cudaGetLastError());
     return FIM_OK;
 }
@@ -432,7 +541,7 @@ int fim_mlp_backward(fim_ctx *ctx, const float *params, const float *x, const fl
                      const float *cache, int64_t B, float *grad, float *loss_out, int bf16) {
     FIM_NVTX("fim_mlp_backward");
     if (!ctx || !params || !x || !y || !t || !cache || !grad || B <= 0) return FIM_E_INVAL;
-    const int nb = (int)ceil_div64(B, 128);
+    const int nb = (int)ceil_div64(B, MS);
     const int nchunks = (int)ceil_div64(B, GCHUNK);
     FIM_TRY(fim_reserve(ctx, ctx->mlp_scratch, sizeof(float) * ((size_t)nchunks * P + nb + 1)));
     float *part = ctx->mlp_scratch.as<float>();
@@ -440,8 +549,8 @@ int fim_mlp_backward(fim_ctx *ctx, const float *params, const float *x, const fl
     float *loss = loss_parts + nb;
     const int bf = bf16 ? 1 : 0;
     ctx->launches += 3;
-    mlp_backward_sample_kernel<<<nb, 128, 0, ctx->stream>>>(params, y, t, const_cast<float *>(cache), B, loss_parts, bf);
-    mlp_grad_partial_kernel<<<nchunks, 256, 0, ctx->stream>>>(x, y, t, cache, B, part, bf);
+    mlp_backward_sample_kernel<<<nb, MT, 0, ctx->stream>>>(params, y, t, const_cast<float *>(cache), B, loss_parts, bf);
+    mlp_grad_partial_kernel<<<dim3((unsigned)nchunks, GGROUPS), 256, 0, ctx->stream>>>(x, y, t, cache, B, part, bf);
     mlp_grad_sum_kernel<<<(P + 1 + 255) / 256, 256, 0, ctx->stream>>>(part, nchunks, grad, loss_parts, nb, loss);
     FIM_CUDA_TRY(cudaGetLastError());
     if (loss_out) {
