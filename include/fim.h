@@ -84,7 +84,8 @@ typedef struct {
     uint64_t supports_singletons; /* S(I_k) computed: n_items                      */
     uint64_t supports_pairs;      /* S(I_a n I_b) computed: m'(m'-1)/2 (Eq. 2)     */
     uint64_t supports_dfs;        /* supports of >= 3-itemsets computed by the DFS  */
-    uint64_t dfs_words;           /* 32-bit candidate words ANDed by the DFS        */
+    uint64_t dfs_words;           /* 32-bit candidate words ANDed by the DFS (of
+                                     projected columns where it runs on those)      */
     uint64_t dfs_bytes;           /* bytes the DFS kernel read/wrote algorithmically */
     uint64_t dfs_touched_bytes;   /* the same, counting only 32-byte sectors that can
                                      contribute (zero prefix words are skipped)     */
@@ -96,7 +97,7 @@ typedef struct {
     uint64_t launches_mine;       /* kernels launched by the last fim_mine          */
     uint64_t dfs_busy_ns;         /* DFS workers' time inside tasks, summed         */
     uint64_t dfs_span_ns;         /* first worker start to last worker exit         */
-    uint64_t dfs_workers;         /* DFS workers (CTAs) of the launch               */
+    uint64_t dfs_workers;         /* DFS workers (warps or CTAs) of the launch      */
     uint64_t dfs_root_ns;         /* part of dfs_busy_ns spent in the root classes'
                                      own passes (candidate list + level-0 pass)     */
     float ms_build, ms_singletons, ms_pairs, ms_dfs, ms_compact; /* CUDA-event times */

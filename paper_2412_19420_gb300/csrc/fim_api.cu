@@ -350,11 +350,12 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     cudaEventRecord(ctx->ev[1], st);
     const bool do_pairs = mf >= 2 && (maxlen == 0 || maxlen >= 2);
     const bool do_dfs = do_pairs && mf >= 3 && (maxlen == 0 || maxlen >= 3);
-    // The plain search runs on warp workers (k_proj.cu); the network, diffset,
-    // trace and no-split options, and searches too deep for a warp worker's
-    // stack, on the CTA workers, which look at whole columns.
-    const bool warp_dfs = do_dfs && !ms.cta_dfs &&
-                          !(flags & (FIM_LEARNED | FIM_DIFFSET_RULE | FIM_TRACE | FIM_NO_SPLIT));
+    // The search runs on warp workers (k_proj.cu); the trace and no-split
+    // options, and searches too deep for a warp worker's stack, on the CTA
+    // workers, which look at whole columns.
+    const bool rep = (flags & (FIM_LEARNED | FIM_DIFFSET_RULE)) != 0;  // classes choose their representation
+    const bool net_order = (flags & FIM_LEARNED) && ctx->learned_order;  // the network orders the pair roots
+    const bool warp_dfs = do_dfs && !ms.cta_dfs && !(flags & (FIM_TRACE | FIM_NO_SPLIT));
     // Small matrices of short rows: few triples, which the bit columns
     // themselves count sooner than three more launches would (5,746 x 99: 228
     // against 247 us a mine); rows that hold a third of the frequent items make
@@ -376,7 +377,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     proj.tiles = (unsigned long long)mf * ((proj.wmax + 31) / 32);
     proj.triples = (unsigned long long)mf * mf * mf;
     proj.units = (unsigned long long)mf * proj_triple_units(mf);
-    const bool small_plan = warp_dfs && ctx->n_shards == 1 && proj_small_plan_fits(mf) && proj.wmax <= kProjWmax &&
+    const bool small_plan = warp_dfs && ctx->n_shards == 1 && !net_order && proj_small_plan_fits(mf) && proj.wmax <= kProjWmax &&
                             proj.words <= kSmallPlanWords && proj.rows <= kSmallPlanWords;
     // automatic: keep low-support classes sparse when the frequent item
     // columns do not fit in half of L2 (streaming whole columns from HBM
@@ -442,14 +443,14 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         const int levels_needed = bound > 2 ? bound - 1 : 1;
         ProjParams q{};
         if (on_warps) {
-            const bool triples = !direct && ctx->n_shards == 1 && proj.triples <= kTriples;
+            const bool triples = !direct && ctx->n_shards == 1 && !net_order && proj.triples <= kTriples;
             if (!direct) FIM_TRY(launch_projection(ctx, proj, small_plan, triples, thr));
             if (triples) {
                 q.triple = ctx->proj_triple.as<uint32_t>();
                 q.roots = ctx->proj_roots.as<unsigned long long>();
             } else if (!small_plan) {  // candidate-less pairs dropped, the others ordered
                 FIM_TRY(reserve_root_plan(ctx, npairs_all));
-                FIM_TRY(launch_root_plan(ctx, d_ctr, npairs_all, nullptr, ctx->root_sort, nullptr, st));
+                FIM_TRY(launch_root_plan(ctx, d_ctr, npairs_all, nullptr, net_order ? 2 : ctx->root_sort, nullptr, st));
             }
             q.items = ctx->proj_items.as<ProjItem>();
             q.mat = ctx->proj_mat.as<uint32_t>();
@@ -473,7 +474,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         }
         if (ms.frame_pool == 0) ms.frame_pool = 4LL * mf + 1024;
         FIM_TRY(fim_reserve(ctx, ctx->frame_items, sizeof(uint32_t) * (size_t)workers * ms.frame_pool));
-        if (!on_warps) FIM_TRY(fim_reserve(ctx, ctx->frame_sups, sizeof(uint32_t) * (size_t)workers * ms.frame_pool));
+        if (!on_warps || rep) FIM_TRY(fim_reserve(ctx, ctx->frame_sups, sizeof(uint32_t) * (size_t)workers * ms.frame_pool));
         FIM_TRY(prepare_task_queue(ctx, sizeof(Task) * kTaskCap));
         FIM_TRY(fim_reserve(ctx, ctx->cand_pool, sizeof(uint32_t) * kCandPoolCap));
         if (!small_plan) FIM_TRY(launch_epoch_bump(ctx));

@@ -25,14 +25,17 @@
 // sibling lists sit in its slice of shared memory and spill to global memory.
 // Every wait is bounded (FIM_E_TIMEOUT), and no worker waits for one that has
 // not started.  A search deeper than a worker's stack reports FIM_E_STACK and
-// is mined again by the CTA workers of k_dfs.cu, which also serve the options
-// that look at whole columns (network, diffsets, traces, no splitting).
+// is mined again by the CTA workers of k_dfs.cu, which also serve traces and
+// the no-split option.  With FIM_LEARNED or FIM_DIFFSET_RULE a worker asks the
+// network, or the size rule, for each class's representation (a build of the
+// kernel of its own: the choice costs registers).
 //
 // Prefix extension, ms (one GB300; CTA workers -> this file, projection and
 // triple pass included): 100,000 x 2,000 planted 47.3 -> 5.6 (14 bytes of
 // every column in 15 are gone, and 4.2 million sets come from 24 warps an SM
 // instead of 4 CTAs); 10^7 x 5,000 49 (twice, when its stack had to grow) ->
-// 4.6; 10^6 x 1,000 0.97 -> 0.37; 50,001 x 60 dense 0.73 -> 0.25.  What bounds
+// 4.6; 10^6 x 1,000 0.97 -> 0.37; 50,001 x 60 dense 0.73 -> 0.25; 20,000 x 800
+// planted with the network 4.1 -> 1.3.  What bounds
 // it now: each class's chain of dependent steps (26 cycles from one of a
 // worker's instructions to its next, 0.23 of the issue slots used, ncu), and
 // for the triple pass popc.
@@ -50,6 +53,7 @@ constexpr int PST = 832;         // stack words in shared memory per worker
 // over only the class at hand left most workers waiting (utilisation 0.19).
 constexpr int PGIVE = 8;
 
+template <bool REP>
 struct __align__(16) PWork {
     uint32_t stack[PST];         // stored prefixes, bottom up
     uint32_t frames[PFR];        // sibling lists, bottom up
@@ -59,8 +63,12 @@ struct __align__(16) PWork {
     int ftopS[PLV], ftopG[PLV];  // first free list entry above it, shared / global
     int stopS[PLV], stopG[PLV];  // first free stack word above it
     unsigned long long rec_next, rec_end, it_next, it_end;  // reserved output slots
-    unsigned long long n_sup, n_words, n_bytes, n_classes, emitted, emitted_items;
+    unsigned long long n_sup, n_words, n_bytes, n_classes, n_diff, emitted, emitted_items;
     int max_len;
+    // representation choice (network, diffset rule): supports of the list
+    // entries and of the levels' classes, the network's input and output
+    uint32_t fsup[REP ? PFR : 1], supY[REP ? PLV : 1];
+    float feat[REP ? FIM_MLP_FEATURES : 1], out[2];
 };
 
 __device__ __forceinline__ void perr(const DfsParams &p, int code) { atomicCAS(&p.ctr->err, 0, code); }
@@ -601,13 +609,21 @@ proj_triple_kernel(const ProjItem *__restrict__ items, int mf, const unsigned lo
 // Where a worker's lists and stored prefixes lie.
 struct Space {
     uint32_t *gfr, *gst;     // this worker's global list / stack
+    uint32_t *gfs;           // its list entries' supports (REP)
     int gfr_cap, gst_cap;
 };
 
-__device__ __forceinline__ uint32_t *frame_at(PWork &s, const Space &sp, int pos) {
+template <bool REP>
+__device__ __forceinline__ uint32_t *frame_at(PWork<REP> &s, const Space &sp, int pos) {
     return pos >= 0 ? s.frames + pos : sp.gfr + ~pos;
 }
-__device__ __forceinline__ uint32_t *stack_at(PWork &s, const Space &sp, int pos) {
+template <bool REP>
+__device__ __forceinline__ uint32_t *fsup_at(PWork<REP> &s, const Space &sp, int pos) {
+    if (!REP) return nullptr;
+    return pos >= 0 ? s.fsup + pos : sp.gfs + ~pos;
+}
+template <bool REP>
+__device__ __forceinline__ uint32_t *stack_at(PWork<REP> &s, const Space &sp, int pos) {
     return pos >= 0 ? s.stack + pos : sp.gst + ~pos;
 }
 // Room for `need` entries above (topS, topG): a position, or INT_MIN.
@@ -620,7 +636,8 @@ __device__ __forceinline__ int place(int need, int topS, int capS, int topG, int
 // emitted much reserves ahead (an eighth of what it has emitted, at most 64
 // sets), so that a returning global atomic is paid every few classes; slots
 // left over at its end are holes, which the compactor leaves out.
-__device__ __forceinline__ void take_slots(const DfsParams &p, PWork &s, unsigned tot, unsigned nitems,
+template <bool REP>
+__device__ __forceinline__ void take_slots(const DfsParams &p, PWork<REP> &s, unsigned tot, unsigned nitems,
                                            unsigned long long *rb, unsigned long long *ib) {
     if (s.rec_next + tot > s.rec_end) {
         for (unsigned long long r = s.rec_next; r < s.rec_end; r++)
@@ -652,11 +669,13 @@ __device__ __forceinline__ void take_slots(const DfsParams &p, PWork &s, unsigne
 // and emitted with the prefix s.path[0 .. plen).  2^lg lanes cover 128 words
 // of the prefix at a time, so short columns count 32 >> lg candidates side by
 // side; PG candidates per lane are loaded together.  Returns |F|.
-template <int PG>
-__device__ __forceinline__ int proj_class_pass(const DfsParams &p, PWork &s, uint32_t thr, const uint32_t *src0,
+// REP: diff counts through the diffset, S(X u e) - popc((src0 AND NOT src1) AND
+// col(e)), with the parent supports psup (which also receives the children's).
+template <int PG, bool REP>
+__device__ __forceinline__ int proj_class_pass(const DfsParams &p, PWork<REP> &s, uint32_t thr, const uint32_t *src0,
                                                const uint32_t *src1, const uint32_t *__restrict__ cols,
                                                int64_t stride, int W, int lg, const uint32_t *cand, int k, int plen,
-                                               uint32_t *store, uint32_t *fout) {
+                                               uint32_t *store, uint32_t *fout, uint32_t *psup, bool diff) {
     const int lane = threadIdx.x & 31;
     const int NS = 32 >> lg, sub = lane >> lg;
     const int wl = (lane & ((1 << lg) - 1)) * 4, step = 4 << lg;
@@ -664,6 +683,7 @@ __device__ __forceinline__ int proj_class_pass(const DfsParams &p, PWork &s, uin
     for (int g0 = 0; g0 < k; g0 += PG * NS) {
         const int gn = min(PG * NS, k - g0);
         const uint32_t my = lane < gn ? cand[g0 + lane] : 0u;
+        const uint32_t ps = REP && diff && lane < gn ? psup[g0 + lane] : 0u;
         const int nu = (gn + NS - 1) >> (5 - lg);
         uint32_t ci[PG], acc[PG];
 #pragma unroll
@@ -674,12 +694,14 @@ __device__ __forceinline__ int proj_class_pass(const DfsParams &p, PWork &s, uin
         for (int w0 = 0; w0 < W; w0 += step) {
             const int w = w0 + wl;
             if (w < W) {
-                const uint4 y = and4(*reinterpret_cast<const uint4 *>(src0 + w), *reinterpret_cast<const uint4 *>(src1 + w));
+                const uint4 a = *reinterpret_cast<const uint4 *>(src0 + w), b = *reinterpret_cast<const uint4 *>(src1 + w);
+                uint4 y = and4(a, b);
                 uint4 cv[PG];
 #pragma unroll
                 for (int u = 0; u < PG; u++)
                     if (u < nu) cv[u] = ldg_u4(cols + (int64_t)ci[u] * stride + w);
                 if (g0 == 0 && store && sub == 0) *reinterpret_cast<uint4 *>(store + w) = y;
+                if (REP && diff) y = make_uint4(a.x & ~b.x, a.y & ~b.y, a.z & ~b.z, a.w & ~b.w);
 #pragma unroll
                 for (int u = 0; u < PG; u++)
                     if (u < nu) acc[u] += popc_and4(y, cv[u]);
@@ -704,6 +726,7 @@ __device__ __forceinline__ int proj_class_pass(const DfsParams &p, PWork &s, uin
                     if (lane >> (5 - lg) == u) mine = t;
                 }
         }
+        if (REP && diff) mine = ps - mine;
         const bool f = lane < gn && mine >= thr;
         const uint32_t bal = __ballot_sync(0xffffffffu, f);
         const int tot = __popc(bal);
@@ -717,6 +740,7 @@ __device__ __forceinline__ int proj_class_pass(const DfsParams &p, PWork &s, uin
             if (f) {
                 const int pos = __popc(bal & ((1u << lane) - 1u));
                 fout[nF + pos] = my;
+                if (REP) psup[nF + pos] = mine;
                 if (fits) {
                     const unsigned long long r = rb + pos;
                     p.rec_off[r] = ib + (unsigned long long)pos * len;
@@ -737,20 +761,14 @@ __device__ __forceinline__ int proj_class_pass(const DfsParams &p, PWork &s, uin
         }
         __syncwarp();
     }
-    if (lane == 0) {
-        s.n_sup += (unsigned long long)k;
-        s.n_words += (unsigned long long)k * (unsigned long long)W;
-        s.n_bytes += 4ull * (unsigned long long)W * ((unsigned long long)k + 2ull + (store ? 1ull : 0ull));
-        s.n_classes += 1ull;
-        if (nF > 0 && plen + 1 > s.max_len) s.max_len = plen + 1;
-    }
     return nF;
 }
 
 // Child candidates of sibling j of a list of nF: the later siblings whose pair
 // with it is frequent, in order.  Returns their number; *cit = sibling j.
-__device__ __forceinline__ int siblings(const DfsParams &p, int mpw, const uint32_t *fr, int j, int nF, uint32_t *out,
-                                        uint32_t *cit) {
+template <bool REP>
+__device__ __forceinline__ int siblings(const DfsParams &p, int mpw, const uint32_t *fr, const uint32_t *fs, int j,
+                                        int nF, uint32_t *out, uint32_t *outs, uint32_t *cit) {
     const int lane = threadIdx.x & 31;
     const uint32_t c = fr[j];
     const uint32_t *rb = p.pairbits + (int64_t)(c & 0xFFFFu) * mpw;
@@ -761,7 +779,11 @@ __device__ __forceinline__ int siblings(const DfsParams &p, int mpw, const uint3
         const uint32_t id = d & 0xFFFFu;
         const bool f = l < nF && ((__ldg(rb + (id >> 5)) >> (id & 31)) & 1u);
         const uint32_t bal = __ballot_sync(0xffffffffu, f);
-        if (f) out[k + __popc(bal & ((1u << lane) - 1u))] = d;
+        if (f) {
+            const int at = k + __popc(bal & ((1u << lane) - 1u));
+            out[at] = d;
+            if (REP) outs[at] = fs[l];
+        }
         k += __popc(bal);
     }
     *cit = c;
@@ -770,8 +792,9 @@ __device__ __forceinline__ int siblings(const DfsParams &p, int mpw, const uint3
 
 // Publish the class s.path[0 .. plen) + cit with candidates cand[0 .. k) as a
 // queue slot.  False when the queue or the candidate pool is full.
-__device__ __noinline__ bool give(const DfsParams &p, PWork &s, uint32_t epoch, int plen, uint32_t cit,
-                                  const uint32_t *cand, int k) {
+template <bool REP>
+__device__ __noinline__ bool give(const DfsParams &p, PWork<REP> &s, uint32_t epoch, int plen, uint32_t cit,
+                                  uint32_t sup, const uint32_t *cand, int k) {
     const int lane = threadIdx.x & 31;
     unsigned long long off = 0, slot = ~0ull;
     __syncwarp();
@@ -796,6 +819,7 @@ __device__ __noinline__ bool give(const DfsParams &p, PWork &s, uint32_t epoch, 
     if (lane < plen) tk->items[lane] = s.path[lane];
     if (lane == 0) {
         tk->items[plen] = cit;
+        tk->support = sup;
         tk->len = (uint32_t)(plen + 1);
         tk->n_cand = (uint32_t)k;
         tk->cand_off = off;
@@ -808,12 +832,92 @@ __device__ __noinline__ bool give(const DfsParams &p, PWork &s, uint32_t epoch, 
     return true;
 }
 
-template <int MB, int PG>
+// The scheduling network on one class, by one warp: the arithmetic of
+// dfs_kernel's inference (bf16 weights and activations, float32 sums in the
+// same order); w: the CTA's copy, W1 and W2 transposed to [in][out].
+__device__ void proj_mlp(const __nv_bfloat16 *w, const float *x, float *y) {
+    const __nv_bfloat16 *W1t = w, *b1 = W1t + 64 * 8, *W2t = b1 + 64, *b2 = W2t + 64 * 64, *W3 = b2 + 64,
+                        *b3 = W3 + 2 * 64;
+    const int l = threadIdx.x & 31;
+    auto f = [](__nv_bfloat16 v) { return __bfloat162float(v); };
+    auto rb = [](float v) { return __bfloat162float(__float2bfloat16_rn(v)); };
+    float a0 = f(b1[l]), a1 = f(b1[l + 32]);
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const float xi = rb(x[i]);
+        a0 = fmaf(f(W1t[i * 64 + l]), xi, a0);
+        a1 = fmaf(f(W1t[i * 64 + l + 32]), xi, a1);
+    }
+    const float ha = rb(fmaxf(a0, 0.f)), hb = rb(fmaxf(a1, 0.f));
+    float c0 = f(b2[l]), c1 = f(b2[l + 32]);
+#pragma unroll 4
+    for (int i = 0; i < 64; i++) {
+        const float hi = __shfl_sync(0xffffffffu, i < 32 ? ha : hb, i & 31);
+        c0 = fmaf(f(W2t[i * 64 + l]), hi, c0);
+        c1 = fmaf(f(W2t[i * 64 + l + 32]), hi, c1);
+    }
+    const float g0 = rb(fmaxf(c0, 0.f)), g1 = rb(fmaxf(c1, 0.f));
+    float y0 = f(W3[l]) * g0 + f(W3[l + 32]) * g1;
+    float y1 = f(W3[64 + l]) * g0 + f(W3[64 + l + 32]) * g1;
+    for (int d = 16; d > 0; d >>= 1) {
+        y0 += __shfl_xor_sync(0xffffffffu, y0, d);
+        y1 += __shfl_xor_sync(0xffffffffu, y1, d);
+    }
+    if (l == 0) {
+        y[0] = y0 + f(b3[0]);
+        y[1] = y1 + f(b3[1]);
+    }
+    __syncwarp();
+}
+
+// Whether a class Y = X u {c} (support supY, parent supX, k candidates with
+// parent supports psup) is counted through its diffset: as the network says
+// where the choice can pay for asking it (learned_kmin candidates), or by the
+// size rule.  The choice never changes a count.
+__device__ __noinline__ bool proj_choose_diff(const DfsParams &p, PWork<true> &s, const DbDesc &D, const __nv_bfloat16 *w,
+                                              int ylen, uint32_t supY, uint32_t supX, const uint32_t *psup, int k) {
+    if (p.diffset_rule && !p.learned) return supX - supY < supY;
+    if (!p.learned || k < p.learned_kmin) return false;
+    const int lane = threadIdx.x & 31;
+    float acc = 0.f;
+    for (int c = lane; c < k; c += 32) acc += (float)psup[c];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+        const float sx = supX > 0 ? (float)supX : 1.f, sy = supY > 0 ? (float)supY : 1.f;
+        s.feat[0] = (float)ylen / 16.f;
+        s.feat[1] = log2f(1.f + (float)supY) / 32.f;
+        s.feat[2] = (float)supY / (float)(D.n > 0 ? D.n : 1);
+        s.feat[3] = log2f(1.f + (float)k) / 16.f;
+        s.feat[4] = (float)supY / sx;
+        s.feat[5] = k > 0 ? acc / ((float)k * sx) : 0.f;
+        s.feat[6] = log2f(1.f + (float)D.nw) / 32.f;
+        s.feat[7] = (float)D.thr / sy;
+    }
+    __syncwarp();
+    proj_mlp(w, s.feat, s.out);
+    return s.out[1] > 0.f;
+}
+
+// REP: classes choose their representation (FIM_LEARNED, FIM_DIFFSET_RULE).
+template <int MB, int PG, bool REP>
 __global__ void __launch_bounds__(PW * 32, MB)
 dfs_proj_kernel(const DfsParams p, const ProjParams q) {
     extern __shared__ __align__(16) uint8_t proj_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    PWork &s = reinterpret_cast<PWork *>(proj_smem)[warp];
+    PWork<REP> &s = reinterpret_cast<PWork<REP> *>(proj_smem)[warp];
+    __nv_bfloat16 *const mlp = reinterpret_cast<__nv_bfloat16 *>(proj_smem + sizeof(PWork<REP>) * PW);
+    if (REP && p.learned) {
+        for (int i = threadIdx.x; i < FIM_MLP_PARAMS; i += PW * 32) {
+            int d = i;  // W1 [64][8] and W2 [64][64] are stored [out][in]; kept [in][out]
+            if (i < 64 * 8) d = (i % 8) * 64 + i / 8;
+            else if (i >= 64 * 8 + 64 && i < 64 * 8 + 64 + 64 * 64) {
+                const int k = i - (64 * 8 + 64);
+                d = 64 * 8 + 64 + (k % 64) * 64 + k / 64;
+            }
+            mlp[d] = p.mlp_w[i];
+        }
+        __syncthreads();
+    }
     // workers are numbered across the CTAs, so that few roots spread over the SMs
     const int64_t wid = (int64_t)warp * gridDim.x + blockIdx.x;
     const unsigned long long n_workers = (unsigned long long)gridDim.x * PW;
@@ -824,6 +928,7 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
     if ((unsigned long long)wid >= 8 * nr) return;
     Space sp;
     sp.gfr = p.frame_items + wid * p.frame_pool;
+    sp.gfs = REP ? p.frame_sups + wid * p.frame_pool : nullptr;
     sp.gst = p.stack_bits + wid * q.gstack;
     sp.gfr_cap = (int)p.frame_pool;
     sp.gst_cap = (int)q.gstack;
@@ -835,7 +940,7 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
     if (lane == 0) {
         atomicCAS(&p.ctr->t_first, 0ull, globaltimer_ns());
         s.rec_next = s.rec_end = s.it_next = s.it_end = 0ull;
-        s.n_sup = s.n_words = s.n_bytes = s.n_classes = s.emitted = s.emitted_items = 0ull;
+        s.n_sup = s.n_words = s.n_bytes = s.n_classes = s.n_diff = s.emitted = s.emitted_items = 0ull;
         s.max_len = 0;
     }
     bool roots_left = true;
@@ -894,6 +999,7 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
         if (kind == 2) roots_left = false;
         // ---- its columns and candidates --------------------------------------
         uint32_t a = 0, b = 0, bc = 0;
+        uint32_t supY = 0, supX = 0;  // REP: the class's support and its parent's
         int tlen = 2, kq = 0;
         unsigned long long coff_q = 0;
         if (kind == 1 && q.triple) {
@@ -906,8 +1012,13 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
             const unsigned long long rt = p.root_order ? p.root_order[tt] : tt;
             a = p.root_a[rt];
             b = p.root_b[rt];
+            if (REP) {
+                supY = p.root_sup[rt];
+                supX = __ldg(p.item_sup + __ldg(p.perm + a));
+            }
         } else {
             const Task *tk = p.tasks + t;
+            if (REP) supY = __ldcg(&tk->support);
             tlen = (int)__ldcg(&tk->len);
             kq = (int)__ldcg(&tk->n_cand);
             coff_q = __ldcg(&tk->cand_off);
@@ -955,8 +1066,16 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
                     const uint32_t v = i < ak ? __ldg(row + i) : 0u;
                     const bool f = v != 0u && ((__ldg(rc + (id >> 5)) >> (id & 31)) & 1u);
                     const uint32_t bal = __ballot_sync(0xffffffffu, f);
-                    if (f) fr[k + __popc(bal & ((1u << lane) - 1u))] = (i << 16) | id;
+                    if (f) {
+                        const int at = k + __popc(bal & ((1u << lane) - 1u));
+                        fr[at] = (i << 16) | id;
+                        if (REP) fsup_at(s, sp, f0)[at] = v;
+                    }
                     k += __popc(bal);
+                }
+                if (REP) {
+                    supY = __ldg(row + ci);
+                    supX = (uint32_t)__ldg(p.pair_cnt + (int64_t)a * mf + idb);
                 }
             }
             if (lane == 0) {
@@ -995,6 +1114,7 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
                     while (bits) {
                         const uint32_t id = (uint32_t)(w * 32 + __ffs(bits) - 1);
                         bits &= bits - 1;
+                        if (REP) fsup_at(s, sp, f0)[at] = (uint32_t)__ldg(p.pair_cnt + (int64_t)a * mf + id);
                         fr[at++] = ((uint32_t)__ldg(p.perm + id) << 16) | id;
                     }
                     k += (int)__shfl_sync(0xffffffffu, x, 31);
@@ -1008,7 +1128,11 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
                     if (isb) bcol = i0 + (uint32_t)__ffs(isb) - 1u;
                     const bool f = i < ak && id > b && ((__ldg(rb + (id >> 5)) >> (id & 31)) & 1u);
                     const uint32_t bal = __ballot_sync(0xffffffffu, f);
-                    if (f) fr[k + __popc(bal & ((1u << lane) - 1u))] = (i << 16) | id;
+                    if (f) {
+                        const int at = k + __popc(bal & ((1u << lane) - 1u));
+                        fr[at] = (i << 16) | id;
+                        if (REP) fsup_at(s, sp, f0)[at] = (uint32_t)__ldg(p.pair_cnt + (int64_t)a * mf + id);
+                    }
                     k += __popc(bal);
                 }
             }
@@ -1052,6 +1176,9 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
         }
         if (!ok && lane == 0) perr(p, FIM_E_STACK);
         bool go = ok && k > 0 && len_ok;
+        // this task's classes, supports and longest set
+        uint32_t t_cls = 0, t_sup = 0, t_diff = 0;
+        int t_len = 0;
         while (go) {
             // the error flag and how many workers wait for the queue: loaded
             // here, used after the class has been counted
@@ -1064,14 +1191,24 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
             }
             bool polled = false;
             {
-                uint32_t *cf = frame_at(s, sp, fc);
-                const int nF = proj_class_pass<PG>(p, s, thr, src0, src1, cols, stride, W, lg, cf, kc, plen,
-                                                   kc >= 2 ? stack_at(s, sp, sc) : nullptr, cf);
+                uint32_t *cf = frame_at(s, sp, fc), *cs = fsup_at(s, sp, fc);
+                // (a queued class's prefix comes whole, and a projected pair's
+                // parent is all of T(a): no parent's bitmap to differ from)
+                bool diff = false;
+                if constexpr (REP)
+                    if (L >= 0 || (kind == 1 && (q.triple || q.direct))) diff = proj_choose_diff(p, s, D, mlp, plen, supY, supX, cs, kc);
+                const int nF = proj_class_pass<PG, REP>(p, s, thr, src0, src1, cols, stride, W, lg, cf, kc, plen,
+                                                        kc >= 2 ? stack_at(s, sp, sc) : nullptr, cf, cs, diff);
+                t_cls++;
+                t_sup += (uint32_t)kc;
+                t_diff += diff;
+                if (nF > 0 && plen + 1 > t_len) t_len = plen + 1;
                 // sets of plen + 1 items: their classes give sets of plen + 2
                 if (nF >= 2 && (maxlen == 0 || (uint32_t)plen + 2 <= maxlen)) {
                     L++;
                     if (lane == 0) {
                         const int bS = L > 0 ? s.ftopS[L - 1] : 0, bG = L > 0 ? s.ftopG[L - 1] : 0;
+                        if (REP) s.supY[L] = supY;
                         s.nF[L] = nF;
                         s.cur[L] = 0;
                         s.fpos[L] = fc;
@@ -1101,9 +1238,11 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
                                 const int at = place(s.nF[l], s.ftopS[L], PFR, s.ftopG[L], sp.gfr_cap);
                                 if (at == INT32_MIN) break;
                                 uint32_t *tmp = frame_at(s, sp, at), cit = 0;
-                                const int kd = siblings(p, mpw, frame_at(s, sp, s.fpos[l]), s.cur[l], s.nF[l], tmp, &cit);
+                                const uint32_t *ls = fsup_at(s, sp, s.fpos[l]);
+                                const int kd = siblings<REP>(p, mpw, frame_at(s, sp, s.fpos[l]), ls, s.cur[l], s.nF[l],
+                                                             tmp, fsup_at(s, sp, at), &cit);
                                 if (kd == 1) break;  // too small to move
-                                if (kd > 1 && !give(p, s, epoch, tlen + l, cit, tmp, kd)) break;
+                                if (kd > 1 && !give(p, s, epoch, tlen + l, cit, REP ? ls[s.cur[l]] : 0u, tmp, kd)) break;
                                 given += kd > 1;
                                 __syncwarp();
                                 if (lane == 0) s.cur[l]++;
@@ -1124,7 +1263,12 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
                     break;
                 }
                 uint32_t cit = 0;
-                kc = siblings(p, mpw, frame_at(s, sp, s.fpos[L]), j, nFL, frame_at(s, sp, fc), &cit);
+                kc = siblings<REP>(p, mpw, frame_at(s, sp, s.fpos[L]), fsup_at(s, sp, s.fpos[L]), j, nFL,
+                                   frame_at(s, sp, fc), fsup_at(s, sp, fc), &cit);
+                if (REP) {
+                    supX = s.supY[L];
+                    supY = fsup_at(s, sp, s.fpos[L])[j];
+                }
                 __syncwarp();  // cur[L] and the path have been read
                 if (lane == 0) {
                     s.cur[L] = j + 1;
@@ -1146,6 +1290,12 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
         }
         __syncwarp();
         if (lane == 0) {
+            s.n_sup += t_sup;
+            s.n_classes += t_cls;
+            s.n_diff += t_diff;
+            s.n_words += (unsigned long long)t_sup * (unsigned long long)W;
+            s.n_bytes += 4ull * (unsigned long long)W * ((unsigned long long)t_sup + 3ull * t_cls);
+            if (t_len > s.max_len) s.max_len = t_len;
             busy += globaltimer_ns() - t_task;
             if (kind == 1) {
                 done++;
@@ -1168,6 +1318,7 @@ dfs_proj_kernel(const DfsParams p, const ProjParams q) {
             atomicAdd(&p.ctr->dfs_bytes, s.n_bytes);
             atomicAdd(&p.ctr->dfs_touched, s.n_bytes);
             atomicAdd(&p.ctr->classes, s.n_classes);
+            if (s.n_diff) atomicAdd(&p.ctr->diffset, s.n_diff);
         }
         if (s.max_len) atomicMax(&p.ctr->max_len, s.max_len);
         atomicAdd(&p.ctr->busy_ns, busy);
@@ -1276,9 +1427,14 @@ int launch_proj_small_plan(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr, bool
 }
 
 int launch_dfs_proj(fim_ctx *ctx, const DfsParams &p, const ProjParams &q, int ctas_per_sm) {
-    const size_t smem = sizeof(PWork) * PW;
+    const bool rep = p.learned || p.diffset_rule;
+    const size_t smem = rep ? sizeof(PWork<true>) * PW + sizeof(__nv_bfloat16) * (FIM_MLP_PARAMS + 6)
+                            : sizeof(PWork<false>) * PW;
     const unsigned grid = (unsigned)(ctx->num_sms * ctas_per_sm);
-    auto kern = ctas_per_sm >= 4 ? dfs_proj_kernel<4, 4> : (ctas_per_sm == 3 ? dfs_proj_kernel<3, 8> : dfs_proj_kernel<2, 8>);
+    auto kern = rep ? (ctas_per_sm >= 4 ? dfs_proj_kernel<4, 4, true> : dfs_proj_kernel<2, 8, true>)
+                    : (ctas_per_sm >= 4   ? dfs_proj_kernel<4, 4, false>
+                       : ctas_per_sm == 3 ? dfs_proj_kernel<3, 8, false>
+                                          : dfs_proj_kernel<2, 8, false>);
     FIM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ctx->launches++;
     kern<<<grid, PW * 32, smem, ctx->stream>>>(p, q);

@@ -106,3 +106,30 @@ def test_shards_and_repeats(ctx):
         parts.append(fim.fim_fetch_results(ctx))
     fim.fim_merge_results(ctx, c.n, c.m, parts)
     assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
+
+
+@pytest.mark.parametrize("logit", [-5.0, 5.0, None])
+def test_representation_choice_on_projected_columns(ctx, logit):
+    # the network (forced to either representation, or as drawn) and the size
+    # rule on warp workers: projected, direct and with queued classes
+    w = datagen.mlp_init_weights(2)
+    if logit is not None:
+        w[-1] = logit
+    fim.fim_sched_load_weights(ctx, w)
+    fim.fim_set_tuning(ctx, "learned_kmin", 1)
+    try:
+        for c, minsup in [(datagen.planted(n=60_000, m=500, n_patterns=40, seed=11), 250),
+                          (datagen.random_dense(12_000, 40, 0.3, 3), 300),
+                          (datagen.zipf_baskets(3_000, 90, 0.9, 7.0, 4), 12)]:
+            for flags in (fim.FIM_LEARNED, fim.FIM_DIFFSET_RULE, fim.FIM_LEARNED | fim.FIM_MAXLEN(4)):
+                _check(ctx, c, minsup, flags, **(dict(max_len=4) if flags >> 24 else {}))
+                st = fim.fim_get_stats(ctx)
+                if logit is not None and flags == fim.FIM_LEARNED:
+                    # queued classes have no parent's bitmap to differ from
+                    assert (st["diffset_classes"] > 0) == (logit > 0 and st["classes"] > st["tasks_pushed"])
+            fim.fim_set_tuning(ctx, "learned_order", 1)  # pair roots, in the network's order
+            _check(ctx, c, minsup, fim.FIM_LEARNED)
+            fim.fim_set_tuning(ctx, "learned_order", 0)
+    finally:
+        fim.fim_set_tuning(ctx, "learned_order", 0)
+        fim.fim_set_tuning(ctx, "learned_kmin", 8)
