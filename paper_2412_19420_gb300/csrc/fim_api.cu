@@ -287,8 +287,6 @@ int fim_build_bitmaps(fim_ctx *ctx, const void *indptr, const void *indices, int
     else if (mapped) FIM_TRY(launch_build_bitmaps(ctx, d_ptr, d_idx, h_nnz, nullptr, nullptr, cmp));
     else FIM_TRY(launch_build_bitmaps(ctx, d_ptr, d_idx, h_nnz, indptr, h_nnz > 0 ? indices : nullptr, cmp));
     cudaEventRecord(ctx->ev[1], st);
-    FIM_TRY(launch_item_support(ctx));
-    cudaEventRecord(ctx->ev[2], st);
     BuildFlags bf{};
     FIM_CUDA_TRY(cudaMemcpyAsync(&bf, ctx->dev_flag.p, sizeof(bf), cudaMemcpyDeviceToHost, st));
     FIM_CUDA_TRY(cudaStreamSynchronize(st));
@@ -298,7 +296,7 @@ int fim_build_bitmaps(fim_ctx *ctx, const void *indptr, const void *indices, int
     ctx->row_pairs = bf.row_pairs;
     ctx->rows_kept = ctx->row_cap > 0 && (uint64_t)bf.nnz <= ctx->row_cap;
     cudaEventElapsedTime(&ctx->stats.ms_build, ctx->ev[0], ctx->ev[1]);
-    cudaEventElapsedTime(&ctx->stats.ms_singletons, ctx->ev[1], ctx->ev[2]);
+    ctx->stats.ms_singletons = 0.f;  // counted by the build kernel
     if (ctx->debug_checks) FIM_TRY(run_check_pads(ctx));
     ctx->stats.launches_build = ctx->launches - launches0;
     ctx->built = true;

@@ -421,7 +421,6 @@ void fim_release(fim_ctx *ctx, DevBuf &b);
 // compact: the CSR holds uint32 row offsets and uint16 item ids.
 int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indices, int64_t nnz,
                          const void *h_indptr, const void *h_indices, bool compact);
-int launch_item_support(fim_ctx *ctx);
 int launch_rank_items(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr);
 int launch_emit_singletons(fim_ctx *ctx, MineCounters *d_ctr);
 int launch_max_row_freq(fim_ctx *ctx, const int64_t *d_indptr, const int32_t *d_indices,

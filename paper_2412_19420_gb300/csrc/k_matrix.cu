@@ -1,4 +1,5 @@
-// k_matrix.cu -- matrix construction (Eq. 1) and singleton support (Eq. 3).
+// k_matrix.cu -- matrix construction (Eq. 1), singleton support (Eq. 3) and the
+// internal ids.
 //
 // build_bitmaps_kernel: one CTA owns a block of WB words (32*WB transactions)
 // and a range of IB items.  Each warp streams a 32-row group's elements
@@ -22,7 +23,8 @@ template <bool CMP>
 __global__ void __launch_bounds__(BUILD_THREADS)
 build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__ indices_v,
                      int64_t n, int32_t m, int64_t nnz, int64_t nwp, int ib, int64_t blk0,
-                     uint32_t *__restrict__ bm, BuildFlags *__restrict__ flags, RowCopy rows) {
+                     uint32_t *__restrict__ bm, uint32_t *__restrict__ sup, BuildFlags *__restrict__ flags,
+                     RowCopy rows) {
     using Off = typename std::conditional<CMP, uint32_t, int64_t>::type;
     using Id = typename std::conditional<CMP, unsigned short, int32_t>::type;
     const Off *const indptr = static_cast<const Off *>(indptr_v);
@@ -78,16 +80,29 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         if (__any_sync(0xffffffffu, bad)) continue;  // malformed: flagged, not read
         const int64_t e_begin = __shfl_sync(0xffffffffu, off, 0);
         const uint32_t wl = (uint32_t)((rb - t0) >> 5);
+        // Rows all hold an id (the usual case): their starts are distinct, one
+        // OR over the lanes marks those inside a chunk of 32 ids, and an id's
+        // row is a popcount away; else a binary search over the starts.
+        const bool dense = e_end - e_begin < (1ll << 30) && !__any_sync(0xffffffffu, lane < nr && off_next == off);
+        const int ar = dense ? (int)(off - e_begin) : 0;
+        int before = -1;  // rows begun before the chunk, less one
         for (int64_t e0 = e_begin; e0 < e_end; e0 += 32) {
             const int64_t e = e0 + lane;
             const bool v = e < e_end;
             const int32_t it = v ? (int32_t)indices[e] : 0;
             int r = 0;  // largest r < nr with start(r) <= e
+            if (dense) {
+                const unsigned in = (unsigned)(ar - (int)(e0 - e_begin));
+                const uint32_t heads = __reduce_or_sync(0xffffffffu, lane < nr && in < 32u ? 1u << in : 0u);
+                r = before + __popc(heads & (0xFFFFFFFFu >> (31 - lane)));
+                before += __popc(heads);
+            } else {
 #pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int c = r + step;
-                const int64_t oc = __shfl_sync(0xffffffffu, off, c < 32 ? c : 31);
-                if (c < nr && oc <= e) r = c;
+                for (int step = 16; step > 0; step >>= 1) {
+                    const int c = r + step;
+                    const int64_t oc = __shfl_sync(0xffffffffu, off, c < 32 ? c : 31);
+                    if (c < nr && oc <= e) r = c;
+                }
             }
             if (!v) continue;
             if (it < 0 || it >= m) { bad = 1; continue; }
@@ -111,36 +126,22 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         atomicMax(&flags->max_len, s_max);
         atomicAdd(&flags->row_pairs, s_pairs);
     }
-    // write-out: 16-byte stores, four consecutive threads per 64-byte row
-    for (int k = threadIdx.x; k < icount * (WB / 4); k += blockDim.x) {
+    // write-out: 16-byte stores, four consecutive threads per 64-byte row; the
+    // row's popcount rides along into S(I_j) (Eq. 3).  (A pass of its own over
+    // the columns read all of them back: 0.9 ms on 10^7 x 5,000.)
+    for (int b = 0; b < icount * (WB / 4); b += blockDim.x) {  // block-uniform trips
+        const int k = b + threadIdx.x;
         const int r = k / (WB / 4), c = k % (WB / 4);
-        const uint4 v = make_uint4(tile[(4 * c + 0) * ms + r], tile[(4 * c + 1) * ms + r],
-                                   tile[(4 * c + 2) * ms + r], tile[(4 * c + 3) * ms + r]);
-        *reinterpret_cast<uint4 *>(bm + (int64_t)(i0 + r) * nwp + w0 + 4 * c) = v;
-    }
-}
-
-// S(I_j) = popcount of column j, split over segments of SEG words.
-constexpr int SEG = 8192;
-__global__ void __launch_bounds__(256)
-item_support_kernel(const uint32_t *__restrict__ bm, int64_t nwp, uint32_t *__restrict__ sup) {
-    const int j = blockIdx.x;
-    const int64_t b = (int64_t)blockIdx.y * SEG;
-    const int64_t e = min64(nwp, b + SEG);
-    const uint32_t *col = bm + (int64_t)j * nwp;
-    uint32_t c = 0;
-    for (int64_t w = b + 4 * threadIdx.x; w < e; w += 4 * blockDim.x) {
-        uint4 v = ldg_u4(col + w);
-        c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
-    }
-    c = warp_sum_u32(c);
-    __shared__ uint32_t s[8];
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); k++) t += s[k];
-        if (t) atomicAdd(&sup[j], t);
+        uint32_t cnt = 0;
+        if (r < icount) {
+            const uint4 v = make_uint4(tile[(4 * c + 0) * ms + r], tile[(4 * c + 1) * ms + r],
+                                       tile[(4 * c + 2) * ms + r], tile[(4 * c + 3) * ms + r]);
+            *reinterpret_cast<uint4 *>(bm + (int64_t)(i0 + r) * nwp + w0 + 4 * c) = v;
+            cnt = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+        }
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, 1);
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, 2);
+        if (c == 0 && cnt) atomicAdd(&sup[i0 + r], cnt);
     }
 }
 
@@ -213,6 +214,7 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
     BuildFlags *flags = ctx->dev_flag.as<BuildFlags>();
     cudaStream_t st = ctx->stream;
     FIM_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(BuildFlags), st));
+    FIM_CUDA_TRY(cudaMemsetAsync(ctx->item_sup.p, 0, sizeof(uint32_t) * (size_t)ctx->m, st));
     // the rows, kept as 32-bit offsets and 16-bit ids for the pair pass, where
     // they hold at most kRowCopyItems items on average (longer rows make more
     // pairs than the tensor cores' pass costs)
@@ -268,20 +270,9 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
         dim3 grid((unsigned)(b1 - b0), (unsigned)niblk);
         ctx->launches++;
         kern<<<grid, BUILD_THREADS, smem, st>>>(d_indptr, d_indices, ctx->n, ctx->m, nnz, ctx->nwp, ib, b0,
-                                                ctx->bm.as<uint32_t>(), flags, rows);
+                                                ctx->bm.as<uint32_t>(), ctx->item_sup.as<uint32_t>(), flags, rows);
         FIM_CUDA_TRY(cudaGetLastError());
     }
-    return FIM_OK;
-}
-
-int launch_item_support(fim_ctx *ctx) {
-    uint32_t *sup = ctx->item_sup.as<uint32_t>();
-    FIM_CUDA_TRY(cudaMemsetAsync(sup, 0, sizeof(uint32_t) * (size_t)ctx->m, ctx->stream));
-    if (ctx->m == 0 || ctx->nwp == 0) return FIM_OK;
-    dim3 grid((unsigned)ctx->m, (unsigned)ceil_div64(ctx->nwp, SEG));
-    ctx->launches++;
-    item_support_kernel<<<grid, 256, 0, ctx->stream>>>(ctx->bm.as<uint32_t>(), ctx->nwp, sup);
-    FIM_CUDA_TRY(cudaGetLastError());
     return FIM_OK;
 }
 
