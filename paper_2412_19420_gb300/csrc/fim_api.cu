@@ -37,6 +37,19 @@ constexpr unsigned long long kTriples = 64ull << 20;   // largest table of tripl
 constexpr uint32_t kProjWmax = 1u << 15;         // longest projected column (words)
 constexpr size_t kProjStackBudget = 4ull << 30;  // warp workers' global stacks
 
+constexpr size_t kPinnedBytes = sizeof(MineCounters) > sizeof(BuildFlags) ? sizeof(MineCounters) : sizeof(BuildFlags);
+
+// Read back a device struct (the stream is synchronised): through page-locked
+// memory, which the copy engine writes without a staging pass.
+template <class T>
+int read_back(fim_ctx *ctx, T *host, const void *dev) {
+    static_assert(sizeof(T) <= kPinnedBytes, "landing place");
+    FIM_CUDA_TRY(cudaMemcpyAsync(ctx->pinned, dev, sizeof(T), cudaMemcpyDeviceToHost, ctx->stream));
+    FIM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    memcpy((void *)host, ctx->pinned, sizeof(T));
+    return FIM_OK;
+}
+
 }  // namespace
 
 void fim_set_cuda_error(cudaError_t e, const char *what, const char *file, int line) {
@@ -160,6 +173,12 @@ int fim_create(fim_ctx **out, int device, void *cuda_stream) {
         ctx->own_stream = true;
     }
     for (auto &e : ctx->ev) cudaEventCreate(&e);
+    if (cudaHostAlloc(&ctx->pinned, kPinnedBytes, cudaHostAllocDefault) != cudaSuccess) {
+        (void)cudaGetLastError();
+        ctx->pinned = nullptr;
+        fim_destroy(ctx);
+        return FIM_E_NOMEM;
+    }
     int rc = fim_reserve(ctx, ctx->counters, sizeof(MineCounters));
     if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->dev_flag, sizeof(BuildFlags));
     if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->epoch, sizeof(uint32_t));
@@ -217,6 +236,7 @@ void fim_destroy(fim_ctx *ctx) {
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
+    if (ctx->pinned) cudaFreeHost(ctx->pinned);
     delete ctx;
 }
 
@@ -288,8 +308,7 @@ int fim_build_bitmaps(fim_ctx *ctx, const void *indptr, const void *indices, int
     else FIM_TRY(launch_build_bitmaps(ctx, d_ptr, d_idx, h_nnz, indptr, h_nnz > 0 ? indices : nullptr, cmp));
     cudaEventRecord(ctx->ev[1], st);
     BuildFlags bf{};
-    FIM_CUDA_TRY(cudaMemcpyAsync(&bf, ctx->dev_flag.p, sizeof(bf), cudaMemcpyDeviceToHost, st));
-    FIM_CUDA_TRY(cudaStreamSynchronize(st));
+    FIM_TRY(read_back(ctx, &bf, ctx->dev_flag.p));
     if (bf.bad) return FIM_E_INVAL;
     ctx->max_row_len = bf.max_len;
     ctx->row_nnz = bf.nnz;
@@ -314,6 +333,33 @@ struct MineState {
     bool cta_dfs = false;  // the warp workers' stack was too small: CTA workers
 };
 
+// The search runs on warp workers (k_proj.cu); the trace and no-split
+// options, and searches too deep for a warp worker's stack, on the CTA
+// workers, which look at whole columns.
+bool search_on_warps(uint32_t flags, const MineState &ms) {
+    return !ms.cta_dfs && !(flags & (FIM_TRACE | FIM_NO_SPLIT));
+}
+
+// The largest projection that mf frequent items can have.
+ProjTotals worst_projection(const fim_ctx *ctx, int mf) {
+    ProjTotals t{};
+    const unsigned long long np = (unsigned long long)mf * (unsigned long long)(mf > 0 ? mf - 1 : 0) / 2;
+    t.wmax = (uint32_t)(ceil_div64(ctx->n, 128) * 4);
+    t.words = np * t.wmax;
+    t.rows = (unsigned long long)mf * (unsigned long long)ctx->n;
+    t.cands = np;
+    t.tiles = (unsigned long long)mf * ((t.wmax + 31) / 32);
+    t.triples = (unsigned long long)mf * mf * mf;
+    t.units = (unsigned long long)mf * proj_triple_units(mf);
+    return t;
+}
+
+bool small_plan_takes(const fim_ctx *ctx, int mf, uint32_t flags, const MineState &ms) {
+    const ProjTotals t = worst_projection(ctx, mf);
+    return search_on_warps(flags, ms) && ctx->n_shards == 1 && !((flags & FIM_LEARNED) && ctx->learned_order) &&
+           proj_small_plan_fits(mf) && t.wmax <= kProjWmax && t.words <= kSmallPlanWords && t.rows <= kSmallPlanWords;
+}
+
 // One attempt at the whole mine with the current capacities.  Returns
 // FIM_OK, or an error; *retry is set when a capacity must grow first.
 int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *retry) {
@@ -322,38 +368,43 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     ctx->cur_thr = thr;
     if ((flags & FIM_LEARNED) && !ctx->has_weights) return FIM_E_STATE;
     MineCounters *d_ctr = ctx->counters.as<MineCounters>();
-    FIM_CUDA_TRY(cudaMemsetAsync(d_ctr, 0, sizeof(MineCounters), st));
-    cudaEventRecord(ctx->ev[0], st);
-    FIM_TRY(launch_rank_items(ctx, thr, d_ctr));
-    if (ctx->shard == 0) FIM_TRY(launch_emit_singletons(ctx, d_ctr));
-    FIM_CUDA_TRY(cudaMemcpyAsync(&ctx->host_ctr, d_ctr, sizeof(MineCounters), cudaMemcpyDeviceToHost, st));
-    FIM_CUDA_TRY(cudaStreamSynchronize(st));
-    ctx->mfreq = ctx->host_ctr.m_freq;
-    const int mf = ctx->mfreq;
     const uint32_t maxlen = flags >> 24;
-    {   // the one-entry database table of a single-database mine (DFS, compactor)
-        DbDesc &d = ctx->host_db;
-        d = DbDesc{};
-        d.n = ctx->n;
-        d.nw = ctx->nw;
-        d.nwp = ctx->nwp;
-        d.m = ctx->m;
-        d.mfreq = mf;
-        d.thr = thr;
-        d.maxlen = maxlen;
-        FIM_TRY(fim_reserve(ctx, ctx->dbdesc, sizeof(DbDesc)));
-        ctx->up_desc.clear();  // the batched mine's table is overwritten
+    DbDesc &d = ctx->host_db;  // the one-entry database table of a single-database mine (DFS, compactor)
+    d = DbDesc{};
+    d.n = ctx->n;
+    d.nw = ctx->nw;
+    d.nwp = ctx->nwp;
+    d.m = ctx->m;
+    d.thr = thr;
+    d.maxlen = maxlen;
+    FIM_TRY(fim_reserve(ctx, ctx->dbdesc, sizeof(DbDesc)));
+    ctx->up_desc.clear();  // the batched mine's table is overwritten
+    // Few items, and a search the one-launch plan takes: the whole mine is
+    // queued at once, sized for m' = m, and m' is read on the device (its
+    // read-back in mid-mine left the GPU idle for some 12 us).
+    const bool blind = mine_begin_fits(ctx->m) && ctx->m >= 3 && ctx->nw > 0 && (maxlen == 0 || maxlen >= 3) &&
+                       !(flags & FIM_PAIRS_POPC) && small_plan_takes(ctx, ctx->m, flags, ms);
+    cudaEventRecord(ctx->ev[0], st);
+    if (blind) {
+        FIM_TRY(fim_reserve(ctx, ctx->pair_cnt, sizeof(int) * (size_t)ctx->m * (size_t)ctx->m + 16));
+        FIM_TRY(launch_mine_begin(ctx, d, d_ctr));
+        ctx->mfreq = ctx->m;
+    } else {
+        FIM_CUDA_TRY(cudaMemsetAsync(d_ctr, 0, sizeof(MineCounters), st));
+        FIM_TRY(launch_rank_items(ctx, thr, d_ctr));
+        if (ctx->shard == 0) FIM_TRY(launch_emit_singletons(ctx, d_ctr));
+        FIM_TRY(read_back(ctx, &ctx->host_ctr, d_ctr));
+        ctx->mfreq = ctx->host_ctr.m_freq;
+        d.mfreq = ctx->mfreq;
         FIM_CUDA_TRY(cudaMemcpyAsync(ctx->dbdesc.p, &d, sizeof(DbDesc), cudaMemcpyHostToDevice, st));
     }
+    const int mf = ctx->mfreq;  // m', or its bound m
     cudaEventRecord(ctx->ev[1], st);
     const bool do_pairs = mf >= 2 && (maxlen == 0 || maxlen >= 2);
     const bool do_dfs = do_pairs && mf >= 3 && (maxlen == 0 || maxlen >= 3);
-    // The search runs on warp workers (k_proj.cu); the trace and no-split
-    // options, and searches too deep for a warp worker's stack, on the CTA
-    // workers, which look at whole columns.
     const bool rep = (flags & (FIM_LEARNED | FIM_DIFFSET_RULE)) != 0;  // classes choose their representation
     const bool net_order = (flags & FIM_LEARNED) && ctx->learned_order;  // the network orders the pair roots
-    const bool warp_dfs = do_dfs && !ms.cta_dfs && !(flags & (FIM_TRACE | FIM_NO_SPLIT));
+    const bool warp_dfs = do_dfs && search_on_warps(flags, ms);
     // Small matrices of short rows: few triples, which the bit columns
     // themselves count sooner than three more launches would (5,746 x 99: 228
     // against 247 us a mine); rows that hold a third of the frequent items make
@@ -367,16 +418,8 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     // roots, projection), sized for the worst case, so that nothing has to
     // come back to the host before the search.
     const size_t npairs_all = (size_t)mf * (size_t)(mf > 0 ? mf - 1 : 0) / 2;
-    ProjTotals proj{};
-    proj.wmax = (uint32_t)(ceil_div64(ctx->n, 128) * 4);
-    proj.words = (unsigned long long)npairs_all * proj.wmax;
-    proj.rows = (unsigned long long)mf * (unsigned long long)ctx->n;
-    proj.cands = npairs_all;
-    proj.tiles = (unsigned long long)mf * ((proj.wmax + 31) / 32);
-    proj.triples = (unsigned long long)mf * mf * mf;
-    proj.units = (unsigned long long)mf * proj_triple_units(mf);
-    const bool small_plan = warp_dfs && ctx->n_shards == 1 && !net_order && proj_small_plan_fits(mf) && proj.wmax <= kProjWmax &&
-                            proj.words <= kSmallPlanWords && proj.rows <= kSmallPlanWords;
+    ProjTotals proj = worst_projection(ctx, mf);
+    const bool small_plan = do_dfs && small_plan_takes(ctx, mf, flags, ms);
     // automatic: keep low-support classes sparse when the frequent item
     // columns do not fit in half of L2 (streaming whole columns from HBM
     // is latency-bound; from L2 the dense pass is as fast)
@@ -407,7 +450,8 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         FIM_TRY(fim_reserve(ctx, ctx->pairbits, sizeof(uint32_t) * (size_t)mf * mpw));
         FIM_TRY(fim_reserve(ctx, ctx->roots, sizeof(uint32_t) * 3 * npairs));
         int rc = FIM_E_INVAL;
-        if (!(flags & FIM_PAIRS_POPC))
+        if (blind) rc = launch_pairs_tc_blind(ctx);
+        else if (!(flags & FIM_PAIRS_POPC))
             rc = pairs_rows_pays(ctx) ? launch_pairs_rows(ctx) : launch_pairs_tc(ctx, 0, true, st);
         if (rc == FIM_OK) ctx->stats.pair_path = 1;
         else FIM_TRY(launch_pairs_popc(ctx));
@@ -417,7 +461,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         }
         if (small_plan) {
             FIM_TRY(reserve_root_plan(ctx, npairs));
-            FIM_TRY(launch_proj_small_plan(ctx, thr, d_ctr, !direct));
+            FIM_TRY(launch_proj_small_plan(ctx, mf, thr, d_ctr, !direct));
         } else {
             FIM_TRY(launch_pairs_finalize(ctx, thr, d_ctr));
         }
@@ -442,7 +486,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         ProjParams q{};
         if (on_warps) {
             const bool triples = !direct && ctx->n_shards == 1 && !net_order && proj.triples <= kTriples;
-            if (!direct) FIM_TRY(launch_projection(ctx, proj, small_plan, triples, thr));
+            if (!direct) FIM_TRY(launch_projection(ctx, mf, proj, small_plan, triples, thr));
             if (triples) {
                 q.triple = ctx->proj_triple.as<uint32_t>();
                 q.roots = ctx->proj_roots.as<unsigned long long>();
@@ -553,9 +597,9 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         else FIM_TRY(launch_dfs(ctx, p, workers, ctx->dfs_block));
     }
     cudaEventRecord(ctx->ev[3], st);
-    FIM_CUDA_TRY(cudaMemcpyAsync(&ctx->host_ctr, d_ctr, sizeof(MineCounters), cudaMemcpyDeviceToHost, st));
-    FIM_CUDA_TRY(cudaStreamSynchronize(st));
+    FIM_TRY(read_back(ctx, &ctx->host_ctr, d_ctr));
     const MineCounters &c = ctx->host_ctr;
+    ctx->mfreq = c.m_freq;
     if (c.err == FIM_E_STACK && on_warps) {
         ms.cta_dfs = true;
         *retry = true;
@@ -582,9 +626,9 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         return FIM_OK;
     }
     int lmax = c.max_len;
-    if (ctx->shard == 0 && mf >= 1 && lmax < 1) lmax = 1;
+    if (ctx->shard == 0 && c.m_freq >= 1 && lmax < 1) lmax = 1;
     const unsigned long long n_sets = c.n_records - c.rec_holes;
-    if (ctx->shard == 0 && n_sets > (unsigned long long)mf && lmax < 2) lmax = 2;
+    if (ctx->shard == 0 && n_sets > (unsigned long long)c.m_freq && lmax < 2) lmax = 2;
     ctx->host_ctr.max_len = lmax;
     FIM_TRY(launch_compact(ctx, c.n_records, n_sets, 1, ctx->m));
     cudaEventRecord(ctx->ev[4], st);

@@ -301,6 +301,7 @@ struct fim_ctx {
     DevBuf dbdesc;              // DbDesc table of the mine
     DbDesc host_db{};           // host copy of a single-database table
     MineCounters host_ctr;
+    void *pinned = nullptr;     // page-locked landing place of the read-backs
     unsigned long long rec_cap = 0, rec_items_cap = 0;
 
     // compactor
@@ -423,6 +424,9 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
                          const void *h_indptr, const void *h_indices, bool compact);
 int launch_rank_items(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr);
 int launch_emit_singletons(fim_ctx *ctx, MineCounters *d_ctr);
+// few items: counters cleared, ids, singletons and the table in one launch
+bool mine_begin_fits(int m);
+int launch_mine_begin(fim_ctx *ctx, const DbDesc &d, MineCounters *d_ctr);
 int launch_max_row_freq(fim_ctx *ctx, const int64_t *d_indptr, const int32_t *d_indices,
                         MineCounters *d_ctr);
 
@@ -431,6 +435,7 @@ int launch_pairs_popc(fim_ctx *ctx);
 // tcgen05, the pairs of items a0 .. m' - 1 (0: all); the counts are cleared
 // first unless clear is false
 int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st);
+int launch_pairs_tc_blind(fim_ctx *ctx);
 bool pairs_rows_pays(const fim_ctx *ctx);
 int launch_pairs_rows(fim_ctx *ctx);  // rows, and the most frequent items' block by launch_pairs_tc
 int launch_pairs_finalize(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr);
@@ -445,9 +450,9 @@ int launch_epoch_bump(fim_ctx *ctx);
 // k_proj.cu: projected columns and the prefix extension on them.  The plan
 // synchronises the stream (its totals size the buffers).
 int launch_proj_plan(fim_ctx *ctx, ProjTotals *host);
-int launch_projection(fim_ctx *ctx, const ProjTotals &t, bool cands_listed, bool triples, uint32_t thr);
+int launch_projection(fim_ctx *ctx, int mf, const ProjTotals &t, bool cands_listed, bool triples, uint32_t thr);
 bool proj_small_plan_fits(int mf);
-int launch_proj_small_plan(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr, bool triples);
+int launch_proj_small_plan(fim_ctx *ctx, int mf, uint32_t thr, MineCounters *d_ctr, bool triples);
 unsigned long long proj_triple_units(int mf);  // most units of the triple pass
 int launch_dfs_proj(fim_ctx *ctx, const DfsParams &p, const ProjParams &q, int ctas_per_sm);
 int proj_workers_per_cta();

@@ -199,7 +199,67 @@ __global__ void emit_singletons_kernel(const uint32_t *__restrict__ sup, const i
     }
 }
 
+// The start of a mine with at most MB_MAX items, in one CTA: the counters and the
+// pair counts cleared, internal ids, singleton records and the database table.
+// (A clear, two kernels, a read-back of m' and an upload of the table before:
+// with the read-back in the middle of the mine gone, and the others through
+// page-locked memory, a 10,000 x 169 mine went from 205 to 173 us.)
+constexpr int MB_T = 1024, MB_MAX = 256;
+__global__ void __launch_bounds__(MB_T)
+mine_begin_kernel(DbDesc d, const uint32_t *__restrict__ sup, MineCounters *ctr, DbDesc *__restrict__ dbs,
+                  int32_t *__restrict__ perm, int32_t *__restrict__ rank, int *__restrict__ pair_cnt,
+                  unsigned long long *__restrict__ rec_off, uint32_t *__restrict__ rec_len,
+                  uint32_t *__restrict__ rec_sup, uint32_t *__restrict__ rec_items, unsigned long long rec_cap,
+                  unsigned long long items_cap) {
+    __shared__ uint32_t s[MB_MAX];
+    const int j = threadIdx.x, m = d.m;
+    for (int i = j; i < (int)(sizeof(MineCounters) / 4); i += MB_T) reinterpret_cast<uint32_t *>(ctr)[i] = 0u;
+    for (int i = j; i < (m * m + 3) / 4; i += MB_T) reinterpret_cast<int4 *>(pair_cnt)[i] = make_int4(0, 0, 0, 0);
+    const uint32_t sj = j < m ? sup[j] : 0u;
+    if (j < m) s[j] = sj;
+    const bool f = j < m && sj >= d.thr;
+    const int mf = __syncthreads_count(f);
+    if (j < m && !f) rank[j] = -1;
+    if (f) {
+        int below = 0;
+        for (int i = 0; i < m; i++) {
+            const uint32_t si = s[i];
+            below += si >= d.thr && (si < sj || (si == sj && i < j));
+        }
+        rank[j] = below;
+        perm[below] = j;
+        if ((unsigned long long)below < rec_cap && (unsigned long long)below < items_cap) {
+            rec_off[below] = (unsigned long long)below;
+            rec_len[below] = 1;
+            rec_sup[below] = sj;
+            rec_items[below] = (uint32_t)below;
+        }
+    }
+    if (j == 0) {
+        ctr->m_freq = mf;
+        ctr->n_records = (unsigned long long)mf;
+        ctr->n_rec_items = (unsigned long long)mf;
+        if ((unsigned long long)mf > rec_cap) ctr->overflow = 1;
+        else if ((unsigned long long)mf > items_cap) ctr->overflow = 2;
+        d.mfreq = mf;
+        *dbs = d;
+    }
+}
+
 }  // namespace
+
+bool mine_begin_fits(int m) { return m <= MB_MAX; }
+
+int launch_mine_begin(fim_ctx *ctx, const DbDesc &d, MineCounters *d_ctr) {
+    ctx->launches++;
+    mine_begin_kernel<<<1, MB_T, 0, ctx->stream>>>(
+        d, ctx->item_sup.as<uint32_t>(), d_ctr, ctx->dbdesc.as<DbDesc>(), ctx->perm.as<int32_t>(),
+        ctx->rank.as<int32_t>(), ctx->pair_cnt.as<int>(), ctx->rec_off.as<unsigned long long>(),
+        ctx->rec_len.as<uint32_t>(), ctx->rec_sup.as<uint32_t>(), ctx->rec_items.as<uint32_t>(), ctx->rec_cap,
+        ctx->rec_items_cap);
+    FIM_CUDA_TRY(cudaGetLastError());
+    return FIM_OK;
+}
 
 int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indices, int64_t nnz,
                          const void *h_indptr, const void *h_indices, bool cmp) {

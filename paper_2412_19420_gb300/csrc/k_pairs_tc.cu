@@ -125,8 +125,16 @@ __device__ __forceinline__ Seg next_seg(int64_t w, int64_t w1, int64_t S, int kd
 
 __global__ void __launch_bounds__(THREADS, 1)
 pairs_tc_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ perm, int64_t nwp, int mf, int ld,
-                int ntb, int64_t S, int64_t W, int kd, int *__restrict__ pair_cnt, int *__restrict__ err) {
+                int ntb, int64_t S, int64_t W, int kd, int *__restrict__ pair_cnt, int *__restrict__ err,
+                const int *__restrict__ mf_dev) {
     extern __shared__ uint8_t smem_raw[];
+    if (mf_dev) {  // m' is known on the device alone: all items, sized here
+        mf = ld = *mf_dev;
+        ntb = (mf + TN - 1) / TN;
+        int64_t tiles = 0;
+        for (int ta = 0; ta * TM < mf; ta++) tiles += tiles_of_row(ta, mf, ntb);
+        W = mf >= 2 ? tiles * S : 0;
+    }
     TcSmem &s = *reinterpret_cast<TcSmem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t w0 = (int64_t)blockIdx.x * W / gridDim.x;
@@ -365,8 +373,30 @@ int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st) {
         ctx->launches++;
         pairs_tc_kernel<<<(unsigned)grid, THREADS, smem, st>>>(
             ctx->bm.as<uint32_t>(), ctx->perm.as<int32_t>() + a0, ctx->nwp, mf, ld, ntb, S, W, kd,
-            ctx->pair_cnt.as<int>() + (size_t)a0 * ld + a0, err);
+            ctx->pair_cnt.as<int>() + (size_t)a0 * ld + a0, err, nullptr);
         FIM_CUDA_TRY(cudaGetLastError());
     }
+    return FIM_OK;
+}
+
+// The pass over all pairs of a mine whose m' the host has not read back (the
+// counts were cleared by mine_begin).
+int launch_pairs_tc_blind(fim_ctx *ctx) {
+    const size_t smem = sizeof(TcSmem) + 1024;
+    FIM_CUDA_TRY(cudaFuncSetAttribute(pairs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MineCounters *d_ctr = ctx->counters.as<MineCounters>();
+    // at most as many CTAs as m' = m would need stages
+    const int nta = (int)ceil_div64(ctx->m, TM), ntb = (int)ceil_div64(ctx->m, TN);
+    int64_t tiles = 0;
+    for (int ta = 0; ta < nta; ta++) tiles += tiles_of_row(ta, ctx->m, ntb);
+    const int64_t S = ceil_div64(ctx->nw, 4);
+    int64_t grid = ctx->pairs_split > 0 ? ctx->pairs_split : ctx->num_sms;
+    if (grid > tiles * S) grid = tiles * S;
+    if (grid <= 0) return FIM_OK;
+    ctx->launches++;
+    pairs_tc_kernel<<<(unsigned)grid, THREADS, smem, ctx->stream>>>(
+        ctx->bm.as<uint32_t>(), ctx->perm.as<int32_t>(), ctx->nwp, 0, 0, 0, S, 0,
+        ctx->pairs_kdrain > 0 ? ctx->pairs_kdrain : KDRAIN_MAX, ctx->pair_cnt.as<int>(), &d_ctr->err, &d_ctr->m_freq);
+    FIM_CUDA_TRY(cudaGetLastError());
     return FIM_OK;
 }

@@ -178,7 +178,7 @@ proj_scan_kernel(ProjItem *__restrict__ items, int mf, unsigned long long *__res
 // the place of nine.
 constexpr int SP_MAX = 256, SP_T = 1024;
 __global__ void __launch_bounds__(SP_T)
-proj_small_plan_kernel(const int *__restrict__ pair_cnt, int mf, uint32_t thr, const int32_t *__restrict__ perm,
+proj_small_plan_kernel(const int *__restrict__ pair_cnt, int m, uint32_t thr, const int32_t *__restrict__ perm,
                        const uint32_t *__restrict__ sup, uint32_t *__restrict__ pairbits, MineCounters *ctr,
                        uint32_t *epoch, unsigned long long *__restrict__ rec_off, uint32_t *__restrict__ rec_len,
                        uint32_t *__restrict__ rec_sup, uint32_t *__restrict__ rec_items, unsigned long long rec_cap,
@@ -194,6 +194,7 @@ proj_small_plan_kernel(const int *__restrict__ pair_cnt, int mf, uint32_t thr, c
     __shared__ ProjItem s_it[SP_MAX];
     __shared__ unsigned long long s_base[2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int mf = *(volatile const int *)&ctr->m_freq;  // <= m, the host's bound
     const int mpw = (mf + 31) / 32;
     for (int i = threadIdx.x; i < KB; i += SP_T) hist[i] = 0;
     for (int a = warp; a < mf; a += NW) {
@@ -255,8 +256,10 @@ proj_small_plan_kernel(const int *__restrict__ pair_cnt, int mf, uint32_t thr, c
         if (lane == 31) {  // the totals
             proj_totals(tot, run);
             tot->wmax = wmax;
-            tile0[mf] = run[3];
-            trip0[mf] = run[5];
+            for (int a = mf; a <= m; a++) {  // (the later kernels search m entries)
+                tile0[a] = run[3];
+                trip0[a] = run[5];
+            }
         }
         uint32_t rn = xn - n;
 #pragma unroll
@@ -286,7 +289,10 @@ proj_small_plan_kernel(const int *__restrict__ pair_cnt, int mf, uint32_t thr, c
         }
     }
     __syncthreads();
-    for (int a = threadIdx.x; a < mf; a += SP_T) items[a] = s_it[a];
+    for (int a = threadIdx.x; a < m; a += SP_T) {
+        if (a >= mf) s_it[a].k = 0;
+        items[a] = s_it[a];
+    }
     // pair records and root classes, in (a, b) order; roots counted by their
     // number of candidates
     for (int pass = 0; pass < 2; pass++) {
@@ -505,11 +511,13 @@ proj_gather_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ 
 __global__ void __launch_bounds__(256)
 proj_triple_kernel(const ProjItem *__restrict__ items, int mf, const unsigned long long *__restrict__ trip0,
                    const uint32_t *__restrict__ cands, const uint32_t *__restrict__ mat,
-                   const uint32_t *__restrict__ pairbits, int mpw, uint32_t thr, uint32_t *__restrict__ triple,
+                   const uint32_t *__restrict__ pairbits, const DbDesc *__restrict__ dbs, uint32_t thr,
+                   uint32_t *__restrict__ triple,
                    unsigned long long *__restrict__ roots, MineCounters *ctr, unsigned long long *rec_off,
                    uint32_t *rec_len, uint32_t *rec_sup, uint32_t *rec_items, unsigned long long rec_cap,
                    unsigned long long items_cap) {
     const int lane = threadIdx.x & 31;
+    const int mpw = (dbs->mfreq + 31) / 32;
     const unsigned long long nu = trip0[mf];
     unsigned long long n_sup = 0, n_words = 0, n_bytes = 0;
     bool any = false;
@@ -1352,9 +1360,9 @@ int launch_proj_plan(fim_ctx *ctx, ProjTotals *host) {
 }
 
 // The projected columns of every item of the plan.
-int launch_projection(fim_ctx *ctx, const ProjTotals &t, bool cands_listed, bool triples, uint32_t thr) {
+int launch_projection(fim_ctx *ctx, int mf, const ProjTotals &t, bool cands_listed, bool triples, uint32_t thr) {
     MineCounters *d_ctr = ctx->counters.as<MineCounters>();
-    const int mf = ctx->mfreq, mpw = (int)ceil_div64(mf, 32);
+    const int mpw = (int)ceil_div64(mf, 32);
     cudaStream_t st = ctx->stream;
     FIM_TRY(fim_reserve(ctx, ctx->proj_mat, sizeof(uint32_t) * (size_t)t.words));
     FIM_TRY(fim_reserve(ctx, ctx->proj_list, sizeof(uint32_t) * (size_t)t.rows));
@@ -1390,7 +1398,7 @@ int launch_projection(fim_ctx *ctx, const ProjTotals &t, bool cands_listed, bool
         ctx->launches++;
         proj_triple_kernel<<<(unsigned)blocks, 256, 0, st>>>(
             ctx->proj_items.as<ProjItem>(), mf, ctx->proj_tiles.as<unsigned long long>() + (mf + 1),
-            ctx->proj_cands.as<uint32_t>(), ctx->proj_mat.as<uint32_t>(), ctx->pairbits.as<uint32_t>(), mpw, thr,
+            ctx->proj_cands.as<uint32_t>(), ctx->proj_mat.as<uint32_t>(), ctx->pairbits.as<uint32_t>(), ctx->dbdesc.as<DbDesc>(), thr,
             ctx->proj_triple.as<uint32_t>(), ctx->proj_roots.as<unsigned long long>(), d_ctr,
             ctx->rec_off.as<unsigned long long>(), ctx->rec_len.as<uint32_t>(), ctx->rec_sup.as<uint32_t>(),
             ctx->rec_items.as<uint32_t>(), ctx->rec_cap, ctx->rec_items_cap);
@@ -1405,8 +1413,8 @@ bool proj_small_plan_fits(int mf) { return mf <= SP_MAX; }
 
 // Pair threshold, records, roots and the projection's plan of a small mine
 // (in place of launch_pairs_finalize, the root plan and launch_proj_plan).
-int launch_proj_small_plan(fim_ctx *ctx, uint32_t thr, MineCounters *d_ctr, bool triples) {
-    const int mf = ctx->mfreq;
+// mf: m', or a bound of it.
+int launch_proj_small_plan(fim_ctx *ctx, int mf, uint32_t thr, MineCounters *d_ctr, bool triples) {
     const size_t npairs = (size_t)mf * (mf - 1) / 2;
     FIM_TRY(fim_reserve(ctx, ctx->proj_items, sizeof(ProjItem) * (size_t)mf));
     FIM_TRY(fim_reserve(ctx, ctx->proj_tiles, 2 * sizeof(unsigned long long) * (size_t)(mf + 1)));
