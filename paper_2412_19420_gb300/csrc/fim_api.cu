@@ -69,6 +69,16 @@ int fim_aux_stream(fim_ctx *ctx) {
     return FIM_OK;
 }
 
+int queue_compact_status(fim_ctx *ctx) {
+    if (ctx->compact_waits)
+        FIM_CUDA_TRY(cudaMemcpyAsync(ctx->pinned, ctx->dev_flag.as<int>() + kCompactErr, sizeof(int),
+                                     cudaMemcpyDeviceToHost, ctx->stream));
+    return FIM_OK;
+}
+int compact_status(fim_ctx *ctx) {
+    return ctx->compact_waits && *static_cast<const int *>(ctx->pinned) ? FIM_E_TIMEOUT : FIM_OK;
+}
+
 // Phase times of the last single-database mine, once its work has finished
 // (events ev[1..4] of that mine; called before anything records them again).
 int fim_finish_phase_times(fim_ctx *ctx) {
@@ -180,7 +190,7 @@ int fim_create(fim_ctx **out, int device, void *cuda_stream) {
         return FIM_E_NOMEM;
     }
     int rc = fim_reserve(ctx, ctx->counters, sizeof(MineCounters));
-    if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->dev_flag, sizeof(BuildFlags));
+    if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->dev_flag, kFlagBytes);
     if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->epoch, sizeof(uint32_t));
     if (rc == FIM_OK && cudaMemsetAsync(ctx->epoch.p, 0, sizeof(uint32_t), ctx->stream) != cudaSuccess) rc = FIM_E_CUDA;
     if (rc != FIM_OK) {
@@ -201,7 +211,7 @@ void fim_destroy(fim_ctx *ctx) {
                      &ctx->cand_pool, &ctx->stack_bits, &ctx->frame_items, &ctx->frame_sups,
                      &ctx->rec_off, &ctx->rec_len, &ctx->rec_sup, &ctx->rec_items, &ctx->counters,
                      &ctx->keys, &ctx->idx_a, &ctx->idx_b, &ctx->hist, &ctx->scan_tmp, &ctx->kv_a, &ctx->kv_b,
-                     &ctx->scan_part, &ctx->out_off,
+                     &ctx->out_off,
                      &ctx->out_items, &ctx->out_sup, &ctx->rule_base, &ctx->rule_part, &ctx->rule_bits,
                      &ctx->rule_kbase, &ctx->rule_set, &ctx->rule_mask,
                      &ctx->rule_conf, &ctx->rule_lift, &ctx->rule_sets, &ctx->probe_buf, &ctx->shard_cost, &ctx->merge_off, &ctx->mlp_w32, &ctx->mlp_wbf, &ctx->trace_x,
@@ -732,8 +742,9 @@ int fim_fetch_results(fim_ctx *ctx, uint64_t *n_sets, uint64_t *n_items_total, u
         FIM_CUDA_TRY(cudaMemcpyAsync(items, ctx->out_items.p, sizeof(uint32_t) * ctx->out_items_total, k, st));
     if (ctx->out_sets)
         FIM_CUDA_TRY(cudaMemcpyAsync(supports, ctx->out_sup.p, sizeof(uint32_t) * ctx->out_sets, k, st));
+    FIM_TRY(queue_compact_status(ctx));
     FIM_CUDA_TRY(cudaStreamSynchronize(st));
-    return FIM_OK;
+    return compact_status(ctx);
 }
 
 int fim_get_stats(const fim_ctx *ctx, fim_stats *out) {

@@ -305,7 +305,8 @@ struct fim_ctx {
     unsigned long long rec_cap = 0, rec_items_cap = 0;
 
     // compactor
-    DevBuf keys, idx_a, idx_b, hist, scan_tmp, kv_a, kv_b, scan_part;
+    DevBuf keys, idx_a, idx_b, hist, scan_tmp, kv_a, kv_b;
+    bool compact_waits = false;  // the last compaction's sort had bounded waits: check its error word
     DevBuf out_off, out_items, out_sup;
     uint64_t out_sets = 0, out_items_total = 0;
     uint64_t mine_serial = 0;   // completed fim_mine calls; names the output held
@@ -478,6 +479,13 @@ int launch_root_plan(fim_ctx *ctx, MineCounters *d_ctr, size_t root_cap, const D
 // itemsets, the rest holes (length 0), which sort last and are left out.
 int launch_compact(fim_ctx *ctx, uint64_t n_records, uint64_t n_valid, int n_db, int m_max,
                    bool identity_items = false);
+
+// Queue the compaction's error word's way to page-locked memory; after the next
+// stream synchronisation compact_status says whether a wait ran out.
+constexpr int kCompactErr = sizeof(BuildFlags) / sizeof(int);  // its place in dev_flag, in ints
+constexpr size_t kFlagBytes = sizeof(BuildFlags) + 4 * sizeof(int);
+int queue_compact_status(fim_ctx *ctx);
+int compact_status(fim_ctx *ctx);
 
 // k_csort.cu: the compactor's sort of a small output in one cluster launch
 int cluster_sort_plan(fim_ctx *ctx, uint64_t R, int kw, int *cl, int *cap, int *per);

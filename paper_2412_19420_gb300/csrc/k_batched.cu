@@ -1525,7 +1525,9 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
         FIM_CUDA_TRY(cudaMemcpyAsync(ctx->batch_item_start.data(), istart,
                                      sizeof(unsigned long long) * (n_db + 1), cudaMemcpyDeviceToHost, st));
         cudaEventRecord(ctx->ev[4], st);
+        FIM_TRY(queue_compact_status(ctx));
         FIM_CUDA_TRY(cudaStreamSynchronize(st));
+        FIM_TRY(compact_status(ctx));
         ctx->batch_n_db = n_db;
         ctx->batch_mined = true;
         fim_stats &s = ctx->stats;

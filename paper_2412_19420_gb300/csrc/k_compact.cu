@@ -9,9 +9,8 @@
 //   3. sorts the records by that key with a stable LSD radix sort of
 //      (key word, record) pairs, 64-bit key words from the least significant
 //      one: each word is gathered once into record order, then sorted by its
-//      8-bit digits (per pass a tile histogram with warp-aggregated counts, a
-//      scan of the [digit][tile] counts, a stable scatter ranked with
-//      __match_any_sync that moves the word with its record index);
+//      8-bit digits, one launch a digit (small outputs: one CTA, or the cluster
+//      of k_csort.cu);
 //   4. writes offsets (exclusive scan of the sizes), items and supports.
 #include <utility>
 #include <vector>
@@ -20,9 +19,11 @@
 
 namespace {
 
-constexpr int RT = 256;          // threads per radix tile
-constexpr int RI = 8;            // keys per thread per tile
-constexpr int TILE = RT * RI;    // 2048
+constexpr int RI = 8;            // keys per thread of a radix tile
+
+// Items a set's key is made of in a local copy (longer sets: in place, a chain
+// of round trips to global memory).
+constexpr int PK_LOCAL = 16;
 
 // Big-endian bit packing into 64-bit words (word 0 most significant), handed
 // to emit(word index, word) as they fill.
@@ -49,6 +50,7 @@ struct KeyPack {
     }
 };
 
+// (With the sort in place this pass took 450 us of 4.2 million records, now 189.)
 // dbs/rec_db/db_bits: with several databases the key starts with the record's
 // database (db_bits wide) and items map back through that database's perm.
 __global__ void prep_keys_kernel(unsigned long long R, const unsigned long long *__restrict__ rec_off,
@@ -66,22 +68,26 @@ __global__ void prep_keys_kernel(unsigned long long R, const unsigned long long 
     }
     const unsigned long long off = rec_off[r];
     const uint32_t db = db_bits ? rec_db[r] : 0u;
-    uint32_t *it = items + off;
-    if (perm_base) {  // null: the items are already the caller's ids
-        const int32_t *perm = perm_base + dbs[db].item_off;
-        for (int q = 0; q < len; q++) it[q] = (uint32_t)perm[it[q]];
-    }
-    for (int q = 1; q < len; q++) {  // insertion sort (sets are short)
-        const uint32_t v = it[q];
+    uint32_t *const it = items + off;
+    const int32_t *const perm = perm_base ? perm_base + dbs[db].item_off : nullptr;  // null: already the caller's ids
+    // an insertion sort (sets are short), on a local copy where it fits
+    uint32_t loc[PK_LOCAL];
+    uint32_t *const v = len <= PK_LOCAL ? loc : it;
+    for (int q = 0; q < len; q++) {
+        const uint32_t raw = it[q];
+        const uint32_t x = perm ? (uint32_t)__ldg(perm + raw) : raw;
         int z = q - 1;
-        while (z >= 0 && it[z] > v) { it[z + 1] = it[z]; z--; }
-        it[z + 1] = v;
+        while (z >= 0 && v[z] > x) { v[z + 1] = v[z]; z--; }
+        v[z + 1] = x;
     }
     auto emit = [&](int q, unsigned long long v) { keys[(unsigned long long)q * R + r] = v; };
     KeyPack<decltype(emit)> pk(emit);
     if (db_bits) pk.put((unsigned long long)db, db_bits);
     pk.put((unsigned long long)len, 8);
-    for (int q = 0; q < len; q++) pk.put(it[q], bits);
+    for (int q = 0; q < len; q++) {
+        pk.put(v[q], bits);
+        if (v != it) it[q] = v[q];
+    }
     pk.end(kw);
 }
 
@@ -92,7 +98,7 @@ __global__ void prep_keys_kernel(unsigned long long R, const unsigned long long 
 // 36 us of a 10,000 x 169 mine where this takes 10.  Past OC_MAX records the
 // sort's log^2 steps in one CTA cost more than the cluster's launches (1,500
 // sets: 10 us slower).
-constexpr int OC_T = 512, OC_MAX = 1024, OC_KW = 4, OC_LOCAL = 12;
+constexpr int OC_T = 512, OC_MAX = 1024, OC_KW = 4;
 size_t oc_smem(int kw) { return sizeof(unsigned long long) * (size_t)kw * OC_MAX; }
 __global__ void __launch_bounds__(OC_T)
 one_cta_compact_kernel(int R, int R_valid, const unsigned long long *__restrict__ rec_off,
@@ -117,8 +123,8 @@ one_cta_compact_kernel(int R, int R_valid, const unsigned long long *__restrict_
         uint32_t *const it = items + rec_off[r];
         // an insertion sort (sets are short), on a local copy where it fits: in
         // place it is a chain of round trips to global memory
-        uint32_t loc[OC_LOCAL];
-        uint32_t *const v = len <= OC_LOCAL ? loc : it;
+        uint32_t loc[PK_LOCAL];
+        uint32_t *const v = len <= PK_LOCAL ? loc : it;
         for (int q = 0; q < len; q++) {
             const uint32_t raw = it[q];
             const uint32_t x = perm ? (uint32_t)__ldg(perm + raw) : raw;
@@ -182,27 +188,6 @@ one_cta_compact_kernel(int R, int R_valid, const unsigned long long *__restrict_
     if (tid == 0 && R_valid == OC_MAX) out_off[OC_MAX] = total_items;
 }
 
-__global__ void __launch_bounds__(RT)
-rs_hist_kernel(const unsigned long long *__restrict__ key, unsigned long long n, int shift,
-               uint32_t *__restrict__ hist, int ntiles) {
-    __shared__ uint32_t h[256];
-    const int lane = threadIdx.x & 31;
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const unsigned long long t0 = (unsigned long long)blockIdx.x * TILE;
-#pragma unroll
-    for (int i = 0; i < RI; i++) {
-        const unsigned long long e = t0 + i * RT + threadIdx.x;
-        const uint32_t d = e < n ? (uint32_t)((key[e] >> shift) & 255u) : 256u;
-        // one shared atomic per distinct digit of the warp: a digit that
-        // (nearly) every key shares costs 1/32 of the plain count
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        if (d < 256u && lane == __ffs(peers) - 1) atomicAdd(&h[d], (uint32_t)__popc(peers));
-    }
-    __syncthreads();
-    hist[(size_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
-}
-
 // out[i] = word[idx[i]]: one key word in the records' current order.
 __global__ void gather_word_kernel(const unsigned long long *__restrict__ word, const uint32_t *__restrict__ idx,
                                    unsigned long long n, unsigned long long *__restrict__ out) {
@@ -210,130 +195,184 @@ __global__ void gather_word_kernel(const unsigned long long *__restrict__ word, 
     if (i < n) out[i] = word[idx[i]];
 }
 
-// Three-phase exclusive scan for long arrays: per-chunk sums, a scan of the
-// sums in one CTA, and a rescan of every chunk from its base.
-constexpr int SC_T = 1024, SC_I = 8, SC_CHUNK = SC_T * SC_I;
-__global__ void __launch_bounds__(SC_T)
-scan_reduce_kernel(const uint32_t *__restrict__ a, unsigned long long n, uint32_t *__restrict__ part) {
-    __shared__ uint32_t s[SC_T / 32];
-    const unsigned long long b = (unsigned long long)blockIdx.x * SC_CHUNK;
-    uint32_t v = 0;
-#pragma unroll
-    for (int i = 0; i < SC_I; i++) {
-        const unsigned long long e = b + (unsigned long long)i * SC_T + threadIdx.x;
-        if (e < n) v += a[e];
-    }
-    v = warp_sum_u32(v);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
+// ---- the radix sort of a large output ------------------------------------
+// One pass over the keys counts every digit of every word; one launch turns the
+// counts into bases; then each digit is one launch: a tile ranks its keys
+// (warp match, per-warp counts), publishes its digit counts, adds up its
+// predecessors' (decoupled look-back) and scatters.  (A histogram, three scan
+// launches and a scatter per digit took 55 us of 4.2 million records and 25 of
+// 190,000; a digit is now 44 and 7 us and the count 9 and 1 a digit.  With the
+// keys' local sort, whole compactions: 4.2 million sets 2.0 -> 1.66 ms, 640,000
+// sets 0.82 -> 0.40, 190,000 sets 0.85 -> 0.31.)
+constexpr int RS_MAXPASS = 64;   // digits counted in one launch
+
+struct RsPasses {
+    int n;
+    signed char word[RS_MAXPASS];
+    signed char shift[RS_MAXPASS];
+};
+
+__global__ void __launch_bounds__(512)
+rs_count_kernel(const unsigned long long *__restrict__ keys, unsigned long long n, RsPasses ps,
+                unsigned long long *__restrict__ hist) {
+    extern __shared__ uint32_t rs_h[];  // [ps.n][256]
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < ps.n * 256; i += blockDim.x) rs_h[i] = 0;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        uint32_t t = s[threadIdx.x];
-        t = warp_sum_u32(t);
-        if (threadIdx.x == 0) part[blockIdx.x] = t;
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long b = (unsigned long long)blockIdx.x * blockDim.x; b < n; b += stride) {  // block-uniform
+        const unsigned long long r = b + threadIdx.x;
+        int w = -1;
+        unsigned long long k = 0;
+        for (int p = 0; p < ps.n; p++) {
+            if (ps.word[p] != w) {
+                w = ps.word[p];
+                k = r < n ? keys[(unsigned long long)w * n + r] : 0ull;
+            }
+            const uint32_t d = r < n ? (uint32_t)((k >> ps.shift[p]) & 255u) : 256u;
+            // the keys that share lane 0's digit count as one add (sizes, and
+            // the zeros behind short sets, are shared by nearly all), the
+            // others one by one; a match over the warp took 20 cycles a digit
+            const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+            const uint32_t same = __ballot_sync(0xffffffffu, d == d0);
+            if (lane == 0) {
+                if (d < 256u) atomicAdd(&rs_h[p * 256 + d], (uint32_t)__popc(same));
+            } else if (d != d0 && d < 256u) {
+                atomicAdd(&rs_h[p * 256 + d], 1u);
+            }
+        }
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < ps.n * 256; i += blockDim.x)
+        if (rs_h[i]) atomicAdd(&hist[i], (unsigned long long)rs_h[i]);
 }
 
-__global__ void __launch_bounds__(SC_T)
-scan_apply_kernel(uint32_t *__restrict__ a, unsigned long long n, const uint32_t *__restrict__ part) {
-    __shared__ uint32_t s[SC_T / 32 + 1];
+// Exclusive scan of each digit's 256 counts: one CTA per digit.
+__global__ void __launch_bounds__(256)
+rs_base_kernel(unsigned long long *__restrict__ hist) {
+    __shared__ unsigned long long ws[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // thread t owns elements [b + t*SC_I, b + t*SC_I + SC_I) of the chunk
-    const unsigned long long b = (unsigned long long)blockIdx.x * SC_CHUNK + (unsigned long long)threadIdx.x * SC_I;
-    uint32_t v[SC_I], sum = 0;
-#pragma unroll
-    for (int i = 0; i < SC_I; i++) {
-        v[i] = b + i < n ? a[b + i] : 0u;
-        sum += v[i];
-    }
-    uint32_t x = sum;
+    unsigned long long *h = hist + (size_t)blockIdx.x * 256;
+    const unsigned long long v = h[threadIdx.x];
+    unsigned long long x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31) s[warp] = x;
+    if (lane == 31) ws[warp] = x;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t acc = part[blockIdx.x];
-        for (int w = 0; w < SC_T / 32; w++) { const uint32_t t = s[w]; s[w] = acc; acc += t; }
-    }
-    __syncthreads();
-    uint32_t run = s[warp] + x - sum;
-#pragma unroll
-    for (int i = 0; i < SC_I; i++) {
-        if (b + i < n) a[b + i] = run;
-        run += v[i];
-    }
+    unsigned long long before = x - v;
+    for (int w = 0; w < warp; w++) before += ws[w];
+    h[threadIdx.x] = before;
 }
 
-// Exclusive scan of a uint32 array (length <= a few million) in one CTA.
-__global__ void __launch_bounds__(1024)
-scan_single_kernel(uint32_t *__restrict__ a, unsigned long long n, uint32_t *__restrict__ zero,
-                   unsigned long long nzero) {
-    __shared__ uint32_t s[1024];
-    for (unsigned long long i = threadIdx.x; i < nzero; i += 1024) zero[i] = 0u;  // next pass's histogram
-    const unsigned long long seg = (n + 1023) / 1024;
-    const unsigned long long b = threadIdx.x * seg, e = b + seg < n ? b + seg : n;
-    uint32_t sum = 0;
-    for (unsigned long long i = b; i < e; i++) sum += a[i];
-    s[threadIdx.x] = sum;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        uint32_t v = threadIdx.x >= (unsigned)o ? s[threadIdx.x - o] : 0;
-        __syncthreads();
-        s[threadIdx.x] += v;
-        __syncthreads();
-    }
-    uint32_t run = s[threadIdx.x] - sum;
-    for (unsigned long long i = b; i < e; i++) {
-        const uint32_t v = a[i];
-        a[i] = run;
-        run += v;
-    }
-}
+// A tile's published word of one digit: flag in the top two bits (1: its own
+// count, 2: the count up to and including it), the count below.
+constexpr unsigned long long RS_OWN = 1ull << 62, RS_ALL = 2ull << 62, RS_VAL = RS_OWN - 1;
+constexpr unsigned long long RS_WAIT_NS = 2000000000ull;  // 2 s: far above any legitimate wait
 
-__global__ void __launch_bounds__(RT)
-rs_scatter_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *__restrict__ idx_in,
-                  unsigned long long *__restrict__ key_out, uint32_t *__restrict__ idx_out, unsigned long long n,
-                  int shift, const uint32_t *__restrict__ hist, int ntiles, uint32_t *__restrict__ next_hist,
-                  int next_shift) {
-    __shared__ uint32_t base[256];
-    __shared__ uint32_t wc[RT / 32][257];
+template <int NT>
+__global__ void __launch_bounds__(NT)
+rs_digit_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *__restrict__ idx_in,
+                unsigned long long *__restrict__ key_out, uint32_t *__restrict__ idx_out, unsigned long long n,
+                int shift, const unsigned long long *__restrict__ base, unsigned long long *status,
+                unsigned long long *__restrict__ next_status, uint32_t *__restrict__ ticket, int *__restrict__ err) {
+    constexpr int NW = NT / 32;
+    __shared__ uint32_t wc[NW][256];            // per-warp digit counts, then offsets
+    __shared__ unsigned long long dst[256];     // where the tile's keys of a digit go
+    __shared__ uint32_t s_tile;
+    __shared__ int s_bad;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    base[threadIdx.x] = hist[(size_t)threadIdx.x * ntiles + blockIdx.x];
-    const unsigned long long t0 = (unsigned long long)blockIdx.x * TILE;
+    if (threadIdx.x == 0) {
+        // tiles in the order CTAs start: a tile only waits for tiles that run
+        s_tile = atomicAdd(ticket, 1u);
+        s_bad = 0;
+    }
+    for (int i = threadIdx.x; i < NW * 256; i += NT) (&wc[0][0])[i] = 0;
+    __syncthreads();
+    const unsigned long long tile = s_tile;
+    if (threadIdx.x < 256) next_status[tile * 256 + threadIdx.x] = 0ull;  // the next digit's words
+    const unsigned long long t0 = tile * (NT * RI) + (unsigned long long)warp * (32 * RI);
+    unsigned long long k[RI];
+    uint32_t v[RI], rank[RI];
+#pragma unroll
     for (int i = 0; i < RI; i++) {
-        const unsigned long long e = t0 + i * RT + threadIdx.x;
-        const bool valid = e < n;
-        unsigned long long k = 0;
-        uint32_t v = 0, d = 256;
-        if (valid) { k = key_in[e]; v = idx_in[e]; d = (uint32_t)((k >> shift) & 255u); }
-        for (int q = threadIdx.x; q < (RT / 32) * 257; q += RT) (&wc[0][0])[q] = 0;
-        __syncthreads();
+        const unsigned long long e = t0 + i * 32 + lane;
+        k[i] = e < n ? key_in[e] : 0ull;
+        v[i] = e < n ? idx_in[e] : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < RI; i++) {  // stable within the warp: its keys in order
+        const unsigned long long e = t0 + i * 32 + lane;
+        const uint32_t d = e < n ? (uint32_t)((k[i] >> shift) & 255u) : 256u;
         const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t rank = __popc(peers & ((1u << lane) - 1u));
-        if (valid && rank == 0) wc[warp][d] = __popc(peers);
-        __syncthreads();
-        uint32_t off = 0;
-        if (valid) {
-            off = base[d] + rank;
-            for (int w = 0; w < warp; w++) off += wc[w][d];
-            key_out[off] = k;
-            idx_out[off] = v;
+        const uint32_t below = __popc(peers & ((1u << lane) - 1u));
+        uint32_t c = 0;
+        if (d < 256u) c = wc[warp][d];
+        __syncwarp();
+        rank[i] = c + below;
+        if (d < 256u && below == 0) wc[warp][d] = c + (uint32_t)__popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) {
+        const int d = threadIdx.x;
+        uint32_t cnt = 0;
+        for (int w = 0; w < NW; w++) {
+            const uint32_t c = wc[w][d];
+            wc[w][d] = cnt;
+            cnt += c;
         }
-        if (next_hist) {
-            // the next digit's [digit][tile] count, by destination tile: one
-            // atomic per distinct (digit, tile) of the warp
-            const uint32_t key2 = valid ? ((uint32_t)((k >> next_shift) & 255u) << 20) | (off / TILE) : 0xFFFFFFFFu;
-            const uint32_t peers2 = __match_any_sync(0xffffffffu, key2);
-            if (valid && lane == __ffs(peers2) - 1)
-                atomicAdd(&next_hist[(size_t)(key2 >> 20) * ntiles + (key2 & 0xFFFFFu)], (uint32_t)__popc(peers2));
+        volatile unsigned long long *st = status + d;
+        unsigned long long pre = 0;
+        if (tile == 0) {
+            st[0] = RS_ALL | cnt;
+        } else {
+            st[tile * 256] = RS_OWN | cnt;
+            // predecessors LB at a time, their words loaded together: hundreds
+            // of tiles start at once, and one word after another is a round
+            // trip to L2 each
+            constexpr int LB = 8;
+            const unsigned long long t_wait = globaltimer_ns();
+            long long q = (long long)tile - 1;
+            bool more = true;
+            while (more) {
+                unsigned long long x[LB];
+#pragma unroll
+                for (int i = 0; i < LB; i++) x[i] = q - i >= 0 ? (unsigned long long)st[(q - i) * 256] : (2ull << 62);
+#pragma unroll
+                for (int i = 0; i < LB; i++) {
+                    if (!more) break;
+                    while (!(x[i] >> 62)) {
+                        if (globaltimer_ns() - t_wait > RS_WAIT_NS) {
+                            s_bad = 1;
+                            break;
+                        }
+                        x[i] = st[(q - i) * 256];
+                    }
+                    pre += x[i] & RS_VAL;
+                    more = (x[i] >> 62) == 1;  // else everything before is in it (or the wait ran out)
+                }
+                q -= LB;
+            }
+            st[tile * 256] = RS_ALL | (pre + cnt);
         }
-        __syncthreads();
-        uint32_t add = 0;
-        for (int w = 0; w < RT / 32; w++) add += wc[w][threadIdx.x];
-        base[threadIdx.x] += add;
-        __syncthreads();
+        dst[d] = base[d] + pre;
+    }
+    __syncthreads();
+    if (s_bad) {  // reported, nothing scattered
+        if (threadIdx.x == 0) atomicExch(err, 1);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < RI; i++) {
+        const unsigned long long e = t0 + i * 32 + lane;
+        if (e >= n) continue;
+        const uint32_t d = (uint32_t)((k[i] >> shift) & 255u);
+        const unsigned long long o = dst[d] + wc[warp][d] + rank[i];
+        key_out[o] = k[i];
+        idx_out[o] = v[i];
     }
 }
 
@@ -439,6 +478,7 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
     const int bits = bits_for(m_max);
     const int total_bits = db_bits + 8 + bits * lmax;
     const int kw = (int)ceil_div64(total_bits, 64);
+    ctx->compact_waits = false;
     if (n_db == 1 && R <= OC_MAX && kw <= OC_KW && ctx->compact_cluster) {
         FIM_CUDA_TRY(cudaFuncSetAttribute(one_cta_compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)oc_smem(OC_KW)));
@@ -456,14 +496,9 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
     FIM_TRY(fim_reserve(ctx, ctx->idx_b, sizeof(uint32_t) * R));
     FIM_TRY(fim_reserve(ctx, ctx->kv_a, sizeof(unsigned long long) * R));
     FIM_TRY(fim_reserve(ctx, ctx->kv_b, sizeof(unsigned long long) * R));
-    const int ntiles = (int)ceil_div64((int64_t)R, TILE);
-    const unsigned long long nhist = 256ull * (unsigned long long)ntiles;
-    const int nchunks = (int)ceil_div64((int64_t)nhist, SC_CHUNK);
-    // small sorts (one-CTA scans) fold each digit's histogram into the
-    // previous digit's scatter: two histogram buffers, used in turn
-    const bool fuse = nchunks <= 1;
-    FIM_TRY(fim_reserve(ctx, ctx->hist, sizeof(uint32_t) * nhist * (fuse ? 2 : 1)));
-    FIM_TRY(fim_reserve(ctx, ctx->scan_part, sizeof(uint32_t) * (size_t)nchunks));
+    // radix tiles: 512 threads once they still make two waves
+    const bool wide = (int64_t)R >= (int64_t)ctx->num_sms * 2 * 512 * RI;
+    const int64_t ntiles = ceil_div64((int64_t)R, (wide ? 512 : 256) * RI);
     const int nblk = (int)ceil_div64((int64_t)R, ST);
     FIM_TRY(fim_reserve(ctx, ctx->scan_tmp, sizeof(unsigned long long) * (size_t)nblk));
 
@@ -476,10 +511,20 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
         for (int d = 0; d < 8; d++)
             if (word_lo_bit + d * 8 + 8 > key_pad) passes.push_back({w, d * 8});  // skip pure padding
     }
+    const size_t hist_bytes = sizeof(unsigned long long) * 256 * (passes.size() + 2 * (size_t)ntiles) +
+                              sizeof(uint32_t) * passes.size();
     // a small output is sorted in one cluster launch (keys in distributed
     // shared memory) instead of a launch triple per digit
     int cs_cl = 0, cs_cap = 0, cs_per = 0;
     const bool csort = cluster_sort_plan(ctx, R, kw, &cs_cl, &cs_cap, &cs_per) != 0;
+    if (!csort) {
+        FIM_TRY(fim_reserve(ctx, ctx->hist, hist_bytes));
+        FIM_CUDA_TRY(cudaMemsetAsync(ctx->dev_flag.as<int>() + kCompactErr, 0, sizeof(int), st));
+        if (passes.size() > (size_t)RS_MAXPASS / 2)  // more counters than the default shared memory
+            FIM_CUDA_TRY(cudaFuncSetAttribute(rs_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)(sizeof(uint32_t) * 256 * RS_MAXPASS)));
+    }
+    ctx->compact_waits = !csort;
     int enq_rc = FIM_OK;  // a launch that enqueue() could not make
     // The whole pass sequence, enqueued on st.  Returns the kernel count.
     auto enqueue = [&]() -> uint64_t {
@@ -494,52 +539,52 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
             enq_rc = launch_cluster_sort(ctx, keys, R, kw, passes, cs_cl, cs_cap, cs_per, ia, st);
             nk++;
         } else {
-        // LSD: least significant word first; within a word, low digits first.
-        // (word, record) pairs move together, so each word is gathered into
-        // record order once; the least significant word starts in record
-        // order and is read straight from the key array.
-        unsigned long long *ka = ctx->kv_a.as<unsigned long long>(), *kb = ctx->kv_b.as<unsigned long long>();
-        uint32_t *hist = ctx->hist.as<uint32_t>();
-        uint32_t *hist_nxt = fuse ? hist + nhist : nullptr;
-        const unsigned long long *kin = nullptr;
-        for (size_t i = 0; i < passes.size(); i++) {
-            const int w = passes[i].first, shift = passes[i].second;
-            const bool new_word = i == 0 || passes[i - 1].first != w;
-            if (new_word) {
+            // LSD: least significant word first; within a word, low digits first.
+            // (word, record) pairs move together, so each word is gathered into
+            // record order once; the least significant word starts in record
+            // order and is read straight from the key array.
+            unsigned long long *ka = ctx->kv_a.as<unsigned long long>(), *kb = ctx->kv_b.as<unsigned long long>();
+            const int np = (int)passes.size();
+            // hist: [pass][256] counts, then bases; the look-back words, two
+            // digits' in turn; the tickets
+            unsigned long long *const hist = ctx->hist.as<unsigned long long>();
+            unsigned long long *const status = hist + (size_t)np * 256;
+            const size_t words = (size_t)ntiles * 256;
+            uint32_t *const ticket = reinterpret_cast<uint32_t *>(status + 2 * words);
+            cudaMemsetAsync(hist, 0, hist_bytes, st);
+            for (int p0 = 0; p0 < np; p0 += RS_MAXPASS) {
+                RsPasses ps{};
+                ps.n = np - p0 < RS_MAXPASS ? np - p0 : RS_MAXPASS;
+                for (int p = 0; p < ps.n; p++) {
+                    ps.word[p] = (signed char)passes[p0 + p].first;
+                    ps.shift[p] = (signed char)passes[p0 + p].second;
+                }
+                const int64_t blocks = min64(ceil_div64((int64_t)R, 512), (int64_t)ctx->num_sms * 2);
+                rs_count_kernel<<<(unsigned)blocks, 512, sizeof(uint32_t) * 256 * (size_t)ps.n, st>>>(
+                    keys, R, ps, hist + (size_t)p0 * 256);
+                nk++;
+            }
+            rs_base_kernel<<<(unsigned)np, 256, 0, st>>>(hist);
+            nk++;
+            const unsigned long long *kin = nullptr;
+            for (int i = 0; i < np; i++) {
+                const int w = passes[i].first, shift = passes[i].second;
                 if (i == 0) {
                     kin = keys + (size_t)w * R;  // record order: read the key array itself
-                } else {
-                    gather_word_kernel<<<(unsigned)ceil_div64((int64_t)R, 256), 256, 0, st>>>(
-                        keys + (size_t)w * R, ia, R, ka);
+                } else if (passes[i - 1].first != w) {
+                    gather_word_kernel<<<(unsigned)ceil_div64((int64_t)R, 256), 256, 0, st>>>(keys + (size_t)w * R, ia,
+                                                                                            R, ka);
                     nk++;
                     kin = ka;
                 }
-            }
-            const bool next_fused = fuse && i + 1 < passes.size() && passes[i + 1].first == w;
-            if (new_word || !fuse) {
-                rs_hist_kernel<<<ntiles, RT, 0, st>>>(kin, R, shift, hist, ntiles);
+                unsigned long long *kout = (kin == ka) ? kb : ka;
+                (wide ? rs_digit_kernel<512> : rs_digit_kernel<256>)<<<(unsigned)ntiles, wide ? 512 : 256, 0, st>>>(
+                    kin, ia, kout, ib, R, shift, hist + (size_t)i * 256, status + (i & 1) * words,
+                    status + ((i & 1) ^ 1) * words, ticket + i, ctx->dev_flag.as<int>() + kCompactErr);
                 nk++;
-            }  // else: the previous scatter has counted this digit into hist
-            if (nchunks <= 1) {
-                scan_single_kernel<<<1, 1024, 0, st>>>(hist, nhist, next_fused ? hist_nxt : nullptr,
-                                                       next_fused ? nhist : 0ull);
-                nk += 1;
-            } else {
-                uint32_t *part = ctx->scan_part.as<uint32_t>();
-                scan_reduce_kernel<<<nchunks, SC_T, 0, st>>>(hist, nhist, part);
-                scan_single_kernel<<<1, 1024, 0, st>>>(part, (unsigned long long)nchunks, nullptr, 0ull);
-                scan_apply_kernel<<<nchunks, SC_T, 0, st>>>(hist, nhist, part);
-                nk += 3;
+                uint32_t *t = ia; ia = ib; ib = t;
+                kin = kout;
             }
-            unsigned long long *kout = (kin == ka) ? kb : ka;
-            rs_scatter_kernel<<<ntiles, RT, 0, st>>>(kin, ia, kout, ib, R, shift, hist, ntiles,
-                                                     next_fused ? hist_nxt : nullptr,
-                                                     next_fused ? passes[i + 1].second : 0);
-            nk++;
-            uint32_t *t = ia; ia = ib; ib = t;
-            kin = kout;
-            if (fuse) { uint32_t *h = hist; hist = hist_nxt; hist_nxt = h; }
-        }
         }
         unsigned long long *bsum = ctx->scan_tmp.as<unsigned long long>();
         len_block_sums_kernel<<<nblk, ST, 0, st>>>(ia, ctx->rec_len.as<uint32_t>(), R, bsum);
@@ -565,7 +610,6 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
     mix((uint64_t)(uintptr_t)ctx->out_items.p); mix(identity_items ? 0ull : (uint64_t)(uintptr_t)ctx->perm.p);
     mix((uint64_t)(uintptr_t)ctx->dbdesc.p); mix((uint64_t)(uintptr_t)ctx->rec_db.p);
     mix((uint64_t)(uintptr_t)ctx->kv_a.p); mix((uint64_t)(uintptr_t)ctx->kv_b.p);
-    mix((uint64_t)(uintptr_t)ctx->scan_part.p);
     mix(csort ? (uint64_t)(cs_cl * 100000 + cs_per) : 0ull);
     for (int i = 0; i < 2; i++)
         if (ctx->compact_graph_exec[i] && ctx->compact_key[i] == key) {

@@ -508,7 +508,9 @@ proj_gather_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ 
 // counts stay in triple[] (row b of item a: k entries), from which a root reads
 // its candidates.  As tasks of single workers these classes were few and wide:
 // 1,770 of them, up to 58 candidates each, took most of a 50,001 x 60 mine.
-__global__ void __launch_bounds__(256)
+// (Two CTAs an SM: left to itself the compiler may take 164 registers, one CTA,
+// and half as long again.)
+__global__ void __launch_bounds__(256, 2)
 proj_triple_kernel(const ProjItem *__restrict__ items, int mf, const unsigned long long *__restrict__ trip0,
                    const uint32_t *__restrict__ cands, const uint32_t *__restrict__ mat,
                    const uint32_t *__restrict__ pairbits, const DbDesc *__restrict__ dbs, uint32_t thr,

@@ -344,7 +344,9 @@ int fim_rules(fim_ctx *ctx, uint32_t min_conf_ppm, int max_len, uint64_t *n_rule
         FIM_TRY(scan_into(ctx, SetEvals{v.off, max_len}, (unsigned long long)R, ebase));
         unsigned long long E = 0;
         FIM_CUDA_TRY(cudaMemcpyAsync(&E, ebase + R, sizeof(E), cudaMemcpyDeviceToHost, st));
+        FIM_TRY(queue_compact_status(ctx));
         FIM_CUDA_TRY(cudaStreamSynchronize(st));
+        FIM_TRY(compact_status(ctx));
         ctx->rules_evaluated = E;
         if (E > 0) {
             const unsigned long long nw = (E + 31) / 32;

@@ -212,7 +212,6 @@ int fim_merge_results(fim_ctx *ctx, int64_t n_trans, int32_t n_items, int n_part
     FIM_TRY(fim_reserve(ctx, ctx->rec_sup, sizeof(uint32_t) * ctx->rec_cap));
     FIM_TRY(fim_reserve(ctx, ctx->rec_items, sizeof(uint32_t) * ctx->rec_items_cap));
     FIM_TRY(fim_reserve(ctx, ctx->rec_db, sizeof(uint32_t) * ctx->rec_cap));
-    FIM_TRY(fim_reserve(ctx, ctx->dev_flag, 4 * sizeof(int)));
     int *flag = ctx->dev_flag.as<int>();
     FIM_CUDA_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(int), st));
     unsigned long long sb = 0, ib = 0;
@@ -259,7 +258,9 @@ int fim_merge_results(fim_ctx *ctx, int64_t n_trans, int32_t n_items, int n_part
     cudaEventRecord(ctx->ev[3], st);
     FIM_TRY(launch_compact(ctx, R, R, 1, n_items > 0 ? n_items : 1, /*identity_items=*/true));
     cudaEventRecord(ctx->ev[4], st);
+    FIM_TRY(queue_compact_status(ctx));
     FIM_CUDA_TRY(cudaStreamSynchronize(st));
+    FIM_TRY(compact_status(ctx));
     FIM_CUDA_TRY(cudaGetLastError());
     cudaEventElapsedTime(&ctx->stats.ms_compact, ctx->ev[3], ctx->ev[4]);
     ctx->stats.n_sets = R;

@@ -72,3 +72,27 @@ def test_merged_parts(ctx):
         parts.append(fim.fim_fetch_results(ctx))
     fim.fim_merge_results(ctx, c.n, c.m, parts)
     assert len(want) <= 1024 and fim.fim_fetch_results(ctx).sha256() == want.sha256()
+
+
+def test_large_outputs_radix(ctx):
+    # the digit launches: outputs around their tile sizes (2,048 and 4,096
+    # records), many tiles, several key words, and records with holes
+    cases = [(datagen.planted(n=20_000, m=800, n_patterns=60, seed=4), 100),     # 400,000 sets, 3 words
+             (datagen.planted(n=20_000, m=800, n_patterns=60, seed=4), 240),
+             (datagen.random_dense(2_000, 22, 0.6, 4), 60),                      # 1 to 2 words, ~130,000 sets
+             (datagen.from_lists([list(range(17))] * 5, 17), 5)]                 # 2^17 - 1 sets, all of one support
+    fim.fim_set_tuning(ctx, "compact_cluster", 0)
+    try:
+        for c, thr in cases:
+            want = oracle.apriori(c.indptr, c.indices, c.m, thr)
+            fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+            for _ in range(3):  # direct launches, the capture, the replayed graph
+                fim.fim_mine(ctx, thr)
+                assert fim.fim_fetch_results(ctx).sha256() == want.sha256(), (c.n, len(want))
+        for sets in (2047, 2048, 2049, 4095, 4096, 4097, 12_289):
+            c = datagen.from_lists([[i] for i in range(sets)], sets)
+            fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+            fim.fim_mine(ctx, 1)
+            assert fim.fim_fetch_results(ctx).sha256() == oracle.apriori(c.indptr, c.indices, c.m, 1).sha256()
+    finally:
+        fim.fim_set_tuning(ctx, "compact_cluster", 1)
