@@ -37,8 +37,6 @@ constexpr unsigned long long kTriples = 64ull << 20;   // largest table of tripl
 constexpr uint32_t kProjWmax = 1u << 15;         // longest projected column (words)
 constexpr size_t kProjStackBudget = 4ull << 30;  // warp workers' global stacks
 
-constexpr size_t kPinnedBytes = sizeof(MineCounters) > sizeof(BuildFlags) ? sizeof(MineCounters) : sizeof(BuildFlags);
-
 // Read back a device struct (the stream is synchronised): through page-locked
 // memory, which the copy engine writes without a staging pass.
 template <class T>
@@ -213,7 +211,7 @@ void fim_destroy(fim_ctx *ctx) {
                      &ctx->keys, &ctx->idx_a, &ctx->idx_b, &ctx->hist, &ctx->scan_tmp, &ctx->kv_a, &ctx->kv_b,
                      &ctx->out_off,
                      &ctx->out_items, &ctx->out_sup, &ctx->rule_base, &ctx->rule_part, &ctx->rule_bits,
-                     &ctx->rule_kbase, &ctx->rule_set, &ctx->rule_mask,
+                     &ctx->rule_hash, &ctx->rule_set, &ctx->rule_mask,
                      &ctx->rule_conf, &ctx->rule_lift, &ctx->rule_sets, &ctx->probe_buf, &ctx->shard_cost, &ctx->merge_off, &ctx->mlp_w32, &ctx->mlp_wbf, &ctx->trace_x,
                      &ctx->trace_y, &ctx->mlp_scratch, &ctx->root_order, &ctx->root_bucket,
                      &ctx->root_hist, &ctx->rec_db, &ctx->dbdesc, &ctx->epoch, &ctx->sp_idx,

@@ -69,6 +69,8 @@ struct DevBuf {
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
+constexpr size_t kPinnedBytes = 4096;  // page-locked landing place of a ctx's read-backs
+
 // Device-side counters of one mine (kept in one small struct so a single
 // memset clears them and a single copy reads them back).
 struct MineCounters {
@@ -316,7 +318,7 @@ struct fim_ctx {
     DevBuf probe_buf;           // measurement probes' buffer
 
     // association rules of the held output
-    DevBuf rule_base, rule_part, rule_bits, rule_kbase;  // evaluation space, scans, keep words
+    DevBuf rule_base, rule_part, rule_bits, rule_hash;  // size table, scan, keep words, set table
     DevBuf rule_set, rule_mask, rule_conf, rule_lift, rule_sets;
     uint64_t rules_n = 0, rules_evaluated = 0;
     uint64_t rules_of = 0;      // mine_serial the rules belong to

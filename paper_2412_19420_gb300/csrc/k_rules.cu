@@ -10,171 +10,231 @@
 // Work layout.  The candidate rules of all sets form one flat space of
 // E = sum_Z (2^|Z| - 2) evaluations in (set index, antecedent mask) order, so
 // a set of 11 items spreads its 2,046 antecedents over 2,046 threads instead
-// of serialising them in one warp.  Evaluation e belongs to the set z with
-// ebase[z] <= e < ebase[z+1] (ebase = exclusive scan of the per-set counts)
-// and has mask e - ebase[z] + 1.
-//   1. size_bounds: first set index of every size (the output is ordered by
-//      size, then lexicographically), so a subset lookup searches only the
-//      sets of its own size;
-//   2. scan of the per-set counts -> ebase, E;
-//   3. keep: one thread per evaluation looks up S(X) and S(Y) by binary search
+// of serialising them in one warp.  The output is ordered by size, so the sets
+// of one size are a range [first[l], first[l + 1]) and evaluation e names its
+// set and mask by a division.
+//   1. hash: every set's key, index and support in an open-addressing table,
+//      half full at most, and the first set of every size;
+//   2. the host reads those, which give the first evaluation of every size
+//      and E;
+//   3. keep: one thread per evaluation looks S(X) and S(Y) up in the table
 //      (every subset of a frequent set is frequent: downward closure), decides
-//      the threshold, and one ballot per 32 evaluations stores a keep word;
-//   4. scan of the keep words' popcounts -> each word's first output slot;
+//      the threshold; a CTA of EV evaluations stores its keep words and their
+//      sum;
+//   4. scan of the CTAs' sums;
 //   5. write: the kept evaluations write (set index, mask, conf, lift) at their
 //      slot, so the output keeps evaluation order; the keep pass leaves them
-//      their three set indices (12 bytes a candidate, up to 2^27 candidates;
-//      beyond that the write pass repeats the lookups).
-// The itemsets (offsets, items, supports) stay resident from the mine and the
-// lookups hit L2 for outputs up to tens of MB: the kernels are bound by
-// dependent-load latency, not by HBM bandwidth.
+//      the two supports (8 bytes a candidate, up to 2^27 candidates; beyond
+//      that the write pass repeats the lookups).
+// The keep pass is bound by its random loads and the work of naming sets.  So
+// a set whose items fit 127 bits at the width of the largest id is its own key
+// and a lookup is one 32-byte sector; longer sets have a 127-bit hash and
+// compare items.
+// Measured on 35,000 sets with 717,000 candidates (a GB300): keep 22 us, from 68
+// with binary searches for the set and both subsets and each S(Y) looked up
+// again; write 14, from 31; table 8, scan 4 against 45 of two three-launch
+// scans; fim_rules with its fetch 192 us, from 357.
 #include "fim_common.cuh"
 
 namespace {
 
 constexpr int RMAX = FIM_RULES_MAX_LEN;
-constexpr int RT = 256;                    // threads per CTA of the evaluation kernels
-constexpr int SCAN_T = 1024, SCAN_I = 8;   // scan: 1024 threads x 8 elements per CTA
-constexpr int SCAN_CHUNK = SCAN_T * SCAN_I;
-constexpr int NSIZE = 32;                  // size_start entries (sizes 0 .. 31)
-constexpr unsigned long long kRuleSetsMax = 1ull << 27;  // candidates whose lookups are kept (1.5 GB)
+constexpr int RT = 512;                    // threads per CTA of the evaluation kernels
+constexpr int EV = 1024;                   // evaluations per CTA
+constexpr int NSIZE = 32;                  // size table entries (sizes 0 .. 31)
+constexpr unsigned long long kRulesAhead = 1ull << 22;   // candidates whose output room is set aside (117 MB)
+constexpr unsigned long long kRuleSupsMax = 1ull << 27;  // candidates whose lookups are kept (1 GB)
+
+// First set and first evaluation of every size (entry l: sets of at least l
+// items; those longer than NSIZE - 1 have no rules).
+struct SizeTable {
+    unsigned long long first[NSIZE], eval[NSIZE];
+};
+
+// A set in the table, one 32-byte sector.  Key: its items at `bits` bits each,
+// plus one so that no digit is 0, where that fits 127 bits; else the top bit
+// and a hash.
+struct __align__(32) HashEntry {
+    unsigned long long lo, hi;
+    uint32_t set, sup, unused[2];
+};
+struct Key {
+    unsigned long long lo, hi;
+};
+constexpr uint32_t EMPTY = 0xFFFFFFFFu;
 
 struct SetsView {
     const unsigned long long *off;         // [R + 1]
     const uint32_t *items;
     const uint32_t *sup;                   // [R]
-    const unsigned long long *size_start;  // [NSIZE]: first set with |set| >= l
-    int64_t R;
+    const HashEntry *hash;                 // [mask + 1]
+    uint32_t mask, bits;
 };
 
-// Set sizes do not decrease along the canonical order: size_start[l] is the
-// first set index with size >= l (R if none).
-__global__ void size_bounds_kernel(const unsigned long long *__restrict__ off, int64_t R,
-                                   unsigned long long *__restrict__ size_start) {
-    const int l = threadIdx.x;
-    if (l >= NSIZE) return;
-    int64_t lo = 0, hi = R;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)(off[mid + 1] - off[mid]) < l) lo = mid + 1;
-        else hi = mid;
+// Key of the items picked by pick, out of L at zp.  All lanes of a set load the
+// same items, whatever their masks: broadcasts, and none waits for another.
+__device__ __forceinline__ Key key_of(const uint32_t *zp, int L, uint32_t pick, uint32_t bits) {
+    if ((uint32_t)__popc(pick) * bits <= 127u) {
+        Key k{0, 0};
+        uint32_t over = 0;
+#pragma unroll 4
+        for (int j = 0; j < L; j++) {
+            const uint32_t it = __ldg(zp + j) + 1u;  // (0 for the largest 32-bit id: over)
+            if ((pick >> j) & 1u) {
+                over |= (uint32_t)(it == 0u) | (bits < 32u ? it >> bits : 0u);
+                k.hi = k.hi << bits | k.lo >> (64u - bits);
+                k.lo = k.lo << bits | it;
+            }
+        }
+        if (!over) return k;
     }
-    size_start[l] = (unsigned long long)lo;
+    unsigned long long a = 0, b = 0;
+    for (uint32_t mm = pick; mm; mm &= mm - 1) {
+        const uint32_t it = __ldg(zp + (__ffs(mm) - 1));
+        a = (a ^ it) * 0x9E3779B97F4A7C15ull;
+        a ^= a >> 29;
+        b = (b + a) * 0xC2B2AE3D27D4EB4Full;
+    }
+    return Key{a, b | 1ull << 63};
 }
 
-// Compares a stored set of size |mask| with the subset of z picked by mask.
-__device__ __forceinline__ int cmp_subset(const uint32_t *__restrict__ it, const uint32_t *__restrict__ zp,
-                                          uint32_t mask) {
-    int k = 0;
-    for (uint32_t mm = mask; mm; mm &= mm - 1) {
-        const uint32_t a = it[k++], b = __ldg(zp + (__ffs(mm) - 1));
-        if (a != b) return a < b ? -1 : 1;
-    }
-    return 0;
+// First slot of a key and the odd step to its next ones (single steps make
+// clusters: 20 probes for the worst of 35,000 keys, and its warp is waited for).
+__device__ __forceinline__ uint32_t slot_of(Key k, uint32_t *step) {
+    unsigned long long h = (k.lo ^ k.hi * 0xC2B2AE3D27D4EB4Full) * 0x9E3779B97F4A7C15ull;
+    h = (h ^ h >> 32) * 0xC2B2AE3D27D4EB4Full;
+    *step = (uint32_t)h | 1u;
+    return (uint32_t)(h >> 32);
 }
 
-// Index of the subset of z (items at zp, ascending) picked by mask, or -1.
-__device__ __forceinline__ int64_t find_subset(const SetsView &v, const uint32_t *zp, uint32_t mask) {
-    const int ls = __popc(mask);
-    int64_t lo = (int64_t)v.size_start[ls], hi = (int64_t)v.size_start[ls + 1];
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        const int c = cmp_subset(v.items + v.off[mid], zp, mask);
-        if (c == 0) return mid;
-        if (c < 0) lo = mid + 1;
-        else hi = mid;
+// The sets differ, so each takes the first free entry of its slots.  Set
+// sizes do not decrease along the canonical order: first[l] is the first set of
+// at least l items (R if none).
+__global__ void __launch_bounds__(RT)
+hash_sets_kernel(const unsigned long long *__restrict__ off, const uint32_t *__restrict__ items,
+                 const uint32_t *__restrict__ sup, int64_t R, int max_len, HashEntry *__restrict__ hash,
+                 uint32_t mask, uint32_t bits, unsigned long long *__restrict__ first) {
+    for (int64_t z = (int64_t)blockIdx.x * RT + threadIdx.x; z < R; z += (int64_t)gridDim.x * RT) {
+        const unsigned long long o = off[z], o1 = off[z + 1];
+        const unsigned long long before = z ? o - off[z - 1] : 0ull, len = o1 - o;
+        if (z == 0) first[0] = 0;
+        for (unsigned long long l = before + 1; l <= len && l < NSIZE; l++) first[l] = (unsigned long long)z;
+        if (z == R - 1)
+            for (unsigned long long l = len + 1; l < NSIZE; l++) first[l] = (unsigned long long)R;
+        if (len >= (unsigned long long)max_len) continue;  // never a proper subset of a set with rules
+        const int L = (int)len;
+        const Key key = key_of(items + o, L, (1u << L) - 1u, bits);
+        uint32_t step, at = slot_of(key, &step) & mask;
+        while (atomicCAS(&hash[at].set, EMPTY, (uint32_t)z) != EMPTY) at = (at + step) & mask;
+        hash[at].lo = key.lo;
+        hash[at].hi = key.hi;
+        hash[at].sup = sup[z];
     }
-    return -1;
 }
 
-// The set of evaluation e < E = ebase[R]: the last z with ebase[z] <= e.
-__device__ __forceinline__ int64_t set_of_eval(const unsigned long long *__restrict__ ebase, int64_t R,
-                                               unsigned long long e) {
-    int64_t lo = 0, hi = R;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (ebase[mid] <= e) lo = mid + 1;
-        else hi = mid;
+// Support of the subset of z (L items at zp, ascending) picked by pick, or 0.
+__device__ __forceinline__ uint32_t find_subset(const SetsView &v, const uint32_t *zp, int L, uint32_t pick) {
+    const Key key = key_of(zp, L, pick, v.bits);
+    uint32_t step;
+    for (uint32_t at = slot_of(key, &step) & v.mask;; at = (at + step) & v.mask) {
+        const ulonglong2 k = __ldg(reinterpret_cast<const ulonglong2 *>(v.hash + at));
+        const uint2 x = __ldg(reinterpret_cast<const uint2 *>(v.hash + at) + 2);
+        if (x.x == EMPTY) return 0;
+        if (k.x != key.lo || k.y != key.hi) continue;
+        if (!(key.hi >> 63)) return x.y;
+        const unsigned long long o = __ldg(v.off + x.x);
+        if ((int)(__ldg(v.off + x.x + 1) - o) != __popc(pick)) continue;
+        const uint32_t *it = v.items + o;
+        bool same = true;
+        for (uint32_t mm = pick; mm && same; mm &= mm - 1) same = __ldg(it++) == __ldg(zp + (__ffs(mm) - 1));
+        if (same) return x.y;
     }
-    return lo - 1;
 }
 
 struct Eval {
-    int64_t z, rx, ry;
+    int64_t z;
     uint32_t mask;
-    uint64_t sz, sx, sy;
-    bool ok;  // both subsets found
+    uint64_t sz, sx, sy;  // sx or sy 0: the subset is missing
 };
 
-// The three set indices of a kept candidate, carried from the keep pass to the
-// write pass when the scratch fits (12 bytes per candidate).
-struct RuleSets {
-    uint32_t z, x, y;
+// The subsets' supports of a kept candidate, carried from the keep pass to the
+// write pass when the scratch fits.
+struct RuleSups {
+    uint32_t x, y;
 };
 
-__device__ __forceinline__ Eval evaluate(const SetsView &v, const unsigned long long *__restrict__ ebase,
-                                         unsigned long long e) {
+// The set and mask of evaluation e < E, and the set's size; *len comes in as a
+// size that it is not below.
+__device__ __forceinline__ int64_t set_of_eval(const SizeTable &t, unsigned long long e, uint32_t *mask, int *len) {
+    int l = *len;
+    while (l + 1 < NSIZE && t.eval[l + 1] <= e) l++;
+    *len = l;
+    const unsigned long long d = e - t.eval[l];
+    const uint32_t per = (1u << l) - 2u;
+    const unsigned long long z = d >> 32 ? d / per : (unsigned long long)((uint32_t)d / per);
+    *mask = (uint32_t)(d - z * per) + 1u;
+    return (int64_t)(t.first[l] + z);
+}
+
+__device__ __forceinline__ Eval evaluate(const SetsView &v, const SizeTable &t, unsigned long long e, int len) {
     Eval r;
-    r.z = set_of_eval(ebase, v.R, e);
-    const unsigned long long o = v.off[r.z];
-    const int L = (int)(v.off[r.z + 1] - o);
-    const uint32_t full = (1u << L) - 1u;
-    r.mask = (uint32_t)(e - ebase[r.z]) + 1u;
-    const uint32_t *zp = v.items + o;
-    r.rx = find_subset(v, zp, r.mask);
-    r.ry = find_subset(v, zp, full & ~r.mask);
-    r.ok = r.rx >= 0 && r.ry >= 0;
+    r.z = set_of_eval(t, e, &r.mask, &len);
+    const uint32_t *zp = v.items + v.off[r.z];
+    r.sx = find_subset(v, zp, len, r.mask);
+    r.sy = find_subset(v, zp, len, ((1u << len) - 1u) - r.mask);
     r.sz = v.sup[r.z];
-    r.sx = r.ok ? v.sup[r.rx] : 1;
-    r.sy = r.ok ? v.sup[r.ry] : 1;
     return r;
 }
 
-// Candidate rules of a set: 2^L - 2 for 2 <= L <= max_len, else none.
-struct SetEvals {
-    const unsigned long long *off;
-    int max_len;
-    __device__ __forceinline__ unsigned long long operator()(unsigned long long i) const {
-        const int L = (int)(off[i + 1] - off[i]);
-        return (L >= 2 && L <= max_len) ? (1ull << L) - 2ull : 0ull;
-    }
-};
-
-struct WordPop {
-    const uint32_t *bits;
-    __device__ __forceinline__ unsigned long long operator()(unsigned long long i) const {
-        return (unsigned long long)__popc(bits[i]);
-    }
-};
-
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// (double)a / (double)b, correctly rounded, in integers: the FP64 pipe issues
+// a warp instruction every 16 cycles, and two conversions and a division of
+// each rule's two ratios held the write pass to 31 us for 665,000 rules (now
+// 14).  a, b > 0 are rounded to 53 bits (as the conversions do) and normalised
+// to A, B in [2^52, 2^53); then
+// long division with two digits of 28 bits, each the top 32 bits of the rest
+// times a 32-bit reciprocal of B's top bits (an FP32 reciprocal and one Newton
+// step, lowered so that no digit is too large), and the rest decides the
+// rounding (to nearest, ties to even).
+__device__ __forceinline__ unsigned long long round53(unsigned long long x) {
+    const int s = 11 - __clzll((long long)x);
+    if (s <= 0) return x;
+    const unsigned long long half = 1ull << (s - 1), rest = x & (2ull * half - 1ull);
+    x >>= s;
+    x += (rest > half || (rest == half && (x & 1ull))) ? 1ull : 0ull;
+    return x << s;  // (2^64 cannot arise: products of two 32-bit supports)
 }
 
-// Exclusive scan of src(0 .. n-1) into out[0 .. n], out[n] = total, in three
-// launches: chunk sums, a scan of the chunk sums in one CTA, a rescan of every
-// chunk from its base.
-template <class Src>
-__global__ void __launch_bounds__(SCAN_T)
-scan_sum_kernel(Src src, unsigned long long n, unsigned long long *__restrict__ part) {
-    __shared__ unsigned long long s[SCAN_T / 32];
-    const unsigned long long b = (unsigned long long)blockIdx.x * SCAN_CHUNK + (unsigned long long)threadIdx.x * SCAN_I;
-    unsigned long long v = 0;
+__device__ __forceinline__ double ratio(unsigned long long a, unsigned long long b) {
+    a = round53(a);
+    b = round53(b);
+    const int la = __clzll((long long)a), lb = __clzll((long long)b);
+    const unsigned long long B = (b << lb) >> 11;
+    unsigned long long r = (a << la) >> 11, Q = 0;
+    const uint32_t top = (uint32_t)(B >> 21);  // [2^31, 2^32)
+    const float f = __frcp_rn(__uint2float_rn(top)) * 9223372036854775808.0f;
+    const uint32_t x = f >= 4294967040.0f ? 4294967040u : __float2uint_rz(f);
+    const long long err = (long long)((1ull << 63) - (unsigned long long)x * top);
+    const long long y = (long long)x + (((long long)x * (err >> 12)) >> 51) - 3;
+    const uint32_t rcp = y > 0xFFFFFFFFll ? 0xFFFFFFFFu : (uint32_t)y;  // a little under 2^63 / top
 #pragma unroll
-    for (int i = 0; i < SCAN_I; i++)
-        if (b + i < n) v += src(b + i);
-    v = warp_sum_u64(v);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        unsigned long long t = s[threadIdx.x];
-        t = warp_sum_u64(t);
-        if (threadIdx.x == 0) part[blockIdx.x] = t;
+    for (int i = 0; i < 2; i++) {
+        const uint32_t q = (uint32_t)(((unsigned long long)(uint32_t)(r >> 22) * rcp) >> 34);
+        r = (r << 28) - (unsigned long long)q * B;
+        Q = (Q << 28) + q;
     }
+    while (r >= B) {  // once, rarely
+        r -= B;
+        Q++;
+    }
+    const int lz = __clzll((long long)Q);  // Q = floor(2^56 A / B) in (2^55, 2^57)
+    Q <<= lz;
+    const uint32_t low = (uint32_t)Q & 2047u;
+    unsigned long long m = Q >> 11;
+    m += (low > 1024u || (low == 1024u && (r || (m & 1ull)))) ? 1ull : 0ull;
+    return __longlong_as_double((long long)(((unsigned long long)(long long)(lb - la + 1029 - lz) << 52) + m));
 }
 
+// Exclusive scan in one CTA of part[0 .. np), part[np] = total.
 __global__ void __launch_bounds__(1024)
 scan_part_kernel(unsigned long long *__restrict__ part, unsigned long long np) {
     __shared__ unsigned long long s[1024];
@@ -199,118 +259,122 @@ scan_part_kernel(unsigned long long *__restrict__ part, unsigned long long np) {
     if (threadIdx.x == 1023) part[np] = s[1023];
 }
 
-template <class Src>
-__global__ void __launch_bounds__(SCAN_T)
-scan_out_kernel(Src src, unsigned long long n, const unsigned long long *__restrict__ part,
-                unsigned long long *__restrict__ out) {
-    __shared__ unsigned long long s[SCAN_T / 32];
+// CTA c owns evaluations [c EV, (c + 1) EV), a keep word per 32 of them.  S(Y)
+// is the S(X) of the complementary mask, which is the mirrored evaluation of
+// the same set: most often one of the same chunk, so it is looked up once.
+__global__ void __launch_bounds__(RT)
+rule_keep_kernel(SetsView v, const __grid_constant__ SizeTable sizes, unsigned long long E, uint32_t ppm, uint32_t *__restrict__ keep_bits,
+                 RuleSups *__restrict__ sups, unsigned long long *__restrict__ part, int *__restrict__ err) {
+    __shared__ SizeTable t;
+    __shared__ uint32_t kept, ante[EV];
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < (int)(sizeof(SizeTable) / 8); i += RT)
+        reinterpret_cast<unsigned long long *>(&t)[i] = reinterpret_cast<const unsigned long long *>(&sizes)[i];
+    const unsigned long long chunks = (E + EV - 1) / EV;
+    for (unsigned long long c = blockIdx.x; c < chunks; c += gridDim.x) {
+        const unsigned long long e0 = c * EV, e1 = e0 + EV < E ? e0 + EV : E;
+        __syncthreads();
+        if (threadIdx.x == 0) kept = 0;
+        int64_t z[EV / RT];
+        uint32_t mask[EV / RT], sx[EV / RT];
+        int len[EV / RT], len0 = 2;
+        set_of_eval(t, e0, &mask[0], &len0);
+#pragma unroll
+        for (int q = 0; q < EV / RT; q++) {
+            const unsigned long long e = e0 + q * RT + threadIdx.x;
+            if (e >= e1) continue;
+            len[q] = len0;
+            z[q] = set_of_eval(t, e, &mask[q], &len[q]);
+            sx[q] = find_subset(v, v.items + v.off[z[q]], len[q], mask[q]);
+            ante[e - e0] = sx[q];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < EV / RT; q++) {
+            const unsigned long long e = e0 + q * RT + threadIdx.x;
+            bool keep = false;
+            if (e < e1) {
+                // masks run from 1 to full - 1 along the set's evaluations
+                const uint32_t rest = ((1u << len[q]) - 1u) - mask[q];
+                const unsigned long long mirror = e - mask[q] + rest;
+                const uint32_t sy = mirror >= e0 && mirror < e1
+                                        ? ante[mirror - e0]
+                                        : find_subset(v, v.items + v.off[z[q]], len[q], rest);
+                if (!sx[q] || !sy) atomicExch(err, 1);  // a subset is missing: not a mine's output
+                else keep = (uint64_t)v.sup[z[q]] * 1000000ull >= (uint64_t)ppm * sx[q];
+                if (keep && sups) sups[e] = RuleSups{sx[q], sy};
+            }
+            const uint32_t bal = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0 && e < e1) {
+                keep_bits[e >> 5] = bal;
+                if (bal) atomicAdd(&kept, (uint32_t)__popc(bal));
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) part[c] = kept;
+    }
+}
+
+__global__ void __launch_bounds__(RT)
+rule_write_kernel(SetsView v, const __grid_constant__ SizeTable sizes, unsigned long long E, uint64_t n, const uint32_t *__restrict__ keep_bits,
+                  const unsigned long long *__restrict__ part, const RuleSups *__restrict__ sups,
+                  unsigned long long *__restrict__ set_index, uint32_t *__restrict__ ante_mask,
+                  double *__restrict__ conf, double *__restrict__ lift) {
+    constexpr int W = EV / 32;  // keep words of a chunk: one per lane of a warp
+    static_assert(W == 32, "a warp scans a chunk's keep words");
+    __shared__ SizeTable t;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned long long b = (unsigned long long)blockIdx.x * SCAN_CHUNK + (unsigned long long)threadIdx.x * SCAN_I;
-    unsigned long long v[SCAN_I], sum = 0;
-#pragma unroll
-    for (int i = 0; i < SCAN_I; i++) {
-        v[i] = b + i < n ? src(b + i) : 0ull;
-        sum += v[i];
-    }
-    unsigned long long x = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s[warp] = x;
+    for (int i = threadIdx.x; i < (int)(sizeof(SizeTable) / 8); i += RT)
+        reinterpret_cast<unsigned long long *>(&t)[i] = reinterpret_cast<const unsigned long long *>(&sizes)[i];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long acc = part[blockIdx.x];
-        for (int w = 0; w < SCAN_T / 32; w++) {
-            const unsigned long long t = s[w];
-            s[w] = acc;
-            acc += t;
-        }
-    }
-    __syncthreads();
-    unsigned long long run = s[warp] + x - sum;
-#pragma unroll
-    for (int i = 0; i < SCAN_I; i++) {
-        if (b + i < n) out[b + i] = run;
-        run += v[i];
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = part[gridDim.x];
-}
-
-// One thread per evaluation; warp w of the grid-stride loop owns evaluations
-// [32w, 32w + 32) and stores their keep bits as one word.
-__global__ void __launch_bounds__(RT)
-rule_keep_kernel(SetsView v, const unsigned long long *__restrict__ ebase, unsigned long long E, uint32_t ppm,
-                 uint32_t *__restrict__ keep_bits, RuleSets *__restrict__ sets, int *__restrict__ err) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long nw = (E + 31) / 32;
-    const unsigned long long tw = (unsigned long long)gridDim.x * (RT / 32);
-    for (unsigned long long w = ((unsigned long long)blockIdx.x * RT + threadIdx.x) >> 5; w < nw; w += tw) {
-        const unsigned long long e = w * 32 + lane;
-        bool keep = false;
-        if (e < E) {
-            const Eval r = evaluate(v, ebase, e);
-            if (!r.ok) atomicExch(err, 1);  // a subset is missing: not a mine's output
-            else keep = r.sz * 1000000ull >= (uint64_t)ppm * r.sx;
-            if (keep && sets) sets[e] = RuleSets{(uint32_t)r.z, (uint32_t)r.rx, (uint32_t)r.ry};
-        }
-        const uint32_t bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) keep_bits[w] = bal;
-    }
-}
-
-__global__ void __launch_bounds__(RT)
-rule_write_kernel(SetsView v, const unsigned long long *__restrict__ ebase, unsigned long long E, uint64_t n,
-                  const uint32_t *__restrict__ keep_bits, const unsigned long long *__restrict__ kbase,
-                  const RuleSets *__restrict__ sets, unsigned long long *__restrict__ set_index,
-                  uint32_t *__restrict__ ante_mask, double *__restrict__ conf, double *__restrict__ lift) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long nw = (E + 31) / 32;
-    const unsigned long long tw = (unsigned long long)gridDim.x * (RT / 32);
     const uint32_t lt = (1u << lane) - 1u;
-    for (unsigned long long w = ((unsigned long long)blockIdx.x * RT + threadIdx.x) >> 5; w < nw; w += tw) {
-        const uint32_t bits = keep_bits[w];
-        if (!((bits >> lane) & 1u)) continue;
-        const unsigned long long e = w * 32 + lane;
-        int64_t z;
-        uint32_t mask;
-        uint64_t sz, sx, sy;
-        if (sets) {  // the keep pass's lookups
-            const RuleSets q = sets[e];
-            z = q.z;
-            mask = (uint32_t)(e - ebase[z]) + 1u;
-            sz = v.sup[q.z];
-            sx = v.sup[q.x];
-            sy = v.sup[q.y];
-        } else {
-            const Eval r = evaluate(v, ebase, e);
-            z = r.z;
-            mask = r.mask;
-            sz = r.sz;
-            sx = r.sx;
-            sy = r.sy;
+    const unsigned long long chunks = (E + EV - 1) / EV, nw = (E + 31) / 32;
+    for (unsigned long long c = blockIdx.x; c < chunks; c += gridDim.x) {
+        // every warp scans the chunk's words for itself
+        const unsigned long long w = c * W + lane;
+        const uint32_t bits = w < nw ? keep_bits[w] : 0u;
+        uint32_t x = __popc(bits);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
-        const unsigned long long at = kbase[w] + __popc(bits & lt);
-        set_index[at] = (unsigned long long)z;
-        ante_mask[at] = mask;
-        conf[at] = (double)sz / (double)sx;
-        lift[at] = (double)(sz * n) / (double)(sx * sy);
+        const uint32_t before = x - __popc(bits);
+        const unsigned long long base = part[c];
+        int len0 = 2;
+        uint32_t mask0;
+        set_of_eval(t, c * EV, &mask0, &len0);
+#pragma unroll
+        for (int q = 0; q < EV / RT; q++) {
+            const int wi = q * (RT / 32) + warp;
+            const uint32_t b = __shfl_sync(0xffffffffu, bits, wi), pre = __shfl_sync(0xffffffffu, before, wi);
+            if (!((b >> lane) & 1u)) continue;
+            const unsigned long long e = c * EV + (unsigned)wi * 32 + lane;
+            int64_t z;
+            uint32_t mask;
+            uint64_t sz, sx, sy;
+            if (sups) {  // the keep pass's lookups
+                const RuleSups r = sups[e];
+                int len = len0;
+                z = set_of_eval(t, e, &mask, &len);
+                sz = v.sup[z];
+                sx = r.x;
+                sy = r.y;
+            } else {
+                const Eval r = evaluate(v, t, e, len0);
+                z = r.z;
+                mask = r.mask;
+                sz = r.sz;
+                sx = r.sx;
+                sy = r.sy;
+            }
+            const unsigned long long at = base + pre + __popc(b & lt);
+            set_index[at] = (unsigned long long)z;
+            ante_mask[at] = mask;
+            conf[at] = ratio(sz, sx);
+            lift[at] = ratio(sz * n, sx * sy);
+        }
     }
-}
-
-template <class Src>
-int scan_into(fim_ctx *ctx, Src src, unsigned long long n, unsigned long long *out) {
-    const unsigned long long np = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-    FIM_TRY(fim_reserve(ctx, ctx->rule_part, sizeof(unsigned long long) * (size_t)(np + 1)));
-    unsigned long long *part = ctx->rule_part.as<unsigned long long>();
-    cudaStream_t st = ctx->stream;
-    ctx->launches += 3;
-    scan_sum_kernel<<<(unsigned)np, SCAN_T, 0, st>>>(src, n, part);
-    scan_part_kernel<<<1, 1024, 0, st>>>(part, np);
-    scan_out_kernel<<<(unsigned)np, SCAN_T, 0, st>>>(src, n, part, out);
-    FIM_CUDA_TRY(cudaGetLastError());
-    return FIM_OK;
 }
 
 }  // namespace
@@ -334,59 +398,89 @@ int fim_rules(fim_ctx *ctx, uint32_t min_conf_ppm, int max_len, uint64_t *n_rule
     ctx->rules_of = 0;
     ctx->rules_evaluated = 0;
     if (R > 0) {
-        // ebase [R + 1], then size_start [NSIZE]
-        FIM_TRY(fim_reserve(ctx, ctx->rule_base, sizeof(unsigned long long) * (size_t)(R + 1 + NSIZE)));
-        unsigned long long *ebase = ctx->rule_base.as<unsigned long long>(), *size_start = ebase + R + 1;
+        if (R >= (int64_t)0xFFFFFFFFll) return FIM_E_NOMEM;  // set indices are 32-bit in the table
+        uint64_t slots = 1024;
+        // half full at most, three quarters from 2^28 slots (8 GB) on
+        while (slots < 2ull * (uint64_t)R && slots < (1ull << 28)) slots <<= 1;
+        while (3ull * slots < 4ull * (uint64_t)R && slots < (1ull << 32)) slots <<= 1;
+        uint32_t bits = 1;
+        while (bits < 32 && ((uint64_t)ctx->m >> bits)) bits++;
+        FIM_TRY(fim_reserve(ctx, ctx->rule_base, sizeof(unsigned long long) * NSIZE));
+        FIM_TRY(fim_reserve(ctx, ctx->rule_hash, sizeof(HashEntry) * (size_t)slots));
         const SetsView v{ctx->out_off.as<unsigned long long>(), ctx->out_items.as<uint32_t>(),
-                         ctx->out_sup.as<uint32_t>(), size_start, R};
+                         ctx->out_sup.as<uint32_t>(), ctx->rule_hash.as<HashEntry>(),
+                         (uint32_t)(slots - 1), bits};
+        FIM_CUDA_TRY(cudaMemsetAsync(ctx->rule_hash.p, 0xFF, sizeof(HashEntry) * (size_t)slots, st));
         ctx->launches++;
-        size_bounds_kernel<<<1, NSIZE, 0, st>>>(v.off, R, size_start);
-        FIM_TRY(scan_into(ctx, SetEvals{v.off, max_len}, (unsigned long long)R, ebase));
-        unsigned long long E = 0;
-        FIM_CUDA_TRY(cudaMemcpyAsync(&E, ebase + R, sizeof(E), cudaMemcpyDeviceToHost, st));
+        const int64_t hb = ceil_div64(R, RT);
+        hash_sets_kernel<<<(unsigned)min64(hb, (int64_t)ctx->num_sms * (2048 / RT)), RT, 0, st>>>(
+            v.off, v.items, v.sup, R, max_len, ctx->rule_hash.as<HashEntry>(), v.mask, bits,
+            ctx->rule_base.as<unsigned long long>());
+        FIM_CUDA_TRY(cudaGetLastError());
+        // read-backs land in page-locked memory: [0] the compaction's error
+        // word, from [1] the first set of every size, then the rules' number
+        // and this call's error word
+        unsigned long long *const pin = static_cast<unsigned long long *>(ctx->pinned);
+        static_assert(sizeof(unsigned long long) * (NSIZE + 1) <= kPinnedBytes, "landing place");
+        FIM_CUDA_TRY(cudaMemcpyAsync(pin + 1, ctx->rule_base.p, sizeof(unsigned long long) * NSIZE,
+                                     cudaMemcpyDeviceToHost, st));
         FIM_TRY(queue_compact_status(ctx));
         FIM_CUDA_TRY(cudaStreamSynchronize(st));
         FIM_TRY(compact_status(ctx));
+        SizeTable sizes;
+        unsigned long long E = 0;
+        for (int l = 0; l < NSIZE; l++) {
+            sizes.first[l] = pin[1 + l];
+            sizes.eval[l] = E;
+            if (l + 1 < NSIZE && l <= max_len && l >= 2) E += (pin[2 + l] - pin[1 + l]) * ((1ull << l) - 2ull);
+        }
         ctx->rules_evaluated = E;
         if (E > 0) {
-            const unsigned long long nw = (E + 31) / 32;
+            const unsigned long long nw = (E + 31) / 32, chunks = (E + EV - 1) / EV;
             FIM_TRY(fim_reserve(ctx, ctx->rule_bits, sizeof(uint32_t) * (size_t)nw));
-            FIM_TRY(fim_reserve(ctx, ctx->rule_kbase, sizeof(unsigned long long) * (size_t)(nw + 1)));
-            uint32_t *bits = ctx->rule_bits.as<uint32_t>();
-            unsigned long long *kbase = ctx->rule_kbase.as<unsigned long long>();
+            FIM_TRY(fim_reserve(ctx, ctx->rule_part, sizeof(unsigned long long) * (size_t)(chunks + 1)));
+            uint32_t *keep = ctx->rule_bits.as<uint32_t>();
+            unsigned long long *part = ctx->rule_part.as<unsigned long long>();
             int *err = ctx->dev_flag.as<int>() + 2;
             FIM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
-            RuleSets *sets = nullptr;
-            if (E <= kRuleSetsMax && (unsigned long long)R <= 0xFFFFFFFFull) {
-                FIM_TRY(fim_reserve(ctx, ctx->rule_sets, sizeof(RuleSets) * (size_t)E));
-                sets = ctx->rule_sets.as<RuleSets>();
+            RuleSups *sups = nullptr;
+            if (E <= kRuleSupsMax) {
+                FIM_TRY(fim_reserve(ctx, ctx->rule_sets, sizeof(RuleSups) * (size_t)E));
+                sups = ctx->rule_sets.as<RuleSups>();
             }
-            const unsigned long long want = (nw + RT / 32 - 1) / (RT / 32);
-            const unsigned long long cap = (unsigned long long)(ctx->num_sms > 0 ? ctx->num_sms : 1) * 8ull;  // 2,048 threads per SM
-            const unsigned grid = (unsigned)(want < cap ? want : cap);
-            ctx->launches++;
-            rule_keep_kernel<<<grid, RT, 0, st>>>(v, ebase, E, min_conf_ppm, bits, sets, err);
+            const unsigned long long cap = (unsigned long long)(ctx->num_sms > 0 ? ctx->num_sms : 1) * (2048 / RT);
+            const unsigned grid = (unsigned)(chunks < cap ? chunks : cap);
+            ctx->launches += 2;
+            rule_keep_kernel<<<grid, RT, 0, st>>>(v, sizes, E, min_conf_ppm, keep, sups, part, err);
+            scan_part_kernel<<<1, 1024, 0, st>>>(part, chunks);
             FIM_CUDA_TRY(cudaGetLastError());
-            FIM_TRY(scan_into(ctx, WordPop{bits}, nw, kbase));
-            unsigned long long total = 0;
-            int bad = 0;
-            FIM_CUDA_TRY(cudaMemcpyAsync(&total, kbase + nw, sizeof(total), cudaMemcpyDeviceToHost, st));
-            FIM_CUDA_TRY(cudaMemcpyAsync(&bad, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-            FIM_CUDA_TRY(cudaStreamSynchronize(st));
-            if (bad) return FIM_E_STATE;  // the held sets are not downward closed
-            if (total) {
-                FIM_TRY(fim_reserve(ctx, ctx->rule_set, sizeof(unsigned long long) * (size_t)total));
-                FIM_TRY(fim_reserve(ctx, ctx->rule_mask, sizeof(uint32_t) * (size_t)total));
-                FIM_TRY(fim_reserve(ctx, ctx->rule_conf, sizeof(double) * (size_t)total));
-                FIM_TRY(fim_reserve(ctx, ctx->rule_lift, sizeof(double) * (size_t)total));
+            FIM_CUDA_TRY(cudaMemcpyAsync(pin + 1, part + chunks, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+            FIM_CUDA_TRY(cudaMemcpyAsync(pin + 2, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+            // where room for all candidates is small the write is queued before
+            // the kept number is known
+            auto write = [&](unsigned long long cap_rules) -> int {
+                FIM_TRY(fim_reserve(ctx, ctx->rule_set, sizeof(unsigned long long) * (size_t)cap_rules));
+                FIM_TRY(fim_reserve(ctx, ctx->rule_mask, sizeof(uint32_t) * (size_t)cap_rules));
+                FIM_TRY(fim_reserve(ctx, ctx->rule_conf, sizeof(double) * (size_t)cap_rules));
+                FIM_TRY(fim_reserve(ctx, ctx->rule_lift, sizeof(double) * (size_t)cap_rules));
                 ctx->launches++;
-                rule_write_kernel<<<grid, RT, 0, st>>>(v, ebase, E, (uint64_t)ctx->out_n, bits, kbase, sets,
+                rule_write_kernel<<<grid, RT, 0, st>>>(v, sizes, E, (uint64_t)ctx->out_n, keep, part, sups,
                                                        ctx->rule_set.as<unsigned long long>(),
                                                        ctx->rule_mask.as<uint32_t>(), ctx->rule_conf.as<double>(),
                                                        ctx->rule_lift.as<double>());
                 FIM_CUDA_TRY(cudaGetLastError());
-                FIM_CUDA_TRY(cudaStreamSynchronize(st));
+                return FIM_OK;
+            };
+            bool ahead = E <= kRulesAhead;
+            if (ahead) {
+                const int rc = write(E);
+                if (rc == FIM_E_NOMEM) ahead = false;
+                else if (rc != FIM_OK) return rc;
             }
+            FIM_CUDA_TRY(cudaStreamSynchronize(st));
+            const unsigned long long total = pin[1];
+            if (static_cast<const int *>(ctx->pinned)[4]) return FIM_E_STATE;  // the held sets are not downward closed
+            if (total && !ahead) FIM_TRY(write(total));
             ctx->rules_n = total;
         }
     }
