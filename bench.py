@@ -769,7 +769,17 @@ def _roofline(st, avg, csr, workload, probes):
     hbm, bf16, bf16_s, src = _peaks()
     dom = max(("ms_pairs", "ms_dfs", "ms_compact", "ms_build"), key=lambda p: avg[p])
     if dom == "ms_dfs":
-        roof = _dfs_roofline(st, avg[dom], workload, probes)
+        # warp workers on projected columns, else CTA workers
+        roof = _dfs_roofline(st, avg[dom], workload, probes,
+                             "dfs_proj_kernel" if st["dfs_workers"] > 1024 else "dfs_kernel")
+    elif dom == "ms_pairs" and st["pair_path"] == 1 and st["n_frequent_items"] > 256:
+        # the rows' pairs as atomics in L2 beside the most frequent items'
+        # tensor-core block: the packed rows (16-bit ids, 32-bit offsets) and
+        # the counts, which its atomics bound, not these bytes
+        nbytes = 2 * csr.indices.size + 4 * (csr.n + 1) + 4 * st["n_frequent_items"] ** 2
+        ach = nbytes / (avg[dom] / 1000) / 1e9
+        roof = {"kernel": "pairs_rows_kernel", "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
+                "frac": ach / hbm, "traffic": _kernel_traffic("pairs_rows_kernel", workload)}
     elif dom == "ms_pairs" and st["pair_path"] == 1:
         fl = 2.0 * st["supports_pairs"] * csr.n
         ach = fl / (avg[dom] / 1000) / 1e12
@@ -920,8 +930,8 @@ def main():
         rules = {"min_conf_ppm": args.rules_ppm, "n_rules": int(n_rules), "antecedents_evaluated": evaluated,
                  "ms": round(ms_r, 4), "rules_per_s": n_rules / (ms_r / 1000),
                  "antecedents_per_s": evaluated / (ms_r / 1000),
-                 "timing": "host wall clock around fim_rules (keep and write passes, two scans, "
-                           "three host syncs), median"}
+                 "timing": "host wall clock around fim_rules (set table, keep and write "
+                           "passes, two host syncs), median"}
 
     # ---- roofline of the dominant phase ---------------------------------
     avg = {p: phase[p] / args.steps for p in phase}

@@ -430,8 +430,6 @@ int launch_emit_singletons(fim_ctx *ctx, MineCounters *d_ctr);
 // few items: counters cleared, ids, singletons and the table in one launch
 bool mine_begin_fits(int m);
 int launch_mine_begin(fim_ctx *ctx, const DbDesc &d, MineCounters *d_ctr);
-int launch_max_row_freq(fim_ctx *ctx, const int64_t *d_indptr, const int32_t *d_indices,
-                        MineCounters *d_ctr);
 
 // k_pairs.cu
 int launch_pairs_popc(fim_ctx *ctx);
