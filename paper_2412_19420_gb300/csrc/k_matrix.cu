@@ -5,9 +5,8 @@
 // and a range of IB items.  Each warp streams a 32-row group's elements
 // (coalesced) and ORs every (transaction, item) pair into a shared-memory
 // tile with atomicOr -- OR makes repeated items idempotent, which is the set
-// membership of Eq. 1 -- and the tile goes out as WB-word (64-byte) runs of
-// each item column with 16-byte stores.  A 64-byte run keeps the tile at
-// 64 KB for 1,024 items, so several CTAs share an SM.  The CTA also validates
+// membership of Eq. 1 -- and the tile goes out as WB-word (64- or 32-byte)
+// runs of each item column with 16-byte stores.  The CTA also validates
 // its slice of the CSR (monotone indptr, items in [0, m)).  CMP: the CSR is
 // compact (uint32 row offsets, uint16 item ids) instead of int64 / int32.
 #include <type_traits>
@@ -16,26 +15,26 @@
 
 namespace {
 
-constexpr int WB = 16;          // words per CTA tile row (64 bytes)
-constexpr int BUILD_THREADS = 512;
-
-template <bool CMP>
-__global__ void __launch_bounds__(BUILD_THREADS)
+// WB: words per CTA tile row; T: threads; T / 32 / WB warps share a 32-row group.
+template <bool CMP, int WB, int T>
+__global__ void __launch_bounds__(T)
 build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__ indices_v,
-                     int64_t n, int32_t m, int64_t nnz, int64_t nwp, int ib, int64_t blk0,
+                     int64_t n, int32_t m, int64_t nnz, int64_t nwp, int ib, int ms, int64_t blk0,
                      uint32_t *__restrict__ bm, uint32_t *__restrict__ sup, BuildFlags *__restrict__ flags,
                      RowCopy rows) {
     using Off = typename std::conditional<CMP, uint32_t, int64_t>::type;
     using Id = typename std::conditional<CMP, unsigned short, int32_t>::type;
     const Off *const indptr = static_cast<const Off *>(indptr_v);
     const Id *const indices = static_cast<const Id *>(indices_v);
-    // [WB][ib + 1], word-major and padded: the 32 rows of a warp's group share
+    // [WB][ms], word-major and padded: the 32 rows of a warp's group share
     // their word, so their items' bits spread over the banks
     extern __shared__ __align__(16) uint32_t tile[];
     __shared__ int s_max;
     __shared__ unsigned long long s_pairs;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int ms = ib + 1;
+    constexpr int SPLIT = T / 32 / WB;
+    static_assert(T == 32 * WB * SPLIT && (WB == 8 || WB == 16), "whole warps per row group");
+    const int sub = warp % SPLIT;  // of the warps sharing a group
     const int64_t w0 = (blk0 + (int64_t)blockIdx.x) * WB;
     const int i0 = blockIdx.y * ib;
     const int icount = min(ib, m - i0);
@@ -52,7 +51,7 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
     const bool copy = first && (uint64_t)nnz <= rows.cap;
     if (first && blk0 == 0 && blockIdx.x == 0 && threadIdx.x == 0) flags->nnz = nnz;
 
-    for (int k = threadIdx.x; k < WB * ms; k += blockDim.x) tile[k] = 0u;
+    for (int k = threadIdx.x; k < WB / 4 * ms; k += T) reinterpret_cast<uint4 *>(tile)[k] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) {
         s_max = 0;
         s_pairs = 0;
@@ -61,7 +60,7 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
     // warp w takes 32-row groups: lane i holds the group's start of row i, the
     // warp streams the group's elements 32 at a time (coalesced) and each
     // element finds its row by a binary search over the lanes' starts
-    for (int64_t rb = t0 + 32 * warp; rb < t1; rb += 32 * (int64_t)(blockDim.x >> 5)) {
+    for (int64_t rb = t0 + 32 * (warp / SPLIT); rb < t1; rb += 32 * WB) {
         const int nr = (int)min64(32, t1 - rb);
         const int64_t off = (int64_t)indptr[rb + (lane < nr ? lane : nr)];
         const int64_t e_end = (int64_t)indptr[rb + nr];
@@ -69,7 +68,7 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         if (lane == nr - 1) off_next = e_end;
         if (lane < nr) {
             if (off_next < off || off < 0 || off_next > nnz) bad = 1;
-            else {
+            else if (sub == 0) {
                 const int64_t len = off_next - off;
                 my_max = max(my_max, (int)min64(len, 1 << 30));
                 my_pairs += (unsigned long long)len * (unsigned long long)(len - 1) / 2;
@@ -86,16 +85,18 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         const bool dense = e_end - e_begin < (1ll << 30) && !__any_sync(0xffffffffu, lane < nr && off_next == off);
         const int ar = dense ? (int)(off - e_begin) : 0;
         int before = -1;  // rows begun before the chunk, less one
-        for (int64_t e0 = e_begin; e0 < e_end; e0 += 32) {
+        for (int64_t e0 = e_begin + 32 * sub; e0 < e_end; e0 += 32 * SPLIT) {
             const int64_t e = e0 + lane;
             const bool v = e < e_end;
             const int32_t it = v ? (int32_t)indices[e] : 0;
             int r = 0;  // largest r < nr with start(r) <= e
             if (dense) {
-                const unsigned in = (unsigned)(ar - (int)(e0 - e_begin));
+                const int at = (int)(e0 - e_begin);
+                const unsigned in = (unsigned)(ar - at);
+                if (SPLIT > 1) before = __popc(__ballot_sync(0xffffffffu, lane < nr && ar < at)) - 1;
                 const uint32_t heads = __reduce_or_sync(0xffffffffu, lane < nr && in < 32u ? 1u << in : 0u);
                 r = before + __popc(heads & (0xFFFFFFFFu >> (31 - lane)));
-                before += __popc(heads);
+                if (SPLIT == 1) before += __popc(heads);
             } else {
 #pragma unroll
                 for (int step = 16; step > 0; step >>= 1) {
@@ -126,10 +127,10 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         atomicMax(&flags->max_len, s_max);
         atomicAdd(&flags->row_pairs, s_pairs);
     }
-    // write-out: 16-byte stores, four consecutive threads per 64-byte row; the
-    // row's popcount rides along into S(I_j) (Eq. 3).  (A pass of its own over
+    // write-out: 16-byte stores, WB / 4 consecutive threads per column; the
+    // column's popcount rides along into S(I_j) (Eq. 3).  (A pass of its own over
     // the columns read all of them back: 0.9 ms on 10^7 x 5,000.)
-    for (int b = 0; b < icount * (WB / 4); b += blockDim.x) {  // block-uniform trips
+    for (int b = 0; b < icount * (WB / 4); b += T) {  // block-uniform trips
         const int k = b + threadIdx.x;
         const int r = k / (WB / 4), c = k % (WB / 4);
         uint32_t cnt = 0;
@@ -140,7 +141,7 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
             cnt = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
         }
         cnt += __shfl_xor_sync(0xffffffffu, cnt, 1);
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, 2);
+        if (WB == 16) cnt += __shfl_xor_sync(0xffffffffu, cnt, 2);
         if (c == 0 && cnt) atomicAdd(&sup[i0 + r], cnt);
     }
 }
@@ -263,13 +264,25 @@ int launch_mine_begin(fim_ctx *ctx, const DbDesc &d, MineCounters *d_ctr) {
 
 int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indices, int64_t nnz,
                          const void *h_indptr, const void *h_indices, bool cmp) {
-    auto kern = cmp ? build_bitmaps_kernel<true> : build_bitmaps_kernel<false>;
     const size_t ib_bytes = csr_id_bytes(cmp);
+    // Up to 1,024 items: 64-byte runs, several CTAs an SM.  More: 32-byte runs of
+    // up to 7,200 items and one CTA an SM, four warps to a row group, so that
+    // every id is read once (blocks of 1,024 items read the ids m / 1,024
+    // times): 10^7 x 5,000 3.13 -> 2.92 ms, 100,000 x 2,000 75 -> 67 us from
+    // device memory; from mapped host memory the ids cross the link once.  (512
+    // threads 3.25 ms, two blocks of 2,500 items 2.95, two CTAs an SM 3.85.)
+    const bool wide = ctx->m > 1024;
+    const int WB = wide ? 8 : 16, T = wide ? 1024 : 512, most = wide ? 7200 : 1024;
+    auto kern = cmp ? build_bitmaps_kernel<true, 16, 512> : build_bitmaps_kernel<false, 16, 512>;
+    if (wide) kern = cmp ? build_bitmaps_kernel<true, 8, 1024> : build_bitmaps_kernel<false, 8, 1024>;
     const int64_t nblk = ctx->nwp / WB;
-    int ib = ctx->m < 1024 ? ctx->m : 1024;
+    const int niblk = (int)ceil_div64(ctx->m > 0 ? ctx->m : 1, most);
+    int ib = (int)ceil_div64(ctx->m, niblk);
     if (ib < 1) ib = 1;
-    const int niblk = (int)ceil_div64(ctx->m > 0 ? ctx->m : 1, ib);
-    const size_t smem = (size_t)(ib + 1) * WB * sizeof(uint32_t);
+    // the write-out's four (two) threads of a column on banks of their own
+    // (10^7 x 5,000 3.31 -> 3.13 ms)
+    const int ms = ib + ((WB == 16 ? 2 : 4) - ib % 8 + 8) % 8;
+    const size_t smem = (size_t)ms * WB * sizeof(uint32_t);
     FIM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     BuildFlags *flags = ctx->dev_flag.as<BuildFlags>();
     cudaStream_t st = ctx->stream;
@@ -329,7 +342,7 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
         }
         dim3 grid((unsigned)(b1 - b0), (unsigned)niblk);
         ctx->launches++;
-        kern<<<grid, BUILD_THREADS, smem, st>>>(d_indptr, d_indices, ctx->n, ctx->m, nnz, ctx->nwp, ib, b0,
+        kern<<<grid, T, smem, st>>>(d_indptr, d_indices, ctx->n, ctx->m, nnz, ctx->nwp, ib, ms, b0,
                                                 ctx->bm.as<uint32_t>(), ctx->item_sup.as<uint32_t>(), flags, rows);
         FIM_CUDA_TRY(cudaGetLastError());
     }
