@@ -36,9 +36,9 @@
 // instead of 4 CTAs); 10^7 x 5,000 49 (twice, when its stack had to grow) ->
 // 4.6; 10^6 x 1,000 0.97 -> 0.37; 50,001 x 60 dense 0.73 -> 0.25; 20,000 x 800
 // planted with the network 4.1 -> 1.3.  What bounds
-// it now: each class's chain of dependent steps (26 cycles from one of a
-// worker's instructions to its next, 0.23 of the issue slots used, ncu), and
-// for the triple pass popc.
+// it now: each class's chain of dependent steps (12 cycles from one of a
+// worker's instructions to its next, 0.48 of the issue slots used on 100,000 x
+// 2,000, ncu), and for the triple pass popc.
 #include "fim_common.cuh"
 
 namespace {
