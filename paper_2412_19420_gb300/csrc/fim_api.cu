@@ -460,7 +460,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         int rc = FIM_E_INVAL;
         if (blind) rc = launch_pairs_tc_blind(ctx);
         else if (!(flags & FIM_PAIRS_POPC))
-            rc = pairs_rows_pays(ctx) ? launch_pairs_rows(ctx) : launch_pairs_tc(ctx, 0, true, st);
+            rc = pairs_rows_pays(ctx) ? launch_pairs_rows(ctx) : launch_pairs_tc(ctx, 0, true, st, ctx->num_sms);
         if (rc == FIM_OK) ctx->stats.pair_path = 1;
         else FIM_TRY(launch_pairs_popc(ctx));
         if (sp_items) {  // launched after the pair pass, so that its CTAs take the SMs first

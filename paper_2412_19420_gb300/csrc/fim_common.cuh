@@ -433,9 +433,9 @@ int launch_mine_begin(fim_ctx *ctx, const DbDesc &d, MineCounters *d_ctr);
 
 // k_pairs.cu
 int launch_pairs_popc(fim_ctx *ctx);
-// tcgen05, the pairs of items a0 .. m' - 1 (0: all); the counts are cleared
-// first unless clear is false
-int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st);
+// tcgen05, the pairs of items a0 .. m' - 1 (0: all), on `ctas` SMs; the counts
+// are cleared first unless clear is false
+int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st, int ctas);
 int launch_pairs_tc_blind(fim_ctx *ctx);
 bool pairs_rows_pays(const fim_ctx *ctx);
 int launch_pairs_rows(fim_ctx *ctx);  // rows, and the most frequent items' block by launch_pairs_tc

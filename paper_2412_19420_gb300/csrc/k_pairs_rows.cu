@@ -18,14 +18,16 @@
 // L2 takes 220 G/s of them over a 73 MB table (measured).
 //
 // The pairs among the kTop most frequent items are the hottest addresses and a
-// dense block: they go to the tensor cores beside this kernel, on the side
-// stream (a handful of MMA stages per SM), and are skipped here.
+// dense block: they go to the tensor cores, on the side stream, and are skipped
+// here.
 //
 // Pair pass, ms (tensor cores alone -> rows and the top block): 10^7 x 5,000
-// 92.2 -> 4.3, 10^6 x 1,000 0.64 -> 0.37.
+// 92.2 -> 4.3, 10^6 x 1,000 0.64 -> 0.3.
 //
 // The rows must name an item once (the supports' sum is compared with the
 // number of ids); other matrices take the tensor-core pass.
+#include <algorithm>
+
 #include "fim_common.cuh"
 
 namespace {
@@ -129,6 +131,12 @@ pairs_rows_kernel(const uint32_t *__restrict__ ptr, const unsigned short *__rest
     }
 }
 
+constexpr size_t kBesideBytes = 16u << 20;  // counts that the top block may run beside
+constexpr double kStageUs = 0.59;       // a 128-transaction stage of one tensor-core tile
+
+// The row pass's REDs.
+double rows_us(const fim_ctx *ctx) { return (double)ctx->row_pairs / 220e3 + 15.0; }
+
 }  // namespace
 
 // The row pass pays where its REDs (220 G/s) take less than the tensor cores'
@@ -143,9 +151,8 @@ bool pairs_rows_pays(const fim_ctx *ctx) {
     double tiles = 0;
     for (int ta = 0; ta < nta; ta++) tiles += ntb - (ta >> 1);
     const double stages = (double)((ctx->nw + 3) / 4);
-    const double tc_us = (tiles - 2.0) * stages / ctx->num_sms * 0.59;
-    const double rows_us = (double)ctx->row_pairs / 220e3 + 15.0;
-    return rows_us < tc_us;
+    const double tc_us = (tiles - 2.0) * stages / ctx->num_sms * kStageUs;
+    return rows_us(ctx) < tc_us;
 }
 
 int launch_pairs_rows(fim_ctx *ctx) {
@@ -157,12 +164,28 @@ int launch_pairs_rows(fim_ctx *ctx) {
     FIM_CUDA_TRY(cudaMemsetAsync(ctx->pair_cnt.p, 0, sizeof(int) * (size_t)mf * mf, st));
     FIM_CUDA_TRY(cudaEventRecord(ctx->pair_ev[0], st));
     FIM_CUDA_TRY(cudaStreamWaitEvent(ctx->aux_stream, ctx->pair_ev[0], 0));
-    FIM_TRY(launch_pairs_tc(ctx, a0, false, ctx->aux_stream));
+    // A tensor-core CTA fills an SM's shared memory, so on all SMs the top
+    // block's two tiles hold the row pass back, which fewer SMs keep bound by its
+    // REDs.  So the block gets half as many SMs again as would let it end with
+    // the rows (it runs slower beside them): 10^6 x 1,000 0.355 -> 0.28 to
+    // 0.32 ms for both (1x: 0.308, 2x: 0.328), 333,333 x 701 0.148 -> 0.113.  Where the
+    // counts are a large part of L2 the block's reads evict them, and it goes
+    // first on all SMs: 10^7 x 5,000 (73 MB) 4.33 ms, beside the rows 4.95.
+    const bool beside = sizeof(int) * (size_t)mf * mf <= kBesideBytes;
+    const double block_us = 2.0 * (double)((ctx->nw + 3) / 4) * kStageUs;
+    int tc = ctx->num_sms;
+    if (beside) tc = (int)std::min(1.5 * block_us / rows_us(ctx) + 1.0, ctx->num_sms / 2.0);
+    if (tc < 1) tc = 1;
+    FIM_TRY(launch_pairs_tc(ctx, a0, false, ctx->aux_stream, tc));
     FIM_CUDA_TRY(cudaEventRecord(ctx->pair_ev[1], ctx->aux_stream));
     const size_t smem = sizeof(unsigned short) * ((((size_t)ctx->m + 7) & ~(size_t)7) + PR_W * 2 * PR_CAP);
     FIM_CUDA_TRY(cudaFuncSetAttribute(pairs_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int64_t grid = ceil_div64(ceil_div64(ctx->n, 32), PR_W);
-    if (grid > (int64_t)ctx->num_sms * 8) grid = (int64_t)ctx->num_sms * 8;
+    // beside the block, resident CTAs only: a grid-stride share that waited for
+    // an SM would end late
+    int64_t room = (int64_t)ctx->num_sms * 8;
+    if (beside) room = (int64_t)std::max(1, ctx->num_sms - tc) * std::min(8, (int)(227 * 1024 / (smem + 1024)));
+    if (grid > room) grid = room;
     ctx->launches++;
     pairs_rows_kernel<<<(unsigned)grid, PR_T, smem, st>>>(ctx->row_ptr.as<uint32_t>(),
                                                           ctx->row_idx.as<unsigned short>(), ctx->n,

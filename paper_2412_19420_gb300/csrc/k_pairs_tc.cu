@@ -354,7 +354,7 @@ pairs_tc_kernel(const uint32_t *__restrict__ bm, const int32_t *__restrict__ per
 
 }  // namespace
 
-int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st) {
+int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st, int ctas) {
     const int ld = ctx->mfreq, mf = ld - a0;
     if (mf < 2) return FIM_OK;
     const int nta = (int)ceil_div64(mf, TM), ntb = (int)ceil_div64(mf, TN);
@@ -363,7 +363,7 @@ int launch_pairs_tc(fim_ctx *ctx, int a0, bool clear, cudaStream_t st) {
     const int64_t S = ceil_div64(ctx->nw, 4);  // 128 transactions per stage
     const int64_t W = tiles * S;
     const int kd = ctx->pairs_kdrain > 0 ? ctx->pairs_kdrain : KDRAIN_MAX;
-    int64_t grid = ctx->pairs_split > 0 ? ctx->pairs_split : ctx->num_sms;
+    int64_t grid = ctx->pairs_split > 0 ? ctx->pairs_split : ctas;
     if (grid > W) grid = W;
     const size_t smem = sizeof(TcSmem) + 1024;
     FIM_CUDA_TRY(cudaFuncSetAttribute(pairs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
