@@ -478,12 +478,16 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     }
     cudaEventRecord(ctx->ev[2], st);
     bool on_warps = warp_dfs;
+    bool search = do_dfs;
     ctx->dfs_workers = ctx->num_sms * ctx->dfs_ctas_per_sm;
-    if (do_dfs) {
-        if (warp_dfs && !direct && !small_plan) {
-            FIM_TRY(launch_proj_plan(ctx, &proj));
-            on_warps = proj.words <= kProjWords && proj.wmax <= kProjWmax && proj.cands < 0xFFFFFFFFull;
-        }
+    if (warp_dfs && !direct && !small_plan) {
+        FIM_TRY(launch_proj_plan(ctx, &proj));
+        on_warps = proj.words <= kProjWords && proj.wmax <= kProjWmax && proj.cands < 0xFFFFFFFFull;
+        // no item has two later partners: there is no third item to try, and
+        // neither triples nor root classes are planned for a search
+        search = proj.cands > 0;
+    }
+    if (search) {
         const int workers = ctx->dfs_workers * (on_warps ? proj_workers_per_cta() : 1);
         ctx->dfs_workers = workers;
         // deepest class: a prefix can hold at most min(longest row, m') items

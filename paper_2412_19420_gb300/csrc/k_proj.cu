@@ -1361,7 +1361,7 @@ int launch_proj_plan(fim_ctx *ctx, ProjTotals *host) {
     return FIM_OK;
 }
 
-// The projected columns of every item of the plan.
+// The projected columns of every item of the plan, which has candidates.
 int launch_projection(fim_ctx *ctx, int mf, const ProjTotals &t, bool cands_listed, bool triples, uint32_t thr) {
     MineCounters *d_ctr = ctx->counters.as<MineCounters>();
     const int mpw = (int)ceil_div64(mf, 32);
@@ -1369,7 +1369,6 @@ int launch_projection(fim_ctx *ctx, int mf, const ProjTotals &t, bool cands_list
     FIM_TRY(fim_reserve(ctx, ctx->proj_mat, sizeof(uint32_t) * (size_t)t.words));
     FIM_TRY(fim_reserve(ctx, ctx->proj_list, sizeof(uint32_t) * (size_t)t.rows));
     FIM_TRY(fim_reserve(ctx, ctx->proj_cands, sizeof(uint32_t) * (size_t)t.cands));
-    if (t.cands == 0) return FIM_OK;
     if (!cands_listed) {
         ctx->launches++;
         proj_cands_kernel<<<(unsigned)ceil_div64((int64_t)mf * 32, 256), 256, 0, st>>>(

@@ -1,0 +1,61 @@
+"""Mines at the edges of what the search and the record arena are sized for,
+against the oracle or closed forms, on contexts whose earlier calls left other
+contents in the buffers."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2412_19420_gb300 import datagen
+
+pytestmark = pytest.mark.gpu
+fim = pytest.importorskip("paper_2412_19420_gb300.fim")
+
+
+@pytest.fixture()
+def ctx():
+    c = fim.fim_create(0)
+    yield c
+    fim.fim_destroy(c)
+
+
+def _disjoint_pairs(n, m, n_pairs, per, seed):
+    """m frequent items of which only the pairs {2i, 2i + 1}, i < n_pairs, are
+    frequent: no item has two partners."""
+    rng = np.random.default_rng(seed)
+    rows = [[] for _ in range(n)]
+    for i in range(n_pairs):
+        for r in rng.choice(n // 2, size=per, replace=False):
+            rows[r] += [2 * i, 2 * i + 1]
+    free = rng.permutation(np.arange(n // 2, n))
+    at = 0
+    for j in range(2 * n_pairs, m):  # the others alone in their rows
+        for r in free[at:at + per]:
+            rows[r].append(j)
+        at += per
+    return datagen.from_lists([sorted(set(x)) for x in rows], m)
+
+
+# an earlier call that leaves a root order behind, longer than the new roots
+# and meant for other ones: a small matrix mined on its bit columns, a trace, a
+# batch, a shard
+@pytest.mark.parametrize("first", ["direct", "trace", "batch", "shard", "none"])
+def test_pairs_without_third_items(ctx, first):
+    a = datagen.zipf_baskets(3_000, 90, 0.9, 7.0, 4)
+    if first != "none":
+        fim.fim_build_bitmaps(ctx, a.indptr, a.indices, a.m)
+        if first == "direct":
+            fim.fim_mine(ctx, 12)
+        elif first == "trace":
+            fim.fim_mine(ctx, 12, fim.FIM_TRACE)
+        elif first == "shard":
+            fim.fim_mine_shard(ctx, 12, 0, 0, 2)
+        else:
+            fim.fim_mine_batched(ctx, fim.BatchDescriptor([a] * 3, [12] * 3))
+    c = _disjoint_pairs(16_000, 300, 9, 25, 3)
+    want = oracle.apriori(c.indptr, c.indices, c.m, 20)
+    assert len(want) == 309
+    fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+    for _ in range(2):
+        fim.fim_mine(ctx, 20)
+        assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
+        assert fim.fim_get_stats(ctx)["supports_dfs"] == 0
