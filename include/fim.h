@@ -228,6 +228,9 @@ int fim_get_stats(const fim_ctx *ctx, fim_stats *out);
  *                                publishes this work-queue slot, so the worker
  *                                that takes it (and the drain) must time out;
  *                                -1 (default) = off
+ *   "test_record_cap"  0..2^30   for tests: fim_mine starts with room for this many
+ *                                sets (and grows as usual when they do not fit);
+ *                                0 (default) = automatic
  *   "upload_mapped"    0, 1      host input to fim_build_bitmaps and
  *                                fim_mine_batched that lives in page-locked, mapped
  *                                memory (cudaHostAlloc, cudaHostRegister) is read

@@ -77,6 +77,17 @@ int compact_status(fim_ctx *ctx) {
     return ctx->compact_waits && *static_cast<const int *>(ctx->pinned) ? FIM_E_TIMEOUT : FIM_OK;
 }
 
+// Workers reserve record slots ahead.  A used slot past the arena's end is an
+// overflow; a reservation that only ends past it is not, and its slots there
+// are holes that exist in the counts alone: the compaction must not look at
+// them.
+void drop_slots_past_arena(fim_ctx *ctx) {
+    MineCounters &c = ctx->host_ctr;
+    if (c.n_records <= ctx->rec_cap) return;
+    c.rec_holes -= c.n_records - ctx->rec_cap;
+    c.n_records = ctx->rec_cap;
+}
+
 // Phase times of the last single-database mine, once its work has finished
 // (events ev[1..4] of that mine; called before anything records them again).
 int fim_finish_phase_times(fim_ctx *ctx) {
@@ -637,6 +648,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         *retry = true;
         return FIM_OK;
     }
+    drop_slots_past_arena(ctx);
     int lmax = c.max_len;
     if (ctx->shard == 0 && c.m_freq >= 1 && lmax < 1) lmax = 1;
     const unsigned long long n_sets = c.n_records - c.rec_holes;
@@ -668,7 +680,10 @@ int fim_mine(fim_ctx *ctx, uint64_t minsup, uint32_t flags) {
     uint64_t thr64 = (flags & FIM_STRICT) ? minsup + 1 : minsup;
     if ((flags & FIM_STRICT) && minsup == UINT64_MAX) thr64 = UINT64_MAX;
     const uint32_t thr = thr64 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)thr64;
-    if (ctx->rec_cap == 0) {
+    if (ctx->test_record_cap > 0) {
+        ctx->rec_cap = (unsigned long long)ctx->test_record_cap;
+        if (ctx->rec_items_cap == 0) ctx->rec_items_cap = 1ull << 23;
+    } else if (ctx->rec_cap == 0) {
         ctx->rec_cap = 1ull << 20;
         ctx->rec_items_cap = 1ull << 23;
     }
@@ -779,6 +794,7 @@ int fim_set_tuning(fim_ctx *ctx, const char *key, int64_t v) {
         {"spin_limit_ms", &ctx->spin_limit_ms, 1, 600000},
         {"debug_checks", &ctx->debug_checks, 0, 1},
         {"test_withhold_task", &ctx->test_withhold_task, -1, 1 << 20},
+        {"test_record_cap", &ctx->test_record_cap, 0, 1 << 30},
         {"upload_streams", &ctx->upload_streams, 1, 2},
         {"batch_pairs_shape", &ctx->batch_pairs_shape, 0, kBatchPairsShapeCount - 1},
         {"batch_build_block", &ctx->batch_build_block, 16, 64},

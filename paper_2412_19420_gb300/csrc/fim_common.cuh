@@ -305,6 +305,7 @@ struct fim_ctx {
     MineCounters host_ctr;
     void *pinned = nullptr;     // page-locked landing place of the read-backs
     unsigned long long rec_cap = 0, rec_items_cap = 0;
+    int test_record_cap = 0;    // test hook: the record arena's first capacity, in sets (0: automatic)
 
     // compactor
     DevBuf keys, idx_a, idx_b, hist, scan_tmp, kv_a, kv_b;
@@ -414,6 +415,7 @@ struct fim_ctx {
 };
 
 int fim_reserve(fim_ctx *ctx, DevBuf &b, size_t bytes);
+void drop_slots_past_arena(fim_ctx *ctx);  // after a mine without overflow: reserved slots that the arena lacks
 int fim_aux_stream(fim_ctx *ctx);  // create the side stream (highest priority) once
 int fim_finish_phase_times(fim_ctx *ctx);  // the last single mine's phase times, once it has finished
 void fim_release(fim_ctx *ctx, DevBuf &b);

@@ -1503,6 +1503,7 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
             ctx->rec_items_cap = c.n_rec_items + c.n_rec_items / 4 + 4096;
             continue;  // buffers grow; the new pointers give a new graph key
         }
+        drop_slots_past_arena(ctx);
         // ---- canonical order by (database, size, items) ----------------------
         FIM_TRY(launch_compact(ctx, c.n_records, c.n_records - c.rec_holes, n_db, L.m_max > 0 ? L.m_max : 1));
         FIM_TRY(fim_reserve(ctx, ctx->batch_slices, sizeof(unsigned long long) * 2 * (size_t)(n_db + 1)));

@@ -59,3 +59,21 @@ def test_pairs_without_third_items(ctx, first):
         fim.fim_mine(ctx, 20)
         assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
         assert fim.fim_get_stats(ctx)["supports_dfs"] == 0
+
+
+def test_reservations_that_end_past_the_arena(ctx):
+    # workers reserve up to 64 record slots ahead: capacities from exactly the
+    # sets to beyond all reservations, so that the last one ends on either side
+    c = datagen.from_lists([list(range(14))] * 40, 14)
+    want = oracle.apriori(c.indptr, c.indices, c.m, 40)
+    sets = (1 << 14) - 1
+    assert len(want) == sets
+    fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+    grown = 0
+    for cap in range(sets, sets + 8192, 5):
+        fim.fim_set_tuning(ctx, "test_record_cap", cap)
+        fim.fim_mine(ctx, 40)
+        assert fim.fim_fetch_results(ctx).sha256() == want.sha256(), cap
+        grown += fim.fim_get_stats(ctx)["launches_mine"] > 12
+    assert 0 < grown < 1638  # the arena was too small at first, and large enough at last
+    fim.fim_set_tuning(ctx, "test_record_cap", 0)
