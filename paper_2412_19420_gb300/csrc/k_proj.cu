@@ -577,8 +577,13 @@ proj_triple_kernel(const ProjItem *__restrict__ items, int mf, const unsigned lo
             rb = atomicAdd(&ctr->n_records, (unsigned long long)tot);
             ib3 = atomicAdd(&ctr->n_rec_items, 3ull * tot);
             if (more) {
-                q = atomicAdd(&ctr->n_triples, (unsigned long long)__popc(more));
-                atomicAdd((unsigned long long *)&ctr->pending, (unsigned long long)__popc(more));
+                // only the roots that fit are stored and searched, so only they
+                // are pending (the others are beyond the records, whose overflow
+                // repeats the mine)
+                const unsigned long long n = (unsigned long long)__popc(more);
+                q = atomicAdd(&ctr->n_triples, n);
+                if (q < rec_cap)
+                    atomicAdd((unsigned long long *)&ctr->pending, q + n <= rec_cap ? n : rec_cap - q);
             }
         }
         rb = __shfl_sync(0xffffffffu, rb, 0);
@@ -600,7 +605,6 @@ proj_triple_kernel(const ProjItem *__restrict__ items, int mf, const unsigned lo
             }
             if (ci + 1 < it.k) {
                 const unsigned long long at = q + __popc(more & lt);
-                // (never beyond the records, whose overflow repeats the mine)
                 if (at < rec_cap) roots[at] = (unsigned long long)lo << 32 | bi << 16 | ci;
             }
         }

@@ -77,3 +77,34 @@ def test_reservations_that_end_past_the_arena(ctx):
         grown += fim.fim_get_stats(ctx)["launches_mine"] > 12
     assert 0 < grown < 1638  # the arena was too small at first, and large enough at last
     fim.fim_set_tuning(ctx, "test_record_cap", 0)
+
+
+def test_more_triples_than_records_fit(ctx):
+    # 2,300 frequent triples and a search below them; room for fewer roots than
+    # there are, for exactly as many, and for all records
+    c = datagen.from_lists([list(range(25)) for _ in range(4)] + [[r % 25] for r in range(40_000)], 25)
+    fim.fim_set_tuning(ctx, "spin_limit_ms", 2_000)
+    fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+    for max_len in (3, 4):
+        want = oracle.apriori(c.indptr, c.indices, c.m, 4, max_len=max_len)
+        for cap in (1, 24, 326, 1_000, 2_023, 2_024, 2_299, 2_300, 2_624, 2_625, 2_626, 20_000):
+            fim.fim_set_tuning(ctx, "test_record_cap", cap)
+            fim.fim_mine(ctx, 4, fim.FIM_MAXLEN(max_len))
+            assert fim.fim_fetch_results(ctx).sha256() == want.sha256(), (max_len, cap)
+
+
+def test_a_million_triples_on_a_fresh_context(ctx):
+    # all triples of 200 items: more than the 2^20 records a context begins with
+    n, m = 2_000, 200
+    indptr = np.arange(n + 1, dtype=np.int64) * m
+    indices = np.tile(np.arange(m, dtype=np.int32), n)
+    fim.fim_set_tuning(ctx, "spin_limit_ms", 2_000)
+    fim.fim_build_bitmaps(ctx, indptr, indices, m)
+    fim.fim_mine(ctx, n, fim.FIM_MAXLEN(3))
+    got = fim.fim_fetch_results(ctx)
+    n1, n2, n3 = m, m * (m - 1) // 2, m * (m - 1) * (m - 2) // 6
+    assert len(got) == n1 + n2 + n3 and np.all(got.supports == n)
+    tri = got.items[n1 + 2 * n2:].reshape(-1, 3).astype(np.int64)
+    assert np.all(np.diff(tri, axis=1) > 0)
+    key = (tri[:, 0] * m + tri[:, 1]) * m + tri[:, 2]
+    assert np.all(np.diff(key) > 0)
