@@ -221,12 +221,18 @@ int fim_get_stats(const fim_ctx *ctx, fim_stats *out);
  *                                supports at the threshold, sets strictly increasing
  *                                in (size, items) order); FIM_E_CHECK otherwise
  *                                (default 0)
- *   "spin_limit_ms"    1..600000 longest a device-side wait (the DFS work queue)
- *                                spins before the mine ends with FIM_E_TIMEOUT
- *                                (default 60000); the ctx stays usable
+ *   "spin_limit_ms"    1..600000 longest a device-side wait (the DFS work queue,
+ *                                and up to 2 s the output sort) spins before the
+ *                                mine, or for the sort the call that reads its
+ *                                output, ends with FIM_E_TIMEOUT (default 60000);
+ *                                the ctx stays usable
  *   "test_withhold_task" -1..2^20 fault injection for tests: the DFS never
  *                                publishes this work-queue slot, so the worker
  *                                that takes it (and the drain) must time out;
+ *                                -1 (default) = off
+ *   "test_withhold_tile" -1..2^20 fault injection for tests: the output sort's
+ *                                launches (large outputs) never publish this tile's
+ *                                counts, so the tiles behind it must time out;
  *                                -1 (default) = off
  *   "test_record_cap"  0..2^30   for tests: fim_mine starts with room for this many
  *                                sets (and grows as usual when they do not fit);

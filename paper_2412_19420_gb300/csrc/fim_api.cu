@@ -794,6 +794,7 @@ int fim_set_tuning(fim_ctx *ctx, const char *key, int64_t v) {
         {"spin_limit_ms", &ctx->spin_limit_ms, 1, 600000},
         {"debug_checks", &ctx->debug_checks, 0, 1},
         {"test_withhold_task", &ctx->test_withhold_task, -1, 1 << 20},
+        {"test_withhold_tile", &ctx->test_withhold_tile, -1, 1 << 20},
         {"test_record_cap", &ctx->test_record_cap, 0, 1 << 30},
         {"upload_streams", &ctx->upload_streams, 1, 2},
         {"batch_pairs_shape", &ctx->batch_pairs_shape, 0, kBatchPairsShapeCount - 1},

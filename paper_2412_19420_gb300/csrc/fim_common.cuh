@@ -399,6 +399,7 @@ struct fim_ctx {
     int debug_checks = 0;       // device-side invariant checks after build and mine
     int spin_limit_ms = 60000;  // longest device-side wait before FIM_E_TIMEOUT
     int test_withhold_task = -1; // test hook: the DFS never publishes this queue slot
+    int test_withhold_tile = -1; // test hook: the output sort never publishes this tile's counts
     int upload_mapped = 1;      // host input in pinned, mapped memory: build reads it in place
     int upload_chunks = 4;      // host input: index upload chunks overlapped with the build
     int upload_streams = 2;     // copy streams the chunks alternate over

@@ -190,9 +190,10 @@ one_cta_compact_kernel(int R, int R_valid, const unsigned long long *__restrict_
 
 // out[i] = word[idx[i]]: one key word in the records' current order.
 __global__ void gather_word_kernel(const unsigned long long *__restrict__ word, const uint32_t *__restrict__ idx,
-                                   unsigned long long n, unsigned long long *__restrict__ out) {
+                                   unsigned long long n, unsigned long long *__restrict__ out,
+                                   const int *__restrict__ err) {
     const unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = word[idx[i]];
+    if (i < n && *err == 0) out[i] = word[idx[i]];
 }
 
 // ---- the radix sort of a large output ------------------------------------
@@ -270,14 +271,20 @@ rs_base_kernel(unsigned long long *__restrict__ hist) {
 // A tile's published word of one digit: flag in the top two bits (1: its own
 // count, 2: the count up to and including it), the count below.
 constexpr unsigned long long RS_OWN = 1ull << 62, RS_ALL = 2ull << 62, RS_VAL = RS_OWN - 1;
-constexpr unsigned long long RS_WAIT_NS = 2000000000ull;  // 2 s: far above any legitimate wait
+// A look-back waits 2 s at most (far above any legitimate wait), or the ctx's
+// spin limit.  On expiry the tile sets the error word and scatters nothing, so
+// record numbers are missing from then on: later launches look at the word
+// first and leave them alone, and the output pass writes the records as they
+// lie.  The call that reads the output reports FIM_E_TIMEOUT.
+constexpr unsigned long long RS_WAIT_NS = 2000000000ull;
 
 template <int NT>
 __global__ void __launch_bounds__(NT)
 rs_digit_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *__restrict__ idx_in,
                 unsigned long long *__restrict__ key_out, uint32_t *__restrict__ idx_out, unsigned long long n,
                 int shift, const unsigned long long *__restrict__ base, unsigned long long *status,
-                unsigned long long *__restrict__ next_status, uint32_t *__restrict__ ticket, int *__restrict__ err) {
+                unsigned long long *__restrict__ next_status, uint32_t *__restrict__ ticket, int *err,
+                unsigned long long wait_ns, long long withhold) {
     constexpr int NW = NT / 32;
     __shared__ uint32_t wc[NW][256];            // per-warp digit counts, then offsets
     __shared__ unsigned long long dst[256];     // where the tile's keys of a digit go
@@ -287,10 +294,11 @@ rs_digit_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *_
     if (threadIdx.x == 0) {
         // tiles in the order CTAs start: a tile only waits for tiles that run
         s_tile = atomicAdd(ticket, 1u);
-        s_bad = 0;
+        s_bad = *(volatile int *)err;
     }
     for (int i = threadIdx.x; i < NW * 256; i += NT) (&wc[0][0])[i] = 0;
     __syncthreads();
+    if (s_bad) return;  // (a running tile that needs this one's counts sees the word too)
     const unsigned long long tile = s_tile;
     if (threadIdx.x < 256) next_status[tile * 256 + threadIdx.x] = 0ull;  // the next digit's words
     const unsigned long long t0 = tile * (NT * RI) + (unsigned long long)warp * (32 * RI);
@@ -326,10 +334,11 @@ rs_digit_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *_
         }
         volatile unsigned long long *st = status + d;
         unsigned long long pre = 0;
+        const bool publish = (long long)tile != withhold;  // (the fault-injection hook withholds one tile's)
         if (tile == 0) {
-            st[0] = RS_ALL | cnt;
+            if (publish) st[0] = RS_ALL | cnt;
         } else {
-            st[tile * 256] = RS_OWN | cnt;
+            if (publish) st[tile * 256] = RS_OWN | cnt;
             // predecessors LB at a time, their words loaded together: hundreds
             // of tiles start at once, and one word after another is a round
             // trip to L2 each
@@ -345,7 +354,7 @@ rs_digit_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *_
                 for (int i = 0; i < LB; i++) {
                     if (!more) break;
                     while (!(x[i] >> 62)) {
-                        if (globaltimer_ns() - t_wait > RS_WAIT_NS) {
+                        if (globaltimer_ns() - t_wait > wait_ns || *(volatile int *)err) {
                             s_bad = 1;
                             break;
                         }
@@ -356,7 +365,7 @@ rs_digit_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *_
                 }
                 q -= LB;
             }
-            st[tile * 256] = RS_ALL | (pre + cnt);
+            if (publish) st[tile * 256] = RS_ALL | (pre + cnt);
         }
         dst[d] = base[d] + pre;
     }
@@ -376,14 +385,20 @@ rs_digit_kernel(const unsigned long long *__restrict__ key_in, const uint32_t *_
     }
 }
 
+// The record at position q of the sorted order; record q itself after a sort
+// whose look-back ran out (err), which left record numbers unwritten.
+__device__ __forceinline__ uint32_t sorted_record(const uint32_t *idx, unsigned long long q, const int *err) {
+    return err && *err ? (uint32_t)q : idx[q];
+}
+
 // Sizes in sorted order, block sums for the offset scan.
 constexpr int ST = 1024;
 __global__ void __launch_bounds__(ST)
 len_block_sums_kernel(const uint32_t *__restrict__ idx, const uint32_t *__restrict__ rec_len,
-                      unsigned long long R, unsigned long long *__restrict__ bsum) {
+                      unsigned long long R, unsigned long long *__restrict__ bsum, const int *__restrict__ err) {
     __shared__ unsigned long long s[ST / 32];
     const unsigned long long q = (unsigned long long)blockIdx.x * ST + threadIdx.x;
-    unsigned long long v = q < R ? rec_len[idx[q]] : 0;
+    unsigned long long v = q < R ? rec_len[sorted_record(idx, q, err)] : 0;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -423,13 +438,13 @@ emit_sorted_kernel(const uint32_t *__restrict__ idx, unsigned long long R,
                    const uint32_t *__restrict__ rec_sup, const uint32_t *__restrict__ items,
                    const unsigned long long *__restrict__ bsum, unsigned long long *__restrict__ out_off,
                    uint32_t *__restrict__ out_items, uint32_t *__restrict__ out_sup,
-                   unsigned long long total_items) {
+                   unsigned long long total_items, const int *__restrict__ err) {
     __shared__ unsigned long long s[ST / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long q = (unsigned long long)blockIdx.x * ST + threadIdx.x;
     uint32_t r = 0;
     unsigned long long len = 0;
-    if (q < R) { r = idx[q]; len = rec_len[r]; }
+    if (q < R) { r = sorted_record(idx, q, err); len = rec_len[r]; }
     unsigned long long x = len;
     for (int o = 1; o < 32; o <<= 1) {
         unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
@@ -525,6 +540,9 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
                                               (int)(sizeof(uint32_t) * 256 * RS_MAXPASS)));
     }
     ctx->compact_waits = !csort;
+    int *const err = csort ? nullptr : ctx->dev_flag.as<int>() + kCompactErr;
+    const unsigned long long spin_ns = (unsigned long long)ctx->spin_limit_ms * 1000000ull;
+    const unsigned long long wait_ns = spin_ns < RS_WAIT_NS ? spin_ns : RS_WAIT_NS;
     int enq_rc = FIM_OK;  // a launch that enqueue() could not make
     // The whole pass sequence, enqueued on st.  Returns the kernel count.
     auto enqueue = [&]() -> uint64_t {
@@ -573,28 +591,28 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
                     kin = keys + (size_t)w * R;  // record order: read the key array itself
                 } else if (passes[i - 1].first != w) {
                     gather_word_kernel<<<(unsigned)ceil_div64((int64_t)R, 256), 256, 0, st>>>(keys + (size_t)w * R, ia,
-                                                                                            R, ka);
+                                                                                            R, ka, err);
                     nk++;
                     kin = ka;
                 }
                 unsigned long long *kout = (kin == ka) ? kb : ka;
                 (wide ? rs_digit_kernel<512> : rs_digit_kernel<256>)<<<(unsigned)ntiles, wide ? 512 : 256, 0, st>>>(
                     kin, ia, kout, ib, R, shift, hist + (size_t)i * 256, status + (i & 1) * words,
-                    status + ((i & 1) ^ 1) * words, ticket + i, ctx->dev_flag.as<int>() + kCompactErr);
+                    status + ((i & 1) ^ 1) * words, ticket + i, err, wait_ns, ctx->test_withhold_tile);
                 nk++;
                 uint32_t *t = ia; ia = ib; ib = t;
                 kin = kout;
             }
         }
         unsigned long long *bsum = ctx->scan_tmp.as<unsigned long long>();
-        len_block_sums_kernel<<<nblk, ST, 0, st>>>(ia, ctx->rec_len.as<uint32_t>(), R, bsum);
+        len_block_sums_kernel<<<nblk, ST, 0, st>>>(ia, ctx->rec_len.as<uint32_t>(), R, bsum, err);
         scan_u64_single_kernel<<<1, 1024, 0, st>>>(bsum, (unsigned long long)nblk);
         emit_sorted_kernel<<<nblk, ST, 0, st>>>(ia, R, ctx->rec_off.as<unsigned long long>(),
                                                 ctx->rec_len.as<uint32_t>(), ctx->rec_sup.as<uint32_t>(),
                                                 ctx->rec_items.as<uint32_t>(), bsum,
                                                 ctx->out_off.as<unsigned long long>(),
                                                 ctx->out_items.as<uint32_t>(), ctx->out_sup.as<uint32_t>(),
-                                                total_items);
+                                                total_items, err);
         return nk + 3;
     };
     // A shape met a second time (same sizes, same buffers) is captured into a
@@ -611,6 +629,7 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
     mix((uint64_t)(uintptr_t)ctx->dbdesc.p); mix((uint64_t)(uintptr_t)ctx->rec_db.p);
     mix((uint64_t)(uintptr_t)ctx->kv_a.p); mix((uint64_t)(uintptr_t)ctx->kv_b.p);
     mix(csort ? (uint64_t)(cs_cl * 100000 + cs_per) : 0ull);
+    mix(csort ? 0ull : wait_ns); mix(csort ? 0ull : (uint64_t)(int64_t)ctx->test_withhold_tile);
     for (int i = 0; i < 2; i++)
         if (ctx->compact_graph_exec[i] && ctx->compact_key[i] == key) {
             FIM_CUDA_TRY(cudaGraphLaunch((cudaGraphExec_t)ctx->compact_graph_exec[i], st));

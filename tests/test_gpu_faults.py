@@ -83,3 +83,39 @@ def test_debug_checks_pass_on_correct_runs(ctx):
             assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
     finally:
         fim.fim_set_tuning(ctx, "debug_checks", 0)
+
+
+def test_withheld_sort_tile_times_out_and_ctx_survives(ctx):
+    # a tile of the output sort that never publishes its counts: the tiles
+    # behind it give up, later launches leave the unwritten record numbers
+    # alone, every reader of the output reports the timeout, and the same ctx
+    # is exact again (launched directly, captured and replayed)
+    c, thr = datagen.planted(n=20_000, m=800, n_patterns=60, seed=4), 240
+    want = oracle.apriori(c.indptr, c.indices, c.m, thr)
+    fim.fim_set_tuning(ctx, "compact_cluster", 0)
+    fim.fim_set_tuning(ctx, "spin_limit_ms", 200)
+    fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+    timed_out = pytest.raises(fim.FimError, match=rf"\({fim.FIM_E_TIMEOUT}\)")
+    try:
+        for _ in range(3):
+            fim.fim_mine(ctx, thr)
+            assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
+            parts = [fim.fim_fetch_results(ctx)]
+            for tile in (0, 1, 3):
+                fim.fim_set_tuning(ctx, "test_withhold_tile", tile)
+                for _ in range(3):
+                    fim.fim_mine(ctx, thr)
+                    with timed_out:
+                        fim.fim_fetch_results(ctx)
+                    with timed_out:
+                        fim.fim_rules(ctx, 900_000, 3)
+                with timed_out:
+                    fim.fim_merge_results(ctx, c.n, c.m, parts)
+                with timed_out:
+                    fim.fim_mine_batched(ctx, fim.BatchDescriptor([c, c], [thr, thr]))
+                fim.fim_set_tuning(ctx, "test_withhold_tile", -1)
+                fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+    finally:
+        fim.fim_set_tuning(ctx, "test_withhold_tile", -1)
+        fim.fim_set_tuning(ctx, "compact_cluster", 1)
+        fim.fim_set_tuning(ctx, "spin_limit_ms", 60_000)
