@@ -485,6 +485,7 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
     FIM_TRY(fim_reserve(ctx, ctx->out_sup, sizeof(uint32_t) * (R ? R : 1)));
     ctx->out_sets = R_valid;  // the holes sort after every itemset: emitted last, never fetched
     ctx->out_items_total = total_items;
+    ctx->compact_waits = false;  // until a sort with look-backs is queued
     if (R == 0) {
         FIM_CUDA_TRY(cudaMemsetAsync(ctx->out_off.p, 0, sizeof(unsigned long long), st));
         return FIM_OK;
@@ -493,7 +494,6 @@ int launch_compact(fim_ctx *ctx, uint64_t R, uint64_t R_valid, int n_db, int m_m
     const int bits = bits_for(m_max);
     const int total_bits = db_bits + 8 + bits * lmax;
     const int kw = (int)ceil_div64(total_bits, 64);
-    ctx->compact_waits = false;
     if (n_db == 1 && R <= OC_MAX && kw <= OC_KW && ctx->compact_cluster) {
         FIM_CUDA_TRY(cudaFuncSetAttribute(one_cta_compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)oc_smem(OC_KW)));

@@ -119,3 +119,23 @@ def test_withheld_sort_tile_times_out_and_ctx_survives(ctx):
         fim.fim_set_tuning(ctx, "test_withhold_tile", -1)
         fim.fim_set_tuning(ctx, "compact_cluster", 1)
         fim.fim_set_tuning(ctx, "spin_limit_ms", 60_000)
+
+
+def test_an_empty_mine_after_a_timed_out_sort(ctx):
+    # the earlier mine's error is not reported again for an output without sets
+    c = datagen.planted(n=20_000, m=800, n_patterns=60, seed=4)
+    fim.fim_set_tuning(ctx, "compact_cluster", 0)
+    fim.fim_set_tuning(ctx, "spin_limit_ms", 200)
+    fim.fim_set_tuning(ctx, "test_withhold_tile", 0)
+    fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+    try:
+        fim.fim_mine(ctx, 240)
+        with pytest.raises(fim.FimError, match=rf"\({fim.FIM_E_TIMEOUT}\)"):
+            fim.fim_fetch_results(ctx)
+        fim.fim_mine(ctx, c.n + 1)
+        assert len(fim.fim_fetch_results(ctx)) == 0
+        assert fim.fim_rules(ctx, 500_000) == 0
+    finally:
+        fim.fim_set_tuning(ctx, "test_withhold_tile", -1)
+        fim.fim_set_tuning(ctx, "compact_cluster", 1)
+        fim.fim_set_tuning(ctx, "spin_limit_ms", 60_000)
