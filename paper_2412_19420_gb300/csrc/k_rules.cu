@@ -189,7 +189,8 @@ __device__ __forceinline__ Eval evaluate(const SetsView &v, const SizeTable &t, 
 // (double)a / (double)b, correctly rounded, in integers: the FP64 pipe issues
 // a warp instruction every 16 cycles, and two conversions and a division of
 // each rule's two ratios held the write pass to 31 us for 665,000 rules (now
-// 14).  a, b > 0 are rounded to 53 bits (as the conversions do) and normalised
+// 14).  a, b > 0 (a zero, which merged sets can bring, takes the FP64 division:
+// 0, infinity or NaN) are rounded to 53 bits (as the conversions do) and normalised
 // to A, B in [2^52, 2^53); then
 // long division with two digits of 28 bits, each the top 32 bits of the rest
 // times a 32-bit reciprocal of B's top bits (an FP32 reciprocal and one Newton
@@ -205,6 +206,7 @@ __device__ __forceinline__ unsigned long long round53(unsigned long long x) {
 }
 
 __device__ __forceinline__ double ratio(unsigned long long a, unsigned long long b) {
+    if (a == 0 || b == 0) return (double)a / (double)b;
     a = round53(a);
     b = round53(b);
     const int la = __clzll((long long)a), lb = __clzll((long long)b);

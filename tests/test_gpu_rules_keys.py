@@ -46,3 +46,42 @@ def test_rules_of_long_sets(m, n, k):
     assert np.array_equal(got.ante_mask, want.ante_mask)
     assert np.array_equal(got.conf.view(np.uint64), want.conf.view(np.uint64))
     assert np.array_equal(got.lift.view(np.uint64), want.lift.view(np.uint64))
+
+
+def _merged_rules(ctx, n_trans, sets, sups):
+    """Rules of at least 0 confidence of merged sets, and the divisions they
+    stand for."""
+    off = np.concatenate([[0], np.cumsum([len(x) for x in sets])]).astype(np.uint64)
+    part = (off, np.concatenate(sets).astype(np.uint32), np.asarray(sups, np.uint32))
+    fim.fim_merge_results(ctx, n_trans, 1 + int(part[1].max()), [part])
+    assert fim.fim_rules(ctx, 0) == sum(2 ** len(x) - 2 for x in sets)
+    got = fim.fim_fetch_rules(ctx)
+    held = fim.fim_fetch_results(ctx)
+    S = held.as_dict()
+    conf, lift = [], []
+    with np.errstate(divide="ignore", invalid="ignore"):
+        for z, mask in zip(got.set_index, got.ante_mask):
+            items = held.items[held.offsets[z]:held.offsets[z + 1]]
+            x = tuple(int(i) for b, i in enumerate(items) if mask >> b & 1)
+            y = tuple(int(i) for b, i in enumerate(items) if not mask >> b & 1)
+            sz, sx, sy = (np.float64(v) for v in (S[tuple(items.tolist())], S[x], S[y]))
+            conf.append(sz / sx)
+            lift.append(sz * n_trans / (sx * sy))
+    assert np.array_equal(got.conf, conf, equal_nan=True)
+    assert np.array_equal(got.lift, lift, equal_nan=True)
+    return got
+
+
+SETS = [[0], [1], [2], [0, 1], [0, 2], [1, 2], [0, 1, 2]]
+
+
+def test_ratios_of_zero():
+    # a merge for no transactions, and merged sets that occur nowhere
+    ctx = fim.fim_create(0)
+    try:
+        got = _merged_rules(ctx, 0, SETS, [9, 8, 7, 5, 4, 3, 2])
+        assert np.all(got.lift == 0) and np.all(got.conf > 0)
+        got = _merged_rules(ctx, 100, SETS, [9, 8, 7, 5, 4, 3, 0])
+        assert np.count_nonzero(got.conf == 0) == 6 == np.count_nonzero(got.lift == 0)
+    finally:
+        fim.fim_destroy(ctx)
