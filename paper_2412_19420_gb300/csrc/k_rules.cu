@@ -132,14 +132,18 @@ hash_sets_kernel(const unsigned long long *__restrict__ off, const uint32_t *__r
     }
 }
 
-// Support of the subset of z (L items at zp, ascending) picked by pick, or 0.
-__device__ __forceinline__ uint32_t find_subset(const SetsView &v, const uint32_t *zp, int L, uint32_t pick) {
+// Support of the subset of z (L items at zp, ascending) picked by pick.  A
+// missing subset (not a mine's output) sets *err; a support of 0 is a support.
+__device__ __forceinline__ uint32_t find_subset(const SetsView &v, const uint32_t *zp, int L, uint32_t pick, int *err) {
     const Key key = key_of(zp, L, pick, v.bits);
     uint32_t step;
     for (uint32_t at = slot_of(key, &step) & v.mask;; at = (at + step) & v.mask) {
         const ulonglong2 k = __ldg(reinterpret_cast<const ulonglong2 *>(v.hash + at));
         const uint2 x = __ldg(reinterpret_cast<const uint2 *>(v.hash + at) + 2);
-        if (x.x == EMPTY) return 0;
+        if (x.x == EMPTY) {
+            atomicExch(err, 1);
+            return 0;
+        }
         if (k.x != key.lo || k.y != key.hi) continue;
         if (!(key.hi >> 63)) return x.y;
         const unsigned long long o = __ldg(v.off + x.x);
@@ -154,7 +158,7 @@ __device__ __forceinline__ uint32_t find_subset(const SetsView &v, const uint32_
 struct Eval {
     int64_t z;
     uint32_t mask;
-    uint64_t sz, sx, sy;  // sx or sy 0: the subset is missing
+    uint64_t sz, sx, sy;
 };
 
 // The subsets' supports of a kept candidate, carried from the keep pass to the
@@ -176,12 +180,12 @@ __device__ __forceinline__ int64_t set_of_eval(const SizeTable &t, unsigned long
     return (int64_t)(t.first[l] + z);
 }
 
-__device__ __forceinline__ Eval evaluate(const SetsView &v, const SizeTable &t, unsigned long long e, int len) {
+__device__ __forceinline__ Eval evaluate(const SetsView &v, const SizeTable &t, unsigned long long e, int len, int *err) {
     Eval r;
     r.z = set_of_eval(t, e, &r.mask, &len);
     const uint32_t *zp = v.items + v.off[r.z];
-    r.sx = find_subset(v, zp, len, r.mask);
-    r.sy = find_subset(v, zp, len, ((1u << len) - 1u) - r.mask);
+    r.sx = find_subset(v, zp, len, r.mask, err);
+    r.sy = find_subset(v, zp, len, ((1u << len) - 1u) - r.mask, err);
     r.sz = v.sup[r.z];
     return r;
 }
@@ -287,7 +291,7 @@ rule_keep_kernel(SetsView v, const __grid_constant__ SizeTable sizes, unsigned l
             if (e >= e1) continue;
             len[q] = len0;
             z[q] = set_of_eval(t, e, &mask[q], &len[q]);
-            sx[q] = find_subset(v, v.items + v.off[z[q]], len[q], mask[q]);
+            sx[q] = find_subset(v, v.items + v.off[z[q]], len[q], mask[q], err);
             ante[e - e0] = sx[q];
         }
         __syncthreads();
@@ -301,9 +305,8 @@ rule_keep_kernel(SetsView v, const __grid_constant__ SizeTable sizes, unsigned l
                 const unsigned long long mirror = e - mask[q] + rest;
                 const uint32_t sy = mirror >= e0 && mirror < e1
                                         ? ante[mirror - e0]
-                                        : find_subset(v, v.items + v.off[z[q]], len[q], rest);
-                if (!sx[q] || !sy) atomicExch(err, 1);  // a subset is missing: not a mine's output
-                else keep = (uint64_t)v.sup[z[q]] * 1000000ull >= (uint64_t)ppm * sx[q];
+                                        : find_subset(v, v.items + v.off[z[q]], len[q], rest, err);
+                keep = (uint64_t)v.sup[z[q]] * 1000000ull >= (uint64_t)ppm * sx[q];
                 if (keep && sups) sups[e] = RuleSups{sx[q], sy};
             }
             const uint32_t bal = __ballot_sync(0xffffffffu, keep);
@@ -321,7 +324,7 @@ __global__ void __launch_bounds__(RT)
 rule_write_kernel(SetsView v, const __grid_constant__ SizeTable sizes, unsigned long long E, uint64_t n, const uint32_t *__restrict__ keep_bits,
                   const unsigned long long *__restrict__ part, const RuleSups *__restrict__ sups,
                   unsigned long long *__restrict__ set_index, uint32_t *__restrict__ ante_mask,
-                  double *__restrict__ conf, double *__restrict__ lift) {
+                  double *__restrict__ conf, double *__restrict__ lift, int *__restrict__ err) {
     constexpr int W = EV / 32;  // keep words of a chunk: one per lane of a warp
     static_assert(W == 32, "a warp scans a chunk's keep words");
     __shared__ SizeTable t;
@@ -363,7 +366,7 @@ rule_write_kernel(SetsView v, const __grid_constant__ SizeTable sizes, unsigned 
                 sx = r.x;
                 sy = r.y;
             } else {
-                const Eval r = evaluate(v, t, e, len0);
+                const Eval r = evaluate(v, t, e, len0, err);
                 z = r.z;
                 mask = r.mask;
                 sz = r.sz;
@@ -469,7 +472,7 @@ int fim_rules(fim_ctx *ctx, uint32_t min_conf_ppm, int max_len, uint64_t *n_rule
                 rule_write_kernel<<<grid, RT, 0, st>>>(v, sizes, E, (uint64_t)ctx->out_n, keep, part, sups,
                                                        ctx->rule_set.as<unsigned long long>(),
                                                        ctx->rule_mask.as<uint32_t>(), ctx->rule_conf.as<double>(),
-                                                       ctx->rule_lift.as<double>());
+                                                       ctx->rule_lift.as<double>(), err);
                 FIM_CUDA_TRY(cudaGetLastError());
                 return FIM_OK;
             };

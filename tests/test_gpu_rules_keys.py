@@ -85,3 +85,16 @@ def test_ratios_of_zero():
         assert np.count_nonzero(got.conf == 0) == 6 == np.count_nonzero(got.lift == 0)
     finally:
         fim.fim_destroy(ctx)
+
+
+def test_subsets_of_support_zero_are_held():
+    # a held set of support 0 is not a missing one; a missing one still is
+    ctx = fim.fim_create(0)
+    try:
+        got = _merged_rules(ctx, 100, SETS, [9, 0, 7, 0, 4, 0, 0])
+        assert np.isnan(got.conf).any()
+        _merged_rules(ctx, 100, SETS, [0] * 7)
+        with pytest.raises(fim.FimError, match=rf"\({fim.FIM_E_STATE}\)"):
+            _merged_rules(ctx, 100, SETS[:1] + SETS[2:], [9, 7, 5, 4, 3, 2])
+    finally:
+        fim.fim_destroy(ctx)
