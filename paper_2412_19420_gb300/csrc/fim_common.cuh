@@ -239,6 +239,14 @@ struct RowCopy {
     uint64_t cap;         // rows with more items in all are not kept
 };
 constexpr uint64_t kRowCopyItems = 24;
+// The row pass walks the ids in steps of 32 with 32-bit indexes: they and one
+// step more must not wrap.
+constexpr uint64_t kRowCopyMost = (1ull << 32) - 64;
+// The cap for n rows.
+inline uint64_t row_copy_cap(int64_t n) {
+    const uint64_t cap = (uint64_t)n * kRowCopyItems;
+    return cap <= kRowCopyMost ? cap : 0;
+}
 
 // The projection of one frequent item a (k_proj.cu): its transactions and
 // the columns of its candidates restricted to them.

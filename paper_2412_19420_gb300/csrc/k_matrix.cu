@@ -293,8 +293,8 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
     // pairs than the tensor cores' pass costs)
     RowCopy rows{};
     if (ctx->n > 0 && ctx->m > 0) {
-        const uint64_t cap = (uint64_t)ctx->n * kRowCopyItems;
-        if (cap < 0xFFFFFFFFull) {
+        const uint64_t cap = row_copy_cap(ctx->n);
+        if (cap > 0) {
             FIM_TRY(fim_reserve(ctx, ctx->row_ptr, sizeof(uint32_t) * (size_t)(ctx->n + 1)));
             FIM_TRY(fim_reserve(ctx, ctx->row_idx, sizeof(unsigned short) * (size_t)cap));
             rows.ptr = ctx->row_ptr.as<uint32_t>();
