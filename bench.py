@@ -772,7 +772,7 @@ def _roofline(st, avg, csr, workload, probes):
         # warp workers on projected columns, else CTA workers
         roof = _dfs_roofline(st, avg[dom], workload, probes,
                              "dfs_proj_kernel" if st["dfs_workers"] > 1024 else "dfs_kernel")
-    elif dom == "ms_pairs" and st["pair_path"] == 1 and st["n_frequent_items"] > 256:
+    elif dom == "ms_pairs" and st["pair_rows"]:
         # the rows' pairs as atomics in L2 beside the most frequent items'
         # tensor-core block: the packed rows (16-bit ids, 32-bit offsets) and
         # the counts, which its atomics bound, not these bytes

@@ -104,7 +104,7 @@ typedef struct {
     uint32_t pair_path;           /* 1 = tcgen05 tensor cores (all pairs, or the block
                                      of the most frequent items beside the row pass),
                                      0 = CUDA-core popc                               */
-    uint32_t reserved;
+    uint32_t pair_rows;           /* 1 = the pairs outside that block came from the rows */
 } fim_stats;
 
 /* One database of a batch (fim_mine_batched).  CSR as for fim_build_bitmaps;
@@ -214,6 +214,12 @@ int fim_get_stats(const fim_ctx *ctx, fim_stats *out);
  *   "pairs_kdrain"     0..32768  128-transaction stages one accumulator sums before
  *                                it is drained (0 = 32768: partial sums stay <= 2^24,
  *                                exact in f32)
+ *   "pairs_rows"       -1, 0, 1  fim_mine's pair supports from the rows, beside the
+ *                                tensor-core block of the 256 most frequent items:
+ *                                1 = wherever that is exact (more than 256 frequent
+ *                                items, rows kept by the build, no row that repeats
+ *                                an item), 0 = never, -1 (default) = where it is
+ *                                expected to be faster
  *   "debug_checks"     0, 1      after fim_build_bitmaps, check on the device that
  *                                every pad bit and pad word of the columns is zero;
  *                                after fim_mine, that the output is canonical (sets

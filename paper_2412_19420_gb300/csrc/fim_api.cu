@@ -461,19 +461,22 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         FIM_CUDA_TRY(cudaEventRecord(ctx->aux_ev[0], st));
         FIM_CUDA_TRY(cudaStreamWaitEvent(ctx->aux_stream, ctx->aux_ev[0], 0));
     }
-    ctx->stats.pair_path = 0;
+    ctx->stats.pair_path = ctx->stats.pair_rows = 0;
     if (do_pairs) {
         const int mpw = (int)ceil_div64(mf, 32);
         const size_t npairs = (size_t)mf * (mf - 1) / 2;
         FIM_TRY(fim_reserve(ctx, ctx->pair_cnt, sizeof(int) * (size_t)mf * mf));
         FIM_TRY(fim_reserve(ctx, ctx->pairbits, sizeof(uint32_t) * (size_t)mf * mpw));
         FIM_TRY(fim_reserve(ctx, ctx->roots, sizeof(uint32_t) * 3 * npairs));
+        const bool rows = !blind && !(flags & FIM_PAIRS_POPC) && pairs_rows_pays(ctx);
         int rc = FIM_E_INVAL;
         if (blind) rc = launch_pairs_tc_blind(ctx);
         else if (!(flags & FIM_PAIRS_POPC))
-            rc = pairs_rows_pays(ctx) ? launch_pairs_rows(ctx) : launch_pairs_tc(ctx, 0, true, st, ctx->num_sms);
-        if (rc == FIM_OK) ctx->stats.pair_path = 1;
-        else FIM_TRY(launch_pairs_popc(ctx));
+            rc = rows ? launch_pairs_rows(ctx) : launch_pairs_tc(ctx, 0, true, st, ctx->num_sms);
+        if (rc == FIM_OK) {
+            ctx->stats.pair_path = 1;
+            ctx->stats.pair_rows = rows;
+        } else FIM_TRY(launch_pairs_popc(ctx));
         if (sp_items) {  // launched after the pair pass, so that its CTAs take the SMs first
             FIM_TRY(launch_sparse_items(ctx, mf, sp_cap, ctx->aux_stream));
             FIM_CUDA_TRY(cudaEventRecord(ctx->aux_ev[1], ctx->aux_stream));
@@ -787,6 +790,7 @@ int fim_set_tuning(fim_ctx *ctx, const char *key, int64_t v) {
         {"root_reverse", &ctx->root_reverse, 0, 1},
         {"pairs_split", &ctx->pairs_split, 0, 4096},
         {"pairs_kdrain", &ctx->pairs_kdrain, 0, 32768},
+        {"pairs_rows", &ctx->pairs_rows, -1, 1},
         {"upload_chunks", &ctx->upload_chunks, 1, 16},
         {"compact_cluster", &ctx->compact_cluster, 0, 1},
         {"upload_mapped", &ctx->upload_mapped, 0, 1},

@@ -389,6 +389,7 @@ struct fim_ctx {
     int l2_bytes = 0;
     int pairs_split = 0;        // split-K factor of the tensor-core pair pass (0 = auto)
     int pairs_kdrain = 0;       // stages (x128 transactions) per exact drain (0 = 64)
+    int pairs_rows = -1;        // pair supports from the rows where exact: -1 where they pay, 0 never, 1 always
     int batch_pairs_shape = 0;  // launch shape of the batched tensor-core pair pass
     int batch_build_block = 32; // words per column a batched build CTA covers (16, 32 or 64)
     int batch_build_coal = 1;   // batched build: a warp reads its rows' ids coalesced

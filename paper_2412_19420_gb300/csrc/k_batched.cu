@@ -1553,6 +1553,7 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
         s.launches_build = 0;
         s.launches_mine = ctx->launches - launches0;
         s.pair_path = pairs_tc ? 1u : 0u;
+        s.pair_rows = 0;
         // phases of the graph: build + singleton supports + rank, pairs +
         // finalize, DFS; then the compaction outside the graph
         s.ms_build = s.ms_singletons = s.ms_pairs = s.ms_dfs = 0.f;

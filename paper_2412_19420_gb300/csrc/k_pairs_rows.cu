@@ -147,6 +147,7 @@ bool pairs_rows_pays(const fim_ctx *ctx) {
     // an item repeated in a row would be counted twice: the supports (set
     // semantics) then sum to less than the ids
     if (!ctx->rows_kept || ctx->host_ctr.sup_sum != (unsigned long long)ctx->row_nnz || mf <= kTop || ctx->pairs_split > 0 || ctx->pairs_kdrain > 0) return false;
+    if (ctx->pairs_rows >= 0) return ctx->pairs_rows != 0;
     const int nta = (mf + 127) / 128, ntb = (mf + 255) / 256;
     double tiles = 0;
     for (int ta = 0; ta < nta; ta++) tiles += ntb - (ta >> 1);

@@ -50,10 +50,10 @@ class fim_stats(ctypes.Structure):
         "classes", "tasks_pushed", "diffset_classes", "peak_device_bytes",
         "launches_build", "launches_mine", "dfs_busy_ns", "dfs_span_ns", "dfs_workers", "dfs_root_ns")] + \
         [(n, ctypes.c_float) for n in ("ms_build", "ms_singletons", "ms_pairs", "ms_dfs", "ms_compact")] + \
-        [("pair_path", ctypes.c_uint32), ("reserved", ctypes.c_uint32)]
+        [("pair_path", ctypes.c_uint32), ("pair_rows", ctypes.c_uint32)]
 
     def as_dict(self) -> dict:
-        return {n: getattr(self, n) for n, _ in self._fields_ if n != "reserved"}
+        return {n: getattr(self, n) for n, _ in self._fields_}
 
 
 class fim_db_desc(ctypes.Structure):

@@ -81,3 +81,55 @@ def test_compact_device_rows_and_rebuilds(ctx):
         fim.fim_mine(ctx, 15)
         want = oracle.apriori(c.indptr, c.indices, c.m, 15)
         assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
+
+
+# The cases above leave the choice to the pass's estimate; here it is made for
+# them, and the statistics say which pass ran.
+
+@pytest.fixture(params=[1, 0])
+def forced(ctx, request):
+    fim.fim_set_tuning(ctx, "pairs_rows", request.param)
+    yield request.param
+    fim.fim_set_tuning(ctx, "pairs_rows", -1)
+
+
+@pytest.mark.parametrize("n,m", [(40_000, 257), (40_001, 300), (39_999, 513), (1_025, 700), (31, 400), (32, 400),
+                                 (33, 400)])
+def test_forced_row_pairs_vs_oracle(ctx, forced, n, m):
+    c = datagen.zipf_baskets(n, m, 0.3, 5.0, [n, m]) if n > 33 else _rows(n, m, n, 22, empty=0.05)
+    mf = np.unique(c.indices).size
+    assert mf > 256
+    for minsup in (1, 12):
+        want = oracle.apriori(c.indptr, c.indices, c.m, minsup, max_len=2)
+        assert _pairs(ctx, c, minsup) == want.sha256()
+        st = fim.fim_get_stats(ctx)
+        assert st["pair_rows"] == (forced and st["n_frequent_items"] > 256)
+
+
+def test_forced_long_and_empty_rows(ctx, forced):
+    long_rows = [(0, 31), (1, 32), (2, 33), (500, 1000), (501, 1024), (502, 1025), (503, 1100), (29_999, 1500)]
+    c = _rows(30_000, 1600, 5, 4, long_rows)
+    want = oracle.apriori(c.indptr, c.indices, c.m, 3, max_len=2)
+    assert _pairs(ctx, c, 3) == want.sha256()
+    assert fim.fim_get_stats(ctx)["pair_rows"] == forced
+
+
+def test_forced_row_pairs_leave_repeated_items_alone(ctx, forced):
+    rng = np.random.default_rng(8)
+    rows = [list(rng.choice(600, size=5, replace=False)) for _ in range(40_000)]
+    for repeats in (0, 1):  # one row that names one item twice
+        rows[77] += rows[77][:repeats]
+        c = datagen.from_lists(rows, 600)
+        want = oracle.apriori(c.indptr, c.indices, c.m, 4, max_len=2)
+        assert _pairs(ctx, c, 4) == want.sha256()
+        assert fim.fim_get_stats(ctx)["pair_rows"] == (forced and not repeats)
+
+
+def test_forced_rows_after_rebuilds(ctx, forced):
+    a, b = datagen.zipf_baskets(50_000, 700, 0.3, 6.0, 1), datagen.zipf_baskets(30_011, 900, 0.3, 5.0, 2)
+    for c in (a, b, a):
+        fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+        fim.fim_mine(ctx, 15)
+        want = oracle.apriori(c.indptr, c.indices, c.m, 15)
+        assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
+        assert fim.fim_get_stats(ctx)["pair_rows"] == forced
