@@ -332,6 +332,7 @@ int fim_build_bitmaps(fim_ctx *ctx, const void *indptr, const void *indices, int
     ctx->max_row_len = bf.max_len;
     ctx->row_nnz = bf.nnz;
     ctx->row_pairs = bf.row_pairs;
+    ctx->tile_pairs = bf.tile_pairs;
     ctx->rows_kept = ctx->row_cap > 0 && (uint64_t)bf.nnz <= ctx->row_cap;
     cudaEventElapsedTime(&ctx->stats.ms_build, ctx->ev[0], ctx->ev[1]);
     ctx->stats.ms_singletons = 0.f;  // counted by the build kernel

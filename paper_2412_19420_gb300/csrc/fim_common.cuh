@@ -231,7 +231,10 @@ struct BuildFlags {
     int max_len;                   // longest row
     long long nnz;                 // indptr[n]
     unsigned long long row_pairs;  // sum over the rows of len (len - 1) / 2
+    unsigned tile_pairs;           // the most of 32 rows [32 t, 32 t + 32), rows of more than kRowLong ids twice
+    unsigned pad;
 };
+constexpr int kRowLong = 1024;     // longest row that the row pass packs; longer ones take it twice as long a pair
 // The rows kept for the pair pass; cap 0: none.
 struct RowCopy {
     uint32_t *ptr;        // [n + 1]
@@ -293,6 +296,7 @@ struct fim_ctx {
     uint64_t row_cap = 0;
     int64_t row_nnz = 0;            // items in the rows
     uint64_t row_pairs = 0;         // pairs of items that share a row
+    uint32_t tile_pairs = 0;        // the most that one warp of the row pass counts in a row (BuildFlags)
     bool rows_kept = false;         // row_ptr / row_idx hold this matrix's rows
     cudaEvent_t pair_ev[2] = {};    // fork and join of the pair pass's two halves
     DevBuf bm, item_sup, perm, rank, dev_flag;

@@ -30,6 +30,7 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
     // their word, so their items' bits spread over the banks
     extern __shared__ __align__(16) uint32_t tile[];
     __shared__ int s_max;
+    __shared__ unsigned s_tile;
     __shared__ unsigned long long s_pairs;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int SPLIT = T / 32 / WB;
@@ -42,6 +43,7 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
     const int64_t t1 = min(n, t0 + WB * 32);
     int bad = 0, my_max = 0;
     unsigned long long my_pairs = 0;
+    unsigned my_tile = 0;
     if (nnz < 0) {  // device input: indptr[n] read here, and indptr[0] checked once
         nnz = (int64_t)indptr[n];
         if (nnz < 0) bad = 1;
@@ -54,6 +56,7 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
     for (int k = threadIdx.x; k < WB / 4 * ms; k += T) reinterpret_cast<uint4 *>(tile)[k] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) {
         s_max = 0;
+        s_tile = 0;
         s_pairs = 0;
     }
     __syncthreads();
@@ -66,17 +69,21 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         const int64_t e_end = (int64_t)indptr[rb + nr];
         int64_t off_next = __shfl_down_sync(0xffffffffu, off, 1);
         if (lane == nr - 1) off_next = e_end;
+        unsigned pairs = 0;  // of this row, for the group's sum
         if (lane < nr) {
             if (off_next < off || off < 0 || off_next > nnz) bad = 1;
             else if (sub == 0) {
                 const int64_t len = off_next - off;
                 my_max = max(my_max, (int)min64(len, 1 << 30));
-                my_pairs += (unsigned long long)len * (unsigned long long)(len - 1) / 2;
+                const unsigned long long np = (unsigned long long)len * (unsigned long long)(len - 1) / 2;
+                my_pairs += np;
+                pairs = (unsigned)min64((int64_t)(len > kRowLong ? 2 * np : np), 1 << 26);
                 if (copy) rows.ptr[rb + lane] = (uint32_t)off;
                 if (copy && rb + lane == n - 1) rows.ptr[n] = (uint32_t)off_next;
             }
         }
         if (__any_sync(0xffffffffu, bad)) continue;  // malformed: flagged, not read
+        if (first && sub == 0) my_tile = max(my_tile, __reduce_add_sync(0xffffffffu, pairs));
         const int64_t e_begin = __shfl_sync(0xffffffffu, off, 0);
         const uint32_t wl = (uint32_t)((rb - t0) >> 5);
         // Rows all hold an id (the usual case): their starts are distinct, one
@@ -119,12 +126,14 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         for (int o = 16; o > 0; o >>= 1) my_pairs += __shfl_xor_sync(0xffffffffu, my_pairs, o);
         if (lane == 0) {
             atomicMax(&s_max, my_max);
+            atomicMax(&s_tile, my_tile);
             atomicAdd(&s_pairs, my_pairs);
         }
     }
     __syncthreads();
     if (first && threadIdx.x == 0 && s_max > 0) {
         atomicMax(&flags->max_len, s_max);
+        atomicMax(&flags->tile_pairs, s_tile);
         atomicAdd(&flags->row_pairs, s_pairs);
     }
     // write-out: 16-byte stores, WB / 4 consecutive threads per column; the

@@ -34,7 +34,7 @@ namespace {
 
 constexpr int PR_T = 256;               // threads per CTA
 constexpr int PR_W = PR_T / 32;
-constexpr int PR_CAP = 1024;            // packed elements a warp holds at a time
+constexpr int PR_CAP = kRowLong;        // packed elements a warp holds at a time
 constexpr int kTop = 256;               // most frequent items: the tensor cores' block
 
 // Rows [r0, r0 + 32) of warp tiles, grid-stride.
@@ -131,16 +131,29 @@ pairs_rows_kernel(const uint32_t *__restrict__ ptr, const unsigned short *__rest
     }
 }
 
-constexpr size_t kBesideBytes = 16u << 20;  // counts that the top block may run beside
+// Counts that the top block may run beside (2 million rows of ten items, block
+// beside the rows against block first: 4 MB 591 against 693 us, 16 MB 614 and
+// 695, 25 MB 750 and 676, 36 MB 622 and 633, 49 MB 729 and 635).
+constexpr size_t kBesideBytes = 16u << 20;
 constexpr double kStageUs = 0.59;       // a 128-transaction stage of one tensor-core tile
 
-// The row pass's REDs.
-double rows_us(const fim_ctx *ctx) { return (double)ctx->row_pairs / 220e3 + 15.0; }
+// The row pass: its REDs, or one warp's where a few rows hold most of the pairs.
+// A RED costs the chip 4.5 ps while the counts fit L2 (100 MB), then more:
+// 9.6 ps at 196 MB, 24 at 400 MB, 35 at 1 GB (2 million rows of ten items over
+// 7,001 to 16,001).  A warp counts 600 to 700 pairs a us of the rows it packs
+// and half as many of longer ones: one row of 1,024 ids among 100,000 short
+// ones takes 0.8 ms, one of 1,500 3.5 and one of 5,000 36, where the tensor
+// cores take 1.35 ms whatever the rows are.
+double rows_us(const fim_ctx *ctx) {
+    const double mb = 4e-6 * (double)ctx->mfreq * (double)ctx->mfreq;
+    const double ps = 4.5 + std::min(30.0, 0.065 * std::max(0.0, mb - 100.0));
+    return std::max((double)ctx->row_pairs * ps * 1e-6, (double)ctx->tile_pairs / 600.0) + 15.0;
+}
 
 }  // namespace
 
-// The row pass pays where its REDs (220 G/s) take less than the tensor cores'
-// tiles outside the top block (0.59 us per 128-transaction stage and SM,
+// The row pass pays where it takes less than the tensor cores' tiles outside
+// the top block (0.59 us per 128-transaction stage and SM,
 // measured on 10^6 x 1,000 and 10^7 x 5,000).
 bool pairs_rows_pays(const fim_ctx *ctx) {
     const int mf = ctx->mfreq;

@@ -133,3 +133,25 @@ def test_forced_rows_after_rebuilds(ctx, forced):
         want = oracle.apriori(c.indptr, c.indices, c.m, 15)
         assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
         assert fim.fim_get_stats(ctx)["pair_rows"] == forced
+
+
+@pytest.mark.parametrize("long_rows,rows_pay", [
+    ([], True),
+    ([(20_000, 300)], True),                            # a tenth of a millisecond: still the rows
+    ([(20_000, 1_500)], False),                         # one warp's work for milliseconds
+    ([(20_000, 5_000)], False),
+    ([(20_000 + i, 400) for i in range(32)], False),    # 32 rows of one warp
+    ([(997 * i, 400) for i in range(32)], True),        # the same rows, spread
+])
+def test_rows_that_one_warp_counts_are_priced(ctx, long_rows, rows_pay):
+    c = _rows(100_000, 5_003, 9, 5, long_rows, empty=0)
+    want = oracle.apriori(c.indptr, c.indices, c.m, 20, max_len=2)
+    for on_device in (False, True):
+        ip, ix = c.indptr, c.indices
+        if on_device:
+            import torch
+            ip, ix = torch.from_numpy(ip).cuda(), torch.from_numpy(ix).cuda()
+        fim.fim_build_bitmaps(ctx, ip, ix, c.m)
+        fim.fim_mine(ctx, 20, fim.FIM_MAXLEN(2))
+        assert fim.fim_get_stats(ctx)["pair_rows"] == rows_pay
+        assert fim.fim_fetch_results(ctx).sha256() == want.sha256()
