@@ -240,6 +240,8 @@ int fim_get_stats(const fim_ctx *ctx, fim_stats *out);
  *                                launches (large outputs) never publish this tile's
  *                                counts, so the tiles behind it must time out;
  *                                -1 (default) = off
+ *   "test_memory_mb"   0..2^30   fault injection for tests: the ctx's reservations
+ *                                past this much device memory fail; 0 (default) = off
  *   "test_record_cap"  0..2^30   for tests: fim_mine starts with room for this many
  *                                sets (and grows as usual when they do not fit);
  *                                0 (default) = automatic

@@ -100,6 +100,30 @@ int fim_finish_phase_times(fim_ctx *ctx) {
     return FIM_OK;
 }
 
+// Device memory for b, `want` bytes or at least `bytes`.
+static int dev_alloc(fim_ctx *ctx, DevBuf &b, size_t want, size_t bytes) {
+    const size_t limit = (size_t)ctx->test_memory_mb << 20;
+    for (size_t n = want;; n = bytes) {
+        if (limit && ctx->bytes_held + n > limit) b.p = nullptr;  // (the fault-injection hook)
+        else if (cudaMalloc(&b.p, n) != cudaSuccess) {
+            (void)cudaGetLastError();
+            b.p = nullptr;
+        }
+        if (b.p) {
+            b.bytes = n;
+            return FIM_OK;
+        }
+        if (n == bytes) return FIM_E_NOMEM;
+    }
+}
+
+void drop_rows(fim_ctx *ctx) {
+    ctx->rows_kept = false;
+    ctx->row_cap = 0;
+    fim_release(ctx, ctx->row_ptr);
+    fim_release(ctx, ctx->row_idx);
+}
+
 int fim_reserve(fim_ctx *ctx, DevBuf &b, size_t bytes) {
     if (bytes == 0) bytes = 16;
     if (bytes <= b.bytes) return FIM_OK;
@@ -112,19 +136,15 @@ int fim_reserve(fim_ctx *ctx, DevBuf &b, size_t bytes) {
     }
     size_t nb = bytes + bytes / 4;
     nb = (nb + 255) & ~(size_t)255;
-    cudaError_t e = cudaMalloc(&b.p, nb);
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        e = cudaMalloc(&b.p, bytes);
-        nb = bytes;
-        if (e != cudaSuccess) {
-            (void)cudaGetLastError();
-            b.p = nullptr;
-            return FIM_E_NOMEM;
-        }
+    int rc = dev_alloc(ctx, b, nb, bytes);
+    if (rc == FIM_E_NOMEM && ctx->row_idx.p && &b != &ctx->row_ptr && &b != &ctx->row_idx) {
+        // the kept rows only make the pair pass faster: their room first
+        FIM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        drop_rows(ctx);
+        rc = dev_alloc(ctx, b, nb, bytes);
     }
-    b.bytes = nb;
-    ctx->bytes_held += nb;
+    if (rc != FIM_OK) return rc;
+    ctx->bytes_held += b.bytes;
     if (ctx->bytes_held > ctx->stats.peak_device_bytes) ctx->stats.peak_device_bytes = ctx->bytes_held;
     return FIM_OK;
 }
@@ -800,6 +820,7 @@ int fim_set_tuning(fim_ctx *ctx, const char *key, int64_t v) {
         {"debug_checks", &ctx->debug_checks, 0, 1},
         {"test_withhold_task", &ctx->test_withhold_task, -1, 1 << 20},
         {"test_withhold_tile", &ctx->test_withhold_tile, -1, 1 << 20},
+        {"test_memory_mb", &ctx->test_memory_mb, 0, 1 << 30},
         {"test_record_cap", &ctx->test_record_cap, 0, 1 << 30},
         {"upload_streams", &ctx->upload_streams, 1, 2},
         {"batch_pairs_shape", &ctx->batch_pairs_shape, 0, kBatchPairsShapeCount - 1},

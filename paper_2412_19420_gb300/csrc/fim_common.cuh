@@ -412,6 +412,7 @@ struct fim_ctx {
     int debug_checks = 0;       // device-side invariant checks after build and mine
     int spin_limit_ms = 60000;  // longest device-side wait before FIM_E_TIMEOUT
     int test_withhold_task = -1; // test hook: the DFS never publishes this queue slot
+    int test_memory_mb = 0;      // test hook: reservations past this much device memory fail (0: off)
     int test_withhold_tile = -1; // test hook: the output sort never publishes this tile's counts
     int upload_mapped = 1;      // host input in pinned, mapped memory: build reads it in place
     int upload_chunks = 4;      // host input: index upload chunks overlapped with the build
@@ -433,6 +434,7 @@ void drop_slots_past_arena(fim_ctx *ctx);  // after a mine without overflow: res
 int fim_aux_stream(fim_ctx *ctx);  // create the side stream (highest priority) once
 int fim_finish_phase_times(fim_ctx *ctx);  // the last single mine's phase times, once it has finished
 void fim_release(fim_ctx *ctx, DevBuf &b);
+void drop_rows(fim_ctx *ctx);  // gives the kept rows' memory back
 
 // ---------------------------------------------------------------- launchers
 // k_matrix.cu

@@ -304,11 +304,17 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
     if (ctx->n > 0 && ctx->m > 0) {
         const uint64_t cap = row_copy_cap(ctx->n);
         if (cap > 0) {
-            FIM_TRY(fim_reserve(ctx, ctx->row_ptr, sizeof(uint32_t) * (size_t)(ctx->n + 1)));
-            FIM_TRY(fim_reserve(ctx, ctx->row_idx, sizeof(unsigned short) * (size_t)cap));
-            rows.ptr = ctx->row_ptr.as<uint32_t>();
-            rows.idx = ctx->row_idx.as<unsigned short>();
-            rows.cap = cap;
+            int rc = fim_reserve(ctx, ctx->row_ptr, sizeof(uint32_t) * (size_t)(ctx->n + 1));
+            if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->row_idx, sizeof(unsigned short) * (size_t)cap);
+            if (rc == FIM_OK) {
+                rows.ptr = ctx->row_ptr.as<uint32_t>();
+                rows.idx = ctx->row_idx.as<unsigned short>();
+                rows.cap = cap;
+            } else if (rc == FIM_E_NOMEM) {
+                drop_rows(ctx);  // without them the pair pass takes the columns
+            } else {
+                return rc;
+            }
         }
     }
     ctx->row_cap = rows.cap;

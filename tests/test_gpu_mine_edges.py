@@ -108,3 +108,41 @@ def test_a_million_triples_on_a_fresh_context(ctx):
     assert np.all(np.diff(tri, axis=1) > 0)
     key = (tri[:, 0] * m + tri[:, 1]) * m + tri[:, 2]
     assert np.all(np.diff(key) > 0)
+
+
+def test_kept_rows_give_way_to_what_a_mine_needs():
+    # the rows that a build keeps for the pair pass are optional: where device
+    # memory runs out (a limit of the context's own), they go first
+    import torch
+    rng = np.random.default_rng(2)
+    n, m = 2_000_000, 300
+    indptr = torch.arange(n + 1, dtype=torch.int64, device="cuda") * 4
+    ids = (rng.integers(0, m, (n, 1)) + np.arange(4) * rng.integers(1, 75, (n, 1))) % m  # four distinct ids a row
+    ids = torch.from_numpy(np.sort(ids, axis=1).astype(np.int32).ravel()).cuda()
+    rows_mb = n * 48 >> 20
+
+    def mine(limit_mb):
+        c = fim.fim_create(0)
+        try:
+            fim.fim_set_tuning(c, "test_memory_mb", limit_mb)
+            fim.fim_set_tuning(c, "pairs_rows", 1)
+            out = []
+            fim.fim_build_bitmaps(c, indptr, ids, m)
+            for _ in range(2):
+                fim.fim_mine(c, 200)
+                out.append(fim.fim_fetch_results(c).sha256())
+            st = fim.fim_get_stats(c)
+            return out, st["pair_rows"], st["peak_device_bytes"] >> 20
+        finally:
+            fim.fim_destroy(c)
+
+    want, rows, peak = mine(0)
+    assert rows == 1 and want[0] == want[1]
+    kept = []
+    for less in (rows_mb // 8, rows_mb // 4, rows_mb // 2, rows_mb - 5):
+        got, rows, _ = mine(peak - less)
+        assert got == want
+        kept.append(rows)
+    assert kept[-1] == 0
+    with pytest.raises(fim.FimError, match=rf"\({fim.FIM_E_NOMEM}\)"):
+        mine(100)
