@@ -242,6 +242,7 @@ struct RowCopy {
     uint64_t cap;         // rows with more items in all are not kept
 };
 constexpr uint64_t kRowCopyItems = 24;
+constexpr int kRowPairsTop = 256;  // most frequent items, whose pairs are the tensor cores' block
 // The row pass walks the ids in steps of 32 with 32-bit indexes: they and one
 // step more must not wrap.
 constexpr uint64_t kRowCopyMost = (1ull << 32) - 64;

@@ -299,9 +299,10 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
     FIM_CUDA_TRY(cudaMemsetAsync(ctx->item_sup.p, 0, sizeof(uint32_t) * (size_t)ctx->m, st));
     // the rows, kept as 32-bit offsets and 16-bit ids for the pair pass, where
     // they hold at most kRowCopyItems items on average (longer rows make more
-    // pairs than the tensor cores' pass costs)
+    // pairs than the tensor cores' pass costs) and there are items outside the
+    // tensor cores' block, which that pass never reads the rows for
     RowCopy rows{};
-    if (ctx->n > 0 && ctx->m > 0) {
+    if (ctx->n > 0 && ctx->m > kRowPairsTop) {
         const uint64_t cap = row_copy_cap(ctx->n);
         if (cap > 0) {
             int rc = fim_reserve(ctx, ctx->row_ptr, sizeof(uint32_t) * (size_t)(ctx->n + 1));

@@ -35,7 +35,7 @@ namespace {
 constexpr int PR_T = 256;               // threads per CTA
 constexpr int PR_W = PR_T / 32;
 constexpr int PR_CAP = kRowLong;        // packed elements a warp holds at a time
-constexpr int kTop = 256;               // most frequent items: the tensor cores' block
+constexpr int kTop = kRowPairsTop;      // most frequent items: the tensor cores' block
 
 // Rows [r0, r0 + 32) of warp tiles, grid-stride.
 __global__ void __launch_bounds__(PR_T)

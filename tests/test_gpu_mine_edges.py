@@ -146,3 +146,24 @@ def test_kept_rows_give_way_to_what_a_mine_needs():
     assert kept[-1] == 0
     with pytest.raises(fim.FimError, match=rf"\({fim.FIM_E_NOMEM}\)"):
         mine(100)
+
+
+def _built_mb(indptr, indices, m):
+    c = fim.fim_create(0)
+    try:
+        fim.fim_build_bitmaps(c, indptr, indices, m)
+        return fim.fim_get_stats(c)["peak_device_bytes"] / 2 ** 20
+    finally:
+        fim.fim_destroy(c)
+
+
+def test_rows_are_kept_only_for_a_pass_that_reads_them():
+    # up to 256 items no pair is outside the tensor cores' block: a build then
+    # holds the columns (with a quarter's slack) and not 48 bytes a row more
+    import torch
+    n = 1_000_000
+    indptr = torch.arange(n + 1, dtype=torch.int64, device="cuda") * 3
+    ids = (torch.arange(3 * n, device="cuda") % 250).to(torch.int32)
+    columns = 1.25 * 256 * 4 * (-(-n // 4096) * 128) / 2 ** 20
+    assert columns <= _built_mb(indptr, ids, 256) <= columns + 2
+    assert _built_mb(indptr, ids, 257) > columns + 40
