@@ -50,7 +50,8 @@ build_bitmaps_kernel(const void *__restrict__ indptr_v, const void *__restrict__
         if (blockIdx.x == 0 && blockIdx.y == 0 && blk0 == 0 && threadIdx.x == 0 && indptr[0] != 0) bad = 1;
     }
     const bool first = blockIdx.y == 0;  // this CTA's items are the first: it also sees to the rows
-    const bool copy = first && (uint64_t)nnz <= rows.cap;
+    // (a matrix without ids is within a cap of 0: where no rows are kept there is nowhere to write)
+    const bool copy = first && rows.ptr != nullptr && (uint64_t)nnz <= rows.cap;
     if (first && blk0 == 0 && blockIdx.x == 0 && threadIdx.x == 0) flags->nnz = nnz;
 
     for (int k = threadIdx.x; k < WB / 4 * ms; k += T) reinterpret_cast<uint4 *>(tile)[k] = make_uint4(0, 0, 0, 0);

@@ -167,3 +167,24 @@ def test_rows_are_kept_only_for_a_pass_that_reads_them():
     columns = 1.25 * 256 * 4 * (-(-n // 4096) * 128) / 2 ** 20
     assert columns <= _built_mb(indptr, ids, 256) <= columns + 2
     assert _built_mb(indptr, ids, 257) > columns + 40
+
+
+@pytest.mark.parametrize("m", [1, 256, 257, 2_000])
+def test_matrices_without_ids(ctx, m):
+    # host, page-locked and device input, with and without room for kept rows
+    import torch
+    for limit_mb in (0, 12):
+        for n in (1, 33, 5_000):
+            indptr, ids = np.zeros(n + 1, np.int64), np.zeros(0, np.int32)
+            for ip, ix in ((indptr, ids), (indptr.astype(np.uint32), ids.astype(np.uint16)),
+                           (torch.from_numpy(indptr).pin_memory().numpy(), ids),
+                           (torch.from_numpy(indptr).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda"))):
+                c = fim.fim_create(0)
+                try:
+                    fim.fim_set_tuning(c, "test_memory_mb", limit_mb)
+                    fim.fim_build_bitmaps(c, ip, ix, m)
+                    fim.fim_set_tuning(c, "test_memory_mb", 0)
+                    fim.fim_mine(c, 1)
+                    assert len(fim.fim_fetch_results(c)) == 0
+                finally:
+                    fim.fim_destroy(c)
