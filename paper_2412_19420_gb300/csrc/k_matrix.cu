@@ -304,7 +304,8 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
     // tensor cores' block, which that pass never reads the rows for
     RowCopy rows{};
     if (ctx->n > 0 && ctx->m > kRowPairsTop) {
-        const uint64_t cap = row_copy_cap(ctx->n);
+        uint64_t cap = row_copy_cap(ctx->n);
+        if (nnz >= 0) cap = (uint64_t)nnz <= cap ? (uint64_t)nnz : 0;  // host input: known, so no more than that
         if (cap > 0) {
             int rc = fim_reserve(ctx, ctx->row_ptr, sizeof(uint32_t) * (size_t)(ctx->n + 1));
             if (rc == FIM_OK) rc = fim_reserve(ctx, ctx->row_idx, sizeof(unsigned short) * (size_t)cap);

@@ -188,3 +188,32 @@ def test_matrices_without_ids(ctx, m):
                     assert len(fim.fim_fetch_results(c)) == 0
                 finally:
                     fim.fim_destroy(c)
+
+
+def test_kept_rows_of_host_input_take_what_they_hold():
+    # pageable and page-locked host arrays, wide and compact, whose number of
+    # ids is known before the build
+    import torch
+    n, m = 1_000_000, 300
+    indptr = np.arange(n + 1, dtype=np.int64) * 3
+    ids = (np.arange(3 * n) % m).astype(np.int32)
+    columns = 1.25 * m * 4 * (-(-n // 4096) * 128) / 2 ** 20
+    rows = 1.25 * (4 * n + 2 * 3 * n) / 2 ** 20
+    for ip, ix in ((indptr, ids), (indptr.astype(np.uint32), ids.astype(np.uint16))):
+        staged = 1.25 * (ip.nbytes + ix.nbytes) / 2 ** 20
+        assert columns + rows <= _built_mb(ip, ix, m) <= columns + rows + staged + 2
+        pinned = [torch.from_numpy(a.view({4: np.int32, 8: np.int64, 2: np.int16}[a.itemsize])).pin_memory().numpy()
+                  .view(a.dtype) for a in (ip, ix)]
+        assert columns + rows <= _built_mb(*pinned, m) <= columns + rows + 2
+    c = fim.fim_create(0)
+    try:  # a matrix of longer rows, then shorter ones, then none kept
+        fim.fim_set_tuning(c, "pairs_rows", 1)
+        for mean, kept in ((20, 1), (4, 1), (30, 0), (4, 1)):
+            d = datagen.zipf_baskets(20_000, 400, 0.3, mean, mean)
+            want = oracle.apriori(d.indptr, d.indices, d.m, 30, max_len=2)
+            fim.fim_build_bitmaps(c, d.indptr, d.indices, d.m)
+            fim.fim_mine(c, 30, fim.FIM_MAXLEN(2))
+            assert fim.fim_fetch_results(c).sha256() == want.sha256()
+            assert fim.fim_get_stats(c)["pair_rows"] == kept
+    finally:
+        fim.fim_destroy(c)
