@@ -411,7 +411,13 @@ int fim_rules(fim_ctx *ctx, uint32_t min_conf_ppm, int max_len, uint64_t *n_rule
         uint32_t bits = 1;
         while (bits < 32 && ((uint64_t)ctx->m >> bits)) bits++;
         FIM_TRY(fim_reserve(ctx, ctx->rule_base, sizeof(unsigned long long) * NSIZE));
-        FIM_TRY(fim_reserve(ctx, ctx->rule_hash, sizeof(HashEntry) * (size_t)slots));
+        // a fuller table where memory is short, with an entry free for a lookup to end at
+        int rc_hash = fim_reserve(ctx, ctx->rule_hash, sizeof(HashEntry) * (size_t)slots);
+        while (rc_hash == FIM_E_NOMEM && slots / 2 > (uint64_t)R) {
+            slots /= 2;
+            rc_hash = fim_reserve(ctx, ctx->rule_hash, sizeof(HashEntry) * (size_t)slots);
+        }
+        FIM_TRY(rc_hash);
         const SetsView v{ctx->out_off.as<unsigned long long>(), ctx->out_items.as<uint32_t>(),
                          ctx->out_sup.as<uint32_t>(), ctx->rule_hash.as<HashEntry>(),
                          (uint32_t)(slots - 1), bits};

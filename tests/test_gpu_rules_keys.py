@@ -98,3 +98,32 @@ def test_subsets_of_support_zero_are_held():
             _merged_rules(ctx, 100, SETS[:1] + SETS[2:], [9, 7, 5, 4, 3, 2])
     finally:
         fim.fim_destroy(ctx)
+
+
+def test_a_fuller_table_where_memory_is_short():
+    # 634,680 sets: a table of 2^21 entries (64 MB), or of 2^20 where only that fits
+    from paper_2412_19420_gb300 import datagen
+    c = datagen.planted(n=20_000, m=800, n_patterns=60, seed=4)
+    got, need = [], []
+    for room_mb in (0, 44, 24):
+        ctx = fim.fim_create(0)
+        try:
+            fim.fim_build_bitmaps(ctx, c.indptr, c.indices, c.m)
+            fim.fim_mine(ctx, 100)
+            sets = len(fim.fim_fetch_results(ctx))
+            assert 2 ** 19 < sets < 2 ** 20
+            held = fim.fim_get_stats(ctx)["peak_device_bytes"] >> 20
+            if room_mb:
+                fim.fim_set_tuning(ctx, "test_memory_mb", held + room_mb)
+            if room_mb == 24:
+                with pytest.raises(fim.FimError, match=rf"\({fim.FIM_E_NOMEM}\)"):
+                    fim.fim_rules(ctx, 300_000, 2)
+                continue
+            fim.fim_rules(ctx, 300_000, 2)
+            r = fim.fim_fetch_rules(ctx)
+            got.append((r.set_index, r.ante_mask, r.conf.view(np.uint64), r.lift.view(np.uint64)))
+            need.append((fim.fim_get_stats(ctx)["peak_device_bytes"] >> 20) - held)
+        finally:
+            fim.fim_destroy(ctx)
+    assert need[0] > 64 and need[1] <= 44
+    assert all(np.array_equal(a, b) for a, b in zip(*got))
