@@ -194,6 +194,13 @@ int fim_get_stats(const fim_ctx *ctx, fim_stats *out);
  *                                0 (default) = eight groups for page-locked host
  *                                input (uploaded group by group, or read in place
  *                                by a build of one CTA per SM), else one
+ *   "dfs_proj"         -1..2     who extends the prefixes of a single mine: 0 = CTAs
+ *                                on the bit columns, 1 = warps on columns projected
+ *                                onto each root item's transactions, 2 = warps on the
+ *                                bit columns, -1 (default) = as their costs are
+ *                                estimated.  FIM_TRACE and FIM_NO_SPLIT mines, and
+ *                                searches too deep or columns too long for warps,
+ *                                take CTAs whatever it says
  *   "dfs_warp"         0, 1      fim_mine_batched with every database's columns at
  *                                most 4,096 words: one warp per prefix-extension
  *                                worker instead of one CTA (default 1)

@@ -376,8 +376,8 @@ struct MineState {
 // The search runs on warp workers (k_proj.cu); the trace and no-split
 // options, and searches too deep for a warp worker's stack, on the CTA
 // workers, which look at whole columns.
-bool search_on_warps(uint32_t flags, const MineState &ms) {
-    return !ms.cta_dfs && !(flags & (FIM_TRACE | FIM_NO_SPLIT));
+bool search_on_warps(const fim_ctx *ctx, uint32_t flags, const MineState &ms) {
+    return !ms.cta_dfs && !(flags & (FIM_TRACE | FIM_NO_SPLIT)) && ctx->dfs_proj != 0;
 }
 
 // The largest projection that mf frequent items can have.
@@ -394,9 +394,16 @@ ProjTotals worst_projection(const fim_ctx *ctx, int mf) {
     return t;
 }
 
+// Whether two items of average support share enough rows, if they are independent.
+bool avg_pair_frequent(const fim_ctx *ctx, uint32_t thr) {
+    if (ctx->m <= 0) return false;
+    const double s = (double)ctx->row_nnz / (double)ctx->m;
+    return s * s >= (double)thr * (double)ctx->n;
+}
+
 bool small_plan_takes(const fim_ctx *ctx, int mf, uint32_t flags, const MineState &ms) {
     const ProjTotals t = worst_projection(ctx, mf);
-    return search_on_warps(flags, ms) && ctx->n_shards == 1 && !((flags & FIM_LEARNED) && ctx->learned_order) &&
+    return search_on_warps(ctx, flags, ms) && ctx->n_shards == 1 && !((flags & FIM_LEARNED) && ctx->learned_order) &&
            proj_small_plan_fits(mf) && t.wmax <= kProjWmax && t.words <= kSmallPlanWords && t.rows <= kSmallPlanWords;
 }
 
@@ -444,16 +451,22 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     const bool do_dfs = do_pairs && mf >= 3 && (maxlen == 0 || maxlen >= 3);
     const bool rep = (flags & (FIM_LEARNED | FIM_DIFFSET_RULE)) != 0;  // classes choose their representation
     const bool net_order = (flags & FIM_LEARNED) && ctx->learned_order;  // the network orders the pair roots
-    const bool warp_dfs = do_dfs && search_on_warps(flags, ms);
-    // Small matrices of short rows: few triples, which the bit columns
-    // themselves count sooner than three more launches would (5,746 x 99: 228
-    // against 247 us a mine); rows that hold a third of the frequent items make
-    // wide classes, better projected (12,060 x 46 at density 0.29: 343 against
-    // 507 us).  With more items than the one-launch plan takes, the plan's
-    // totals come back to the host, and the line lies lower.
-    const bool direct = warp_dfs && (proj_small_plan_fits(mf) ? (int64_t)mf * ctx->nwp <= kDirectWordsShort &&
-                                                                    3 * ctx->max_row_len <= mf
-                                                              : (int64_t)mf * ctx->nwp <= kDirectWords);
+    const bool warp_dfs = do_dfs && search_on_warps(ctx, flags, ms);
+    // Small matrices of short rows in which an average pair is infrequent: few
+    // triples, which the bit columns themselves count sooner than three more
+    // launches would (zipf baskets at 2%, us a mine, bit columns against
+    // projected: 2,000 x 169 155 and 169, 50,000 x 60 172 and 182).  Where the
+    // average pair is frequent, nearly all triples are counted, and whole columns
+    // cost more the longer they are (64 items in 5% of the rows each: 8,000 rows
+    // 213 and 195, 64,000 341 and 218, 128,000 464 and 231, CTA workers 296); the
+    // same for rows that hold a third of the frequent items, which make wide
+    // classes (12,060 x 46 at density 0.29: 507 and 343).  With more items than
+    // the one-launch plan takes, the plan's totals come back to the host, and the
+    // line lies lower.
+    bool direct = warp_dfs && (proj_small_plan_fits(mf) ? (int64_t)mf * ctx->nwp <= kDirectWordsShort &&
+                                                              3 * ctx->max_row_len <= mf && !avg_pair_frequent(ctx, thr)
+                                                        : (int64_t)mf * ctx->nwp <= kDirectWords);
+    if (warp_dfs && ctx->dfs_proj >= 0) direct = ctx->dfs_proj == 2;
     // Few frequent items: one launch plans the whole search (pair threshold,
     // roots, projection), sized for the worst case, so that nothing has to
     // come back to the host before the search.
@@ -831,6 +844,7 @@ int fim_set_tuning(fim_ctx *ctx, const char *key, int64_t v) {
         {"root_sort", &ctx->root_sort, 0, 1},
         {"record_chunk", &ctx->rec_chunk, 1, 1024},
         {"batch_segments", &ctx->batch_segments, 0, 16},
+        {"dfs_proj", &ctx->dfs_proj, -1, 2},
         {"dfs_warp", &ctx->dfs_warp, 0, 1},
         {"dfs_warp_ctas", &ctx->dfs_warp_ctas, 2, 3},
     };

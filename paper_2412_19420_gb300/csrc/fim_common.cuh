@@ -401,6 +401,7 @@ struct fim_ctx {
     int root_sort = 1;          // root order without the network: 0 pair-pass order, 1 candidate count
     int rec_chunk = 1;          // record slots a DFS worker reserves at a time
     int batch_segments = 0;     // database groups the batch graph pipelines (build || pairs); 0 automatic
+    int dfs_proj = -1;          // single mines' search: -1 as it pays, 0 CTA workers, 1 projected columns, 2 bit columns
     int dfs_warp = 1;           // batches of short columns: one warp per prefix-extension worker
     int dfs_warp_ctas = 2;      // CTAs of warp workers per SM (2 or 3)
     bool force_cta_dfs = false; // set while a batch is re-mined with CTA workers
