@@ -2,6 +2,8 @@
 // the three stages of Section III (matrix construction, support calculation,
 // frequent-itemset extraction).  No exception crosses the boundary; every
 // entry point returns a FIM_* status.
+#include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -34,18 +36,27 @@ constexpr int64_t kDirectWordsShort = 3 << 17;   // the same for few items in sh
 constexpr unsigned long long kSmallPlanWords = 64ull << 20;  // worst-case projection of a device-planned mine
 constexpr unsigned long long kProjWords = 1ull << 30;  // largest projection (words)
 constexpr unsigned long long kTriples = 64ull << 20;   // largest table of triple supports
+constexpr int64_t kLongWords = 4096;             // columns from which the CTA workers may be the better ones
 constexpr uint32_t kProjWmax = 1u << 15;         // longest projected column (words)
 constexpr size_t kProjStackBudget = 4ull << 30;  // warp workers' global stacks
 
-// Read back a device struct (the stream is synchronised): through page-locked
-// memory, which the copy engine writes without a staging pass.
+// Read back a device struct, or two (the stream is synchronised): through
+// page-locked memory, which the copy engine writes without a staging pass.
+template <class T, class U>
+int read_back(fim_ctx *ctx, T *host, const void *dev, U *host2, const void *dev2) {
+    constexpr size_t at2 = (sizeof(T) + 15) / 16 * 16;
+    static_assert(at2 + sizeof(U) <= kPinnedBytes, "landing place");
+    char *const land = static_cast<char *>(ctx->pinned);
+    FIM_CUDA_TRY(cudaMemcpyAsync(land, dev, sizeof(T), cudaMemcpyDeviceToHost, ctx->stream));
+    if (host2) FIM_CUDA_TRY(cudaMemcpyAsync(land + at2, dev2, sizeof(U), cudaMemcpyDeviceToHost, ctx->stream));
+    FIM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    memcpy((void *)host, land, sizeof(T));
+    if (host2) memcpy((void *)host2, land + at2, sizeof(U));
+    return FIM_OK;
+}
 template <class T>
 int read_back(fim_ctx *ctx, T *host, const void *dev) {
-    static_assert(sizeof(T) <= kPinnedBytes, "landing place");
-    FIM_CUDA_TRY(cudaMemcpyAsync(ctx->pinned, dev, sizeof(T), cudaMemcpyDeviceToHost, ctx->stream));
-    FIM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    memcpy((void *)host, ctx->pinned, sizeof(T));
-    return FIM_OK;
+    return read_back(ctx, host, dev, static_cast<int *>(nullptr), nullptr);
 }
 
 }  // namespace
@@ -376,8 +387,8 @@ struct MineState {
 // The search runs on warp workers (k_proj.cu); the trace and no-split
 // options, and searches too deep for a warp worker's stack, on the CTA
 // workers, which look at whole columns.
-bool search_on_warps(const fim_ctx *ctx, uint32_t flags, const MineState &ms) {
-    return !ms.cta_dfs && !(flags & (FIM_TRACE | FIM_NO_SPLIT)) && ctx->dfs_proj != 0;
+bool search_on_warps(uint32_t flags, const MineState &ms) {
+    return !ms.cta_dfs && !(flags & (FIM_TRACE | FIM_NO_SPLIT));
 }
 
 // The largest projection that mf frequent items can have.
@@ -401,9 +412,46 @@ bool avg_pair_frequent(const fim_ctx *ctx, uint32_t thr) {
     return s * s >= (double)thr * (double)ctx->n;
 }
 
+// Whether warps on projected columns mine a matrix of long columns sooner than
+// CTAs on the whole ones.  A CTA pass costs a column's length per level and
+// support; the projection costs its gathered bits, and one warp then walks a
+// projected column (about as long where the items are dense) per class.  The
+// levels and supports to expect come from the plan: the frequent pairs' mean
+// support, the share q of an item's rows that a partner holds, and sets of k
+// of as many items as make that many pairs while pair support times q^(k - 2)
+// passes.  The factors (us per 1,000 words or million bits) were fitted to 843 mines
+// of 100,000 to 3 million rows, 6 to 400 items, independent, Zipf and
+// correlated: the choice is within 10% of the better one in 833 of them.
+// 1 million rows, us on CTAs and on projected columns: 64 items at density 0.5,
+// pairs only 795 and 2,038; 24 items at 0.5, sets of up to four 1,586 and
+// 2,081, up to six 14,870 and 8,789; 250 Zipf items at 0.8% 388 and 507, at
+// 0.3% 602 and 631; 40 items at 0.05, sets of four 7,375 and 1,187.
+bool projection_pays(const ProjTotals &t, int64_t nw, double n, uint32_t thr) {
+    const double pairs = (double)t.cands, bits = 32.0 * (double)t.words;
+    const double rows = bits / pairs;  // of an item with candidates
+    const double q = std::min(1.0, t.pair_sum ? (double)t.pair_sum / bits : rows / n);
+    double sup = t.pair_sum ? (double)t.pair_sum / pairs : rows * q;
+    int levels = 2;
+    while (levels < 12 && sup * q >= (double)thr) {
+        sup *= q;
+        levels++;
+    }
+    const double items = (1.0 + sqrt(1.0 + 8.0 * pairs)) / 2.0;
+    double sets = pairs, supports = 0;
+    for (int k = 3; k <= levels + 1 && items > k - 1; k++) {
+        sets *= (items - k + 1) / k;
+        supports += sets;
+    }
+    supports = std::max(supports, ((double)t.triples - pairs) / 2.0);
+    const double L = std::min(levels, 7), kw = (double)nw / 1e3, kmax = (double)t.wmax / 1e3;
+    const double cta_us = 20.0 + 1.27 * L * kw + 0.23 * supports / 1e3 * kw;
+    const double warp_us = (15.0 + 4.6 * L) * kmax + 0.84 * bits / 1e6;
+    return warp_us <= cta_us;
+}
+
 bool small_plan_takes(const fim_ctx *ctx, int mf, uint32_t flags, const MineState &ms) {
     const ProjTotals t = worst_projection(ctx, mf);
-    return search_on_warps(ctx, flags, ms) && ctx->n_shards == 1 && !((flags & FIM_LEARNED) && ctx->learned_order) &&
+    return search_on_warps(flags, ms) && ctx->n_shards == 1 && !((flags & FIM_LEARNED) && ctx->learned_order) &&
            proj_small_plan_fits(mf) && t.wmax <= kProjWmax && t.words <= kSmallPlanWords && t.rows <= kSmallPlanWords;
 }
 
@@ -451,7 +499,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     const bool do_dfs = do_pairs && mf >= 3 && (maxlen == 0 || maxlen >= 3);
     const bool rep = (flags & (FIM_LEARNED | FIM_DIFFSET_RULE)) != 0;  // classes choose their representation
     const bool net_order = (flags & FIM_LEARNED) && ctx->learned_order;  // the network orders the pair roots
-    const bool warp_dfs = do_dfs && search_on_warps(ctx, flags, ms);
+    const bool warp_dfs = do_dfs && search_on_warps(flags, ms);
     // Small matrices of short rows in which an average pair is infrequent: few
     // triples, which the bit columns themselves count sooner than three more
     // launches would (zipf baskets at 2%, us a mine, bit columns against
@@ -473,6 +521,8 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     const size_t npairs_all = (size_t)mf * (size_t)(mf > 0 ? mf - 1 : 0) / 2;
     ProjTotals proj = worst_projection(ctx, mf);
     const bool small_plan = do_dfs && small_plan_takes(ctx, mf, flags, ms);
+    // long columns: the plan's totals come back first, to choose the workers
+    const bool ask = small_plan && !direct && (ctx->dfs_proj == 0 || (ctx->dfs_proj < 0 && ctx->nw >= kLongWords));
     // automatic: keep low-support classes sparse when the frequent item
     // columns do not fit in half of L2 (streaming whole columns from HBM
     // is latency-bound; from L2 the dense pass is as fast)
@@ -517,7 +567,7 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         }
         if (small_plan) {
             FIM_TRY(reserve_root_plan(ctx, npairs));
-            FIM_TRY(launch_proj_small_plan(ctx, mf, thr, d_ctr, !direct));
+            FIM_TRY(launch_proj_small_plan(ctx, mf, thr, d_ctr, !direct && !ask, ask));
         } else {
             FIM_TRY(launch_pairs_finalize(ctx, thr, d_ctr));
         }
@@ -528,9 +578,14 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
     bool on_warps = warp_dfs;
     bool search = do_dfs;
     ctx->dfs_workers = ctx->num_sms * ctx->dfs_ctas_per_sm;
-    if (warp_dfs && !direct && !small_plan) {
-        FIM_TRY(launch_proj_plan(ctx, &proj));
+    int items = mf;  // m', or its bound
+    if (warp_dfs && !direct && (ask || !small_plan)) {
+        if (ask) FIM_TRY(read_back(ctx, &proj, ctx->proj_totals.p, &items, &d_ctr->m_freq));
+        else FIM_TRY(launch_proj_plan(ctx, &proj));
         on_warps = proj.words <= kProjWords && proj.wmax <= kProjWmax && proj.cands < 0xFFFFFFFFull;
+        if (ctx->dfs_proj == 0) on_warps = false;
+        else if (ctx->dfs_proj < 0 && ctx->nw >= kLongWords && proj.cands > 0)
+            on_warps = on_warps && projection_pays(proj, ctx->nw, (double)ctx->n, thr);
         // no item has two later partners: there is no third item to try, and
         // neither triples nor root classes are planned for a search
         search = proj.cands > 0;
@@ -546,6 +601,8 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         ProjParams q{};
         if (on_warps) {
             const bool triples = !direct && ctx->n_shards == 1 && !net_order && proj.triples <= kTriples;
+            if (ask && triples)  // the plan has counted the pairs as roots; the triple pass brings its own
+                FIM_CUDA_TRY(cudaMemsetAsync(&d_ctr->pending, 0, sizeof(d_ctr->pending), st));
             if (!direct) FIM_TRY(launch_projection(ctx, mf, proj, small_plan, triples, thr));
             if (triples) {
                 q.triple = ctx->proj_triple.as<uint32_t>();
@@ -617,9 +674,9 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         p.rec_chunk = ctx->rec_chunk;
         p.root_reverse = ctx->root_reverse;
         const bool sp_late = sp_fits && warp_dfs && !on_warps;
-        if (sp_late) {  // the warp workers' projection was too large after all
-            FIM_TRY(reserve_sparse_items(ctx, mf, sp_cap));
-            FIM_TRY(launch_sparse_items(ctx, mf, sp_cap, st));
+        if (sp_late) {  // the warp workers' projection was too large, or did not pay, after all
+            FIM_TRY(reserve_sparse_items(ctx, items, sp_cap));
+            FIM_TRY(launch_sparse_items(ctx, items, sp_cap, st));
         }
         if (sp_items || sp_late) {
             if (sp_items) FIM_CUDA_TRY(cudaStreamWaitEvent(st, ctx->aux_ev[1], 0));
@@ -637,9 +694,11 @@ int mine_once(fim_ctx *ctx, uint32_t thr, uint32_t flags, MineState &ms, bool *r
         if (on_warps) {
             p.root_order = q.triple ? nullptr : ctx->root_order.as<uint32_t>();
         } else {  // candidate-less roots dropped, the others ordered
-            const int mode = (p.learned && ctx->learned_order) ? 2 : ctx->root_sort;
-            FIM_TRY(reserve_root_plan(ctx, npairs));
-            FIM_TRY(launch_root_plan(ctx, d_ctr, npairs, nullptr, mode, nullptr, st));
+            if (!small_plan) {  // (the one-launch plan has done so)
+                const int mode = (p.learned && ctx->learned_order) ? 2 : ctx->root_sort;
+                FIM_TRY(reserve_root_plan(ctx, npairs));
+                FIM_TRY(launch_root_plan(ctx, d_ctr, npairs, nullptr, mode, nullptr, st));
+            }
             p.root_order = ctx->root_order.as<uint32_t>();
         }
         p.trace = (flags & FIM_TRACE) ? 1 : 0;

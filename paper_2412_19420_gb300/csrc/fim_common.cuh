@@ -268,6 +268,7 @@ struct ProjItem {
 struct ProjTotals {
     unsigned long long words, rows, cands, tiles, triples, units;
     uint32_t wmax, pad;
+    unsigned long long pair_sum;  // supports of those candidates' pairs, summed (small plan, if asked for)
 };
 struct ProjParams {
     const ProjItem *items;
@@ -473,7 +474,7 @@ int launch_epoch_bump(fim_ctx *ctx);
 int launch_proj_plan(fim_ctx *ctx, ProjTotals *host);
 int launch_projection(fim_ctx *ctx, int mf, const ProjTotals &t, bool cands_listed, bool triples, uint32_t thr);
 bool proj_small_plan_fits(int mf);
-int launch_proj_small_plan(fim_ctx *ctx, int mf, uint32_t thr, MineCounters *d_ctr, bool triples);
+int launch_proj_small_plan(fim_ctx *ctx, int mf, uint32_t thr, MineCounters *d_ctr, bool triples, bool ask);
 unsigned long long proj_triple_units(int mf);  // most units of the triple pass
 int launch_dfs_proj(fim_ctx *ctx, const DfsParams &p, const ProjParams &q, int ctas_per_sm);
 int proj_workers_per_cta();

@@ -186,7 +186,7 @@ proj_small_plan_kernel(const int *__restrict__ pair_cnt, int m, uint32_t thr, co
                        uint32_t *__restrict__ root_sup, uint32_t *__restrict__ root_order,
                        ProjItem *__restrict__ items, unsigned long long *__restrict__ tile0,
                        unsigned long long *__restrict__ trip0, uint32_t *__restrict__ cands,
-                       ProjTotals *__restrict__ tot, int triples) {
+                       ProjTotals *__restrict__ tot, int triples, int ask) {
     constexpr int MW = SP_MAX / 32, NW = SP_T / 32, KB = SP_MAX;  // bucket = candidates, 0 .. SP_MAX - 1
     __shared__ uint32_t bits[SP_MAX][MW];
     __shared__ uint32_t rowpos[SP_MAX + 1];
@@ -197,8 +197,11 @@ proj_small_plan_kernel(const int *__restrict__ pair_cnt, int m, uint32_t thr, co
     const int mf = *(volatile const int *)&ctr->m_freq;  // <= m, the host's bound
     const int mpw = (mf + 31) / 32;
     for (int i = threadIdx.x; i < KB; i += SP_T) hist[i] = 0;
+    if (ask && threadIdx.x == 0) tot->pair_sum = 0;
+    if (ask) __syncthreads();
+    unsigned long long pair_sum = 0;
     for (int a = warp; a < mf; a += NW) {
-        uint32_t c = 0;
+        uint32_t c = 0, sum = 0;
         int v[MW];
 #pragma unroll
         for (int w = 0; w < MW; w++) {
@@ -214,7 +217,9 @@ proj_small_plan_kernel(const int *__restrict__ pair_cnt, int m, uint32_t thr, co
                 if (w < mpw) pairbits[a * mpw + w] = bal;
             }
             c += __popc(bal);
+            if (ask && ((bal >> lane) & 1u)) sum += (uint32_t)v[w];
         }
+        if (c >= 2) pair_sum += sum;
         if (lane == 0) {
             const uint32_t S = sup[perm[a]];
             rowpos[a] = c;
@@ -223,6 +228,7 @@ proj_small_plan_kernel(const int *__restrict__ pair_cnt, int m, uint32_t thr, co
             s_it[a].W = (uint32_t)(((uint64_t)S + 127) / 128 * 4);
         }
     }
+    if (ask && pair_sum) atomicAdd(&tot->pair_sum, pair_sum);
     __syncthreads();
     if (warp == 0) {  // prefix sums over the rows, four to a lane
         constexpr int PER = SP_MAX / 32;
@@ -1419,7 +1425,7 @@ bool proj_small_plan_fits(int mf) { return mf <= SP_MAX; }
 // Pair threshold, records, roots and the projection's plan of a small mine
 // (in place of launch_pairs_finalize, the root plan and launch_proj_plan).
 // mf: m', or a bound of it.
-int launch_proj_small_plan(fim_ctx *ctx, int mf, uint32_t thr, MineCounters *d_ctr, bool triples) {
+int launch_proj_small_plan(fim_ctx *ctx, int mf, uint32_t thr, MineCounters *d_ctr, bool triples, bool ask) {
     const size_t npairs = (size_t)mf * (mf - 1) / 2;
     FIM_TRY(fim_reserve(ctx, ctx->proj_items, sizeof(ProjItem) * (size_t)mf));
     FIM_TRY(fim_reserve(ctx, ctx->proj_tiles, 2 * sizeof(unsigned long long) * (size_t)(mf + 1)));
@@ -1434,7 +1440,7 @@ int launch_proj_small_plan(fim_ctx *ctx, int mf, uint32_t thr, MineCounters *d_c
         ctx->rec_items_cap, roots, roots + npairs, roots + 2 * npairs, ctx->root_order.as<uint32_t>(),
         ctx->proj_items.as<ProjItem>(), ctx->proj_tiles.as<unsigned long long>(),
         ctx->proj_tiles.as<unsigned long long>() + (mf + 1), ctx->proj_cands.as<uint32_t>(),
-        ctx->proj_totals.as<ProjTotals>(), triples ? 1 : 0);
+        ctx->proj_totals.as<ProjTotals>(), triples ? 1 : 0, ask ? 1 : 0);
     FIM_CUDA_TRY(cudaGetLastError());
     return FIM_OK;
 }
