@@ -432,6 +432,13 @@ struct fim_ctx {
     uint64_t launches = 0;      // kernels this ctx has launched
 };
 
+// A kernel's shared-memory limit is the process's, not a context's: every launch
+// sets the same one, the most that the kernel is ever launched with, so that no
+// thread lowers it between another's call and launch.
+template <class Kernel>
+cudaError_t fim_allow_smem(Kernel *kern, size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
 int fim_reserve(fim_ctx *ctx, DevBuf &b, size_t bytes);
 void drop_slots_past_arena(fim_ctx *ctx);  // after a mine without overflow: reserved slots that the arena lacks
 int fim_aux_stream(fim_ctx *ctx);  // create the side stream (highest priority) once

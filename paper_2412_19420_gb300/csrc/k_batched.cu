@@ -1296,12 +1296,11 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
             mix(&nu, sizeof(nu));
         }
         const size_t smem_build = (size_t)L.ib * WB * sizeof(uint32_t);
-        FIM_CUDA_TRY(cudaFuncSetAttribute(batch_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem_build));
+        FIM_CUDA_TRY(fim_allow_smem(batch_build_kernel, 1024u * WB * sizeof(uint32_t)));
         const size_t smem_rows = (size_t)(L.m_max | 1) * wbk * sizeof(uint32_t);
         if (rows_build) {
-            FIM_CUDA_TRY(cudaFuncSetAttribute(build_rows_fn(wbk, coal, persist_build),
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows));
+            const size_t most = 1025u * (size_t)wbk * sizeof(uint32_t);
+            FIM_CUDA_TRY(fim_allow_smem(build_rows_fn(wbk, coal, persist_build), most < 227u * 1024u ? most : 227u * 1024u));
         }
         const bool reuse = ctx->batch_graph_exec && ctx->batch_graph_blob == key;
         if (!reuse) {

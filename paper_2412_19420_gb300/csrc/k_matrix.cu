@@ -293,7 +293,7 @@ int launch_build_bitmaps(fim_ctx *ctx, const void *d_indptr, const void *d_indic
     // (10^7 x 5,000 3.31 -> 3.13 ms)
     const int ms = ib + ((WB == 16 ? 2 : 4) - ib % 8 + 8) % 8;
     const size_t smem = (size_t)ms * WB * sizeof(uint32_t);
-    FIM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FIM_CUDA_TRY(fim_allow_smem(kern, (size_t)(most + 8) * WB * sizeof(uint32_t)));
     BuildFlags *flags = ctx->dev_flag.as<BuildFlags>();
     cudaStream_t st = ctx->stream;
     FIM_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(BuildFlags), st));

@@ -172,7 +172,7 @@ extern "C" int fim_pair_supports_noalloc(const int64_t *d_indptr, const int32_t 
     if (nnz < 0 || (nnz > 0 && !d_indices)) return FIM_E_INVAL;
     const int ib = m < 1024 ? m : 1024;
     const size_t smem = (size_t)ib * NA_WB * sizeof(uint32_t);
-    FIM_CUDA_TRY(cudaFuncSetAttribute(na_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FIM_CUDA_TRY(fim_allow_smem(na_build_kernel, 1024u * NA_WB * sizeof(uint32_t)));
     // every word of the m x nwp region is written, so stale contents of an
     // earlier call never leak into this one
     na_build_kernel<<<dim3((unsigned)(nwp / NA_WB), (unsigned)ceil_div64(m, ib)), 256, smem, st>>>(

@@ -193,7 +193,7 @@ int launch_pairs_rows(fim_ctx *ctx) {
     FIM_TRY(launch_pairs_tc(ctx, a0, false, ctx->aux_stream, tc));
     FIM_CUDA_TRY(cudaEventRecord(ctx->pair_ev[1], ctx->aux_stream));
     const size_t smem = sizeof(unsigned short) * ((((size_t)ctx->m + 7) & ~(size_t)7) + PR_W * 2 * PR_CAP);
-    FIM_CUDA_TRY(cudaFuncSetAttribute(pairs_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FIM_CUDA_TRY(fim_allow_smem(pairs_rows_kernel, sizeof(unsigned short) * (((FIM_MAX_ITEMS + 7) & ~7) + PR_W * 2 * PR_CAP)));
     int64_t grid = ceil_div64(ceil_div64(ctx->n, 32), PR_W);
     // beside the block, resident CTAs only: a grid-stride share that waited for
     // an SM would end late
