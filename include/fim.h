@@ -88,8 +88,11 @@ typedef struct {
                                      projected columns where it runs on those)      */
     uint64_t dfs_bytes;           /* bytes the DFS kernel read/wrote algorithmically */
     uint64_t dfs_touched_bytes;   /* the same, counting only 32-byte sectors that can
-                                     contribute (zero prefix words are skipped)     */
-    uint64_t classes;             /* prefix classes expanded                        */
+                                     contribute (CTA workers and batches skip zero
+                                     prefix words; warps on projected columns read
+                                     every word, and this equals dfs_bytes)         */
+    uint64_t classes;             /* prefix classes expanded by DFS workers (a single
+                                     mine's pass over all triples is not among them) */
     uint64_t tasks_pushed;        /* classes handed to the device work queue        */
     uint64_t diffset_classes;     /* classes counted through a diffset              */
     uint64_t peak_device_bytes;   /* device memory held by the ctx                  */
@@ -98,8 +101,9 @@ typedef struct {
     uint64_t dfs_busy_ns;         /* DFS workers' time inside tasks, summed         */
     uint64_t dfs_span_ns;         /* first worker start to last worker exit         */
     uint64_t dfs_workers;         /* DFS workers (warps or CTAs) of the launch      */
-    uint64_t dfs_root_ns;         /* part of dfs_busy_ns spent in the root classes'
-                                     own passes (candidate list + level-0 pass)     */
+    uint64_t dfs_root_ns;         /* CTA workers: part of dfs_busy_ns spent in the root
+                                     classes' own passes (candidate list + level-0
+                                     pass); 0 for warps                             */
     float ms_build, ms_singletons, ms_pairs, ms_dfs, ms_compact; /* CUDA-event times */
     uint32_t pair_path;           /* 1 = tcgen05 tensor cores (all pairs, or the block
                                      of the most frequent items beside the row pass),
@@ -160,7 +164,8 @@ int fim_mine(fim_ctx *ctx, uint64_t minsup, uint32_t flags);
  * cap_items give the capacities of supports/offsets-1 and items.
  * flags: FIM_OUTPUT_HOST (host buffers) or FIM_OUTPUT_DEVICE (device buffers).
  * Errors: FIM_E_STATE (nothing mined), FIM_E_TOO_SMALL (sizes still written),
- * FIM_E_INVAL, FIM_E_CUDA. */
+ * FIM_E_INVAL, FIM_E_CUDA, FIM_E_TIMEOUT (a bounded wait of the output's sort ran
+ * out: fim_mine returns with the sort queued). */
 int fim_fetch_results(fim_ctx *ctx, uint64_t *n_sets, uint64_t *n_items_total,
                       uint64_t *offsets, uint32_t *items, uint32_t *supports,
                       uint64_t cap_sets, uint64_t cap_items, uint32_t flags);
@@ -174,20 +179,25 @@ int fim_get_stats(const fim_ctx *ctx, fim_stats *out);
 
 /* fim_set_tuning -- set one launch-shape parameter of the ctx; it applies to
  * later calls and never changes results.  Keys and ranges:
- *   "dfs_threads"      256, 512  threads of one DFS worker (CTA)
- *   "dfs_ctas_per_sm"  1..4      DFS workers per SM; dfs_threads x dfs_ctas_per_sm
+ *   "dfs_threads"      256, 512  threads of one DFS worker where workers are CTAs
+ *                                (see "dfs_proj")
+ *   "dfs_ctas_per_sm"  1..4      DFS workers per SM, or CTAs of six warp workers;
+ *                                dfs_threads x dfs_ctas_per_sm
  *                                must not exceed 1024 (FIM_E_INVAL otherwise)
  *   "split_depth"      0..8      longest prefix a worker may hand to the queue
  *   "root_reverse"     0, 1      hand out the root classes (frequent pairs) in
  *                                reverse order: pairs of the most frequent items
- *                                first (default 0)
+ *                                first (default 0; a mine whose search starts from
+ *                                triples takes them as it finds them)
  *   "learned_order"    0, 1      FIM_LEARNED also hands out the roots longest-
  *                                predicted-subtree first (default 0)
  *   "root_sort"        0, 1      without the network's order, hand out the roots
  *                                as the pair pass lists them (0) or most
  *                                candidates first (1, default).  Either way a root whose
  *                                class has no candidate is dropped before the
- *                                prefix extension starts
+ *                                prefix extension starts.  Applies to pair roots:
+ *                                CTA workers, batches, split mines and mines whose
+ *                                triples are not counted first
  *   "batch_segments"   0..16     fim_mine_batched pipelines this many groups of
  *                                databases (about equal transactions): a group's
  *                                pair pass runs while the next group is built;
@@ -205,14 +215,16 @@ int fim_get_stats(const fim_ctx *ctx, fim_stats *out);
  *                                most 4,096 words: one warp per prefix-extension
  *                                worker instead of one CTA (default 1)
  *   "dfs_warp_ctas"    2, 3      CTAs of eight such warp workers per SM (default 2)
- *   "record_chunk"     1..1024   result slots a prefix-extension worker reserves
- *                                at a time (default 1: exactly a class's sets);
+ *   "record_chunk"     1..1024   result slots a CTA worker of the prefix extension
+ *                                reserves at a time (default 1: exactly a class's
+ *                                sets; a single mine's warp workers reserve ahead
+ *                                by what they have emitted, 64 sets at most);
  *                                the ones a worker leaves unused are sorted out
  *                                by the compaction
  *   "learned_kmin"     1..2^20   FIM_LEARNED consults the network only for classes
  *                                with at least this many candidates (default 8;
  *                                smaller ones are counted dense)
- *   "sparse_div"       -1..64    a class bitmap b_Y is kept as its non-zero words
+ *   "sparse_div"       -1..64    CTA workers: a class bitmap b_Y is kept as its non-zero words
  *                                when S(Y) x sparse_div <= nw (0 = always dense;
  *                                -1 = automatic, the default: 4 when the frequent
  *                                item columns exceed half of L2, else dense)
@@ -401,7 +413,7 @@ int fim_mine_shard(fim_ctx *ctx, uint64_t minsup, uint32_t flags, int shard, int
  * call does not check.
  * Errors: FIM_E_INVAL (a NULL array, malformed offsets, a set longer than 255
  * items, an item >= n_items, n_trans or n_items out of range), FIM_E_NOMEM,
- * FIM_E_CUDA. */
+ * FIM_E_CUDA, FIM_E_TIMEOUT (a bounded wait of the output's sort ran out). */
 int fim_merge_results(fim_ctx *ctx, int64_t n_trans, int32_t n_items, int n_parts,
                       const uint64_t *n_sets, const uint64_t *n_items_total,
                       const uint64_t *const *offsets, const uint32_t *const *items,
@@ -426,13 +438,18 @@ int fim_merge_results(fim_ctx *ctx, int64_t n_trans, int32_t n_items, int n_part
  * rounded once to double, so results are reproducible bit for bit.  Sets
  * longer than max_len yield no rules (a set of size L has 2^L - 2 of them).
  * The rules stay in device memory of the ctx until the next fim_rules or
- * fim_mine; *n_rules gets their number.  Scratch: 8 bytes per held set and
- * 12 bytes per 32 candidate rules (sum of 2^|Z| - 2), plus 12 bytes per
- * candidate when there are at most 2^27 of them.
+ * fim_mine; *n_rules gets their number.  A ratio with a zero support (merged
+ * sets may have one) is the double division's 0, infinity or NaN.  Scratch: 64
+ * to 128 bytes per held set (43 to 85 from 10^8 sets on; 32 to 64 where that
+ * does not fit), 4 bytes per 32 candidate rules (sum of 2^|Z| - 2) and 8 per
+ * 1,024, plus 8 bytes per candidate when there are at most 2^27 of them; up to
+ * 2^22 candidates the rules' own arrays (28 bytes each) are reserved for all
+ * candidates, where that fits.
  * Errors: FIM_E_STATE (no fim_mine result held, or the held sets are not
  * downward closed), FIM_E_INVAL (min_conf_ppm > 10^6, max_len outside
  * {0} u [2, FIM_RULES_MAX_LEN], n_rules NULL), FIM_E_NOMEM (also when the
- * candidate rules' scratch does not fit), FIM_E_CUDA. */
+ * candidate rules' scratch does not fit), FIM_E_CUDA, FIM_E_TIMEOUT (a bounded
+ * wait of the held itemsets' sort ran out). */
 #define FIM_RULES_MAX_LEN 20
 int fim_rules(fim_ctx *ctx, uint32_t min_conf_ppm, int max_len, uint64_t *n_rules);
 

@@ -14,7 +14,9 @@
 // pass that took a 256-thread CTA 25 us on whole columns is one warp's work on
 // a column of one or a few 128-word chunks, with no block barrier at all.
 // Databases whose whole matrix is small skip the projection: the workers then
-// run on the bit columns themselves (`direct`).
+// run on the bit columns themselves (`direct`).  Long columns of dense items, or
+// with few sets, take the CTA workers of k_dfs.cu instead (projection_pays in
+// fim_api.cu).
 // The first level, S({a, b, c}), is one flat pass over all items
 // (proj_triple_kernel); its frequent triples are the search's roots.
 //
