@@ -1202,6 +1202,7 @@ int fim_mine_batched(fim_ctx *ctx, int n_db, const fim_db_desc *in, uint32_t fla
             FIM_TRY(upload(ctx->up_units, ctx->up_units_buf, ctx->batch_units, pair_units.data(),
                            sizeof(unsigned long long) * pair_units.size()));
         if (pack) {
+            ctx->up_units.clear();  // the device plan writes its own units there
             DevBuf ord_buf{static_cast<char *>(ctx->batch_plan.p) + plan_ord_off, ctx->batch_plan.bytes};
             FIM_TRY(upload(ctx->up_ord, ctx->up_ord_buf, ord_buf, ctx->pair_ord_cache.data(), sizeof(int) * (size_t)n_db));
         }

@@ -189,3 +189,20 @@ def test_small_databases_packed_two_to_a_tile(ctx, pack):
     for flags, ml in ((fim.FIM_MAXLEN(2), 2), (fim.FIM_MAXLEN(3), 3)):
         fim.fim_mine_batched(ctx, dbs, ms, flags)
         _check(ctx, dbs, ms, ml)
+
+
+def test_packing_switched_between_batches(ctx):
+    # the host's unit list is uploaded again after the device plan has written
+    # its own over it: batches of one shape, packed and not in turn
+    dbs = [datagen.zipf_baskets(9_000, 300, 0.8, 5.0, seed) for seed in range(4)]
+    dbs += [datagen.zipf_baskets(9_000, 60, 0.8, 5.0, seed) for seed in range(4)]
+    want = [oracle.apriori(c.indptr, c.indices, c.m, 90).sha256() for c in dbs]
+    try:
+        for pack, pick in ((0, [0]), (1, [4, 5, 6, 7]), (0, [1]), (1, [2]), (0, [3]), (0, [0, 4]), (1, [0, 4]),
+                           (0, [1, 5])):
+            fim.fim_set_tuning(ctx, "batch_pairs_pack", pack)
+            fim.fim_mine_batched(ctx, fim.BatchDescriptor([dbs[i] for i in pick], [90] * len(pick)))
+            for d, i in enumerate(pick):
+                assert fim.fim_fetch_batched(ctx, d).sha256() == want[i], (pack, pick, d)
+    finally:
+        fim.fim_set_tuning(ctx, "batch_pairs_pack", 1)
